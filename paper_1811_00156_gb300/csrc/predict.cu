@@ -114,11 +114,13 @@ template <typename CT>
 __global__ void __launch_bounds__(kCodeThreads) code_queries_kernel(const float *__restrict__ Xq, int64_t Q, int F,
                                                                    const float *__restrict__ fvals, int64_t fstride,
                                                                    const uint32_t *__restrict__ fcard,
-                                                                   CT *__restrict__ codes, int row_words, int steps)
+                                                                   CT *__restrict__ codes, int row_words, int steps,
+                                                                   uint32_t *zero, int nzero)
 {
     extern __shared__ __align__(16) uint32_t code_rows[];         // kCodeThreads * row_words words
     const int tid = threadIdx.x;
     const int64_t q0 = (int64_t)blockIdx.x * kCodeThreads, q = q0 + tid;
+    if (q < nzero) zero[q] = 0u;                                   // the walk's tickets (fewer than Q)
     uint32_t *row = code_rows + (size_t)tid * (size_t)row_words;   // odd row_words: distinct banks
     for (int w = 0; w < row_words; ++w) row[w] = 0u;
     if (q < Q) {
@@ -180,10 +182,10 @@ __host__ __forceinline__ int code_row_words(int F, int code_bytes)
     return w;
 }
 
-// codes of Q queries (row_words words per query) on the stream
+// codes of Q queries (row_words words per query) on the stream; zero: nzero <= Q words to clear
 template <typename CT>
 cudaError_t launch_code_queries(const aiwcrf_forest *f, const float *dXq, int64_t Q, CT *d_codes, int row_words,
-                                cudaStream_t s)
+                                cudaStream_t s, uint32_t *zero = nullptr, int nzero = 0)
 {
     if (Q == 0) return cudaSuccess;
     const size_t smem = (size_t)kCodeThreads * (size_t)row_words * 4;        // <= 66 KB (F <= 128)
@@ -194,7 +196,7 @@ cudaError_t launch_code_queries(const aiwcrf_forest *f, const float *dXq, int64_
     }
     const int steps = 32 - __builtin_clz(f->max_card | 1u);               // bit width of the largest table
     code_queries_kernel<CT><<<(unsigned)((Q + kCodeThreads - 1) / kCodeThreads), kCodeThreads, smem, s>>>(
-        dXq, Q, f->F, f->d_fvals, f->fstride, f->d_fcard, d_codes, row_words, steps);
+        dXq, Q, f->F, f->d_fvals, f->fstride, f->d_fcard, d_codes, row_words, steps, zero, nzero);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -230,14 +232,97 @@ __device__ __forceinline__ void walk_tree(NodePtr tn, const CT *const (&xr)[QPT]
     }
 }
 
+// Split of the trees over CTAs. CTA (tile, part) walks trees [part * per, ...) for its tile of
+// queries; with more than one part, each CTA writes its queries' partial sums (and sums of
+// squares) to sum / sq at [part][tile position] and the last CTA of a tile to arrive (ticket)
+// adds the parts and writes the results: exact integers, so the order does not matter.
+struct TreeParts {
+    int per;                     // trees of one part
+    int64_t stride;              // queries, rounded up to whole tiles
+    int64_t *sum;                // parts x stride
+    uint64_t *sq;                // 2 words per entry of sum, for the variance
+    uint32_t *ticket;            // one per tile, zero on entry
+};
+
+__device__ __forceinline__ void write_query(int64_t q, int64_t acc, u128_t sq, int64_t total_trees, int64_t *out_sum,
+                                            int64_t *out_pred, uint64_t *out_var)
+{
+    if (out_sum) out_sum[q] = acc;
+    if (out_pred) {
+        const i128_t num = (i128_t)2 * acc + total_trees, den = (i128_t)2 * total_trees;
+        i128_t d = num / den;
+        if (num % den != 0 && num < 0) d -= 1;
+        out_pred[q] = (int64_t)d;
+    }
+    if (out_var) {
+        const u128_t V = (u128_t)total_trees * sq - (u128_t)((i128_t)acc * (i128_t)acc);
+        out_var[2 * q] = (uint64_t)V;
+        out_var[2 * q + 1] = (uint64_t)(V >> 64);
+    }
+}
+
+// The end of both walk kernels: the thread's QPT queries' sums to the outputs, or to the parts
+// and, from the tile's last CTA, to the outputs. Query at tile position i is perm[i] with PERM.
+template <int QPT, bool VAR, bool PERM>
+__device__ __forceinline__ void finish_tile(const TreeParts &tp, int64_t (&acc)[QPT], u128_t (&sq)[QPT], int64_t q0,
+                                            int64_t Q, int64_t total_trees, int64_t *out_sum, int64_t *out_pred,
+                                            uint64_t *out_var, const uint32_t *__restrict__ perm)
+{
+    const int tid = threadIdx.x;
+    if (gridDim.y > 1) {
+        __shared__ uint32_t last;
+        int64_t *mine = tp.sum + (size_t)blockIdx.y * (size_t)tp.stride + (size_t)q0;
+#pragma unroll
+        for (int i = 0; i < QPT; ++i) {
+            const int k = tid + i * kPredThreads;
+            mine[k] = acc[i];
+            if (VAR) {
+                uint64_t *m = tp.sq + 2 * ((size_t)blockIdx.y * (size_t)tp.stride + (size_t)q0 + (size_t)k);
+                m[0] = (uint64_t)sq[i];
+                m[1] = (uint64_t)(sq[i] >> 64);
+            }
+        }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last = atomicAdd(&tp.ticket[blockIdx.x], 1u) == gridDim.y - 1 ? 1u : 0u;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+#pragma unroll
+        for (int i = 0; i < QPT; ++i) {
+            const size_t k = (size_t)q0 + (size_t)(tid + i * kPredThreads);
+            int64_t a = 0;
+            u128_t v = 0;
+            for (unsigned z = 0; z < gridDim.y; ++z) {
+                const size_t at = (size_t)z * (size_t)tp.stride + k;
+                a += __ldcg((const long long *)&tp.sum[at]);
+                if (VAR)
+                    v += (u128_t)__ldcg((const unsigned long long *)&tp.sq[2 * at]) |
+                         ((u128_t)__ldcg((const unsigned long long *)&tp.sq[2 * at + 1]) << 64);
+            }
+            acc[i] = a;
+            sq[i] = v;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < QPT; ++i) {
+        const int64_t qs = q0 + tid + i * kPredThreads;
+        if (qs >= Q) continue;
+        write_query(PERM ? (int64_t)perm[qs] : qs, acc[i], sq[i], total_trees, out_sum, out_pred, VAR ? out_var : nullptr);
+    }
+}
+
 // Coded walk. The CTA's 256 * QPT query codes sit in shared memory as rows of ld_words
 // 32-bit words (an odd count, so neighbouring queries hit different banks).
 template <typename CT, int QPT, bool VAR>
 __global__ void __launch_bounds__(kPredThreads) predict_kernel(
-    const uint64_t *__restrict__ nodes, const int64_t *__restrict__ tree_off, int T, const CT *__restrict__ codes,
+    const uint64_t *__restrict__ nodes, const int64_t *__restrict__ tree_off_all, int T_all, const CT *__restrict__ codes,
     int64_t Q, int ld_words, int64_t total_trees, int tree_cap, int64_t *out_sum, int64_t *out_pred,
-    uint64_t *out_var, uint32_t *err)
+    uint64_t *out_var, uint32_t *err, TreeParts tp)
 {
+    // this part's trees
+    const int t_first = (int)blockIdx.y * tp.per, T = min(tp.per, T_all - t_first);
+    const int64_t *tree_off = tree_off_all + t_first;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     uint64_t *slot0 = reinterpret_cast<uint64_t *>(sm_raw);
@@ -300,23 +385,7 @@ __global__ void __launch_bounds__(kPredThreads) predict_kernel(
         if (tid == 0 && t + 2 < T) issue_tree(nodes, tree_off, t + 2, tree_cap, s ? slot1 : slot0, &bar[s]);
     }
 
-#pragma unroll
-    for (int i = 0; i < QPT; ++i) {
-        const int64_t q = q0 + tid + i * kPredThreads;
-        if (q >= Q) continue;
-        if (out_sum) out_sum[q] = acc[i];
-        if (out_pred) {
-            const i128_t num = (i128_t)2 * acc[i] + total_trees, den = (i128_t)2 * total_trees;
-            i128_t d = num / den;
-            if (num % den != 0 && num < 0) d -= 1;
-            out_pred[q] = (int64_t)d;
-        }
-        if (VAR) {
-            const u128_t V = (u128_t)total_trees * sq[i] - (u128_t)((i128_t)acc[i] * (i128_t)acc[i]);
-            out_var[2 * q] = (uint64_t)V;
-            out_var[2 * q + 1] = (uint64_t)(V >> 64);
-        }
-    }
+    finish_tile<QPT, VAR, false>(tp, acc, sq, q0, Q, total_trees, out_sum, out_pred, out_var, nullptr);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -392,11 +461,14 @@ __device__ __forceinline__ void walk_tree4(NodePtr tn, const uint8_t *const (&xr
 // (L2-resident) and added one tree later, so their latency overlaps the next walk.
 template <int QPT, bool VAR, bool PERM>
 __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
-    const uint32_t *__restrict__ c32, const int64_t *__restrict__ tree_off4, const uint64_t *__restrict__ nodes,
-    const int64_t *__restrict__ tree_off, int T, const uint8_t *__restrict__ codes, int64_t Q, int ld_words,
+    const uint32_t *__restrict__ c32, const int64_t *__restrict__ tree_off4_all, const uint64_t *__restrict__ nodes,
+    const int64_t *__restrict__ tree_off_all, int T_all, const uint8_t *__restrict__ codes, int64_t Q, int ld_words,
     int64_t total_trees, int tree_cap, int64_t *out_sum, int64_t *out_pred, uint64_t *out_var, uint32_t *err,
-    const uint32_t *__restrict__ perm)
+    const uint32_t *__restrict__ perm, TreeParts tp)
 {
+    // this part's trees
+    const int t_first = (int)blockIdx.y * tp.per, T = min(tp.per, T_all - t_first);
+    const int64_t *tree_off4 = tree_off4_all + t_first, *tree_off = tree_off_all + t_first;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     __shared__ __align__(8) uint64_t bar[2];
     uint32_t *slot0 = reinterpret_cast<uint32_t *>(sm_raw);
@@ -485,24 +557,7 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
         if (VAR) sq[i] += (u128_t)((i128_t)pend[i] * (i128_t)pend[i]);
     }
 
-#pragma unroll
-    for (int i = 0; i < QPT; ++i) {
-        const int64_t qs = q0 + tid + i * kPredThreads;
-        if (qs >= Q) continue;
-        const int64_t q = PERM ? (int64_t)perm[qs] : qs;
-        if (out_sum) out_sum[q] = acc[i];
-        if (out_pred) {
-            const i128_t num = (i128_t)2 * acc[i] + total_trees, den = (i128_t)2 * total_trees;
-            i128_t d = num / den;
-            if (num % den != 0 && num < 0) d -= 1;
-            out_pred[q] = (int64_t)d;
-        }
-        if (VAR) {
-            const u128_t V = (u128_t)total_trees * sq[i] - (u128_t)((i128_t)acc[i] * (i128_t)acc[i]);
-            out_var[2 * q] = (uint64_t)V;
-            out_var[2 * q + 1] = (uint64_t)(V >> 64);
-        }
-    }
+    finish_tile<QPT, VAR, PERM>(tp, acc, sq, q0, Q, total_trees, out_sum, out_pred, out_var, perm);
 }
 
 // Split features of every tree's first kTopNodes nodes (breadth-first: the top levels).
@@ -723,28 +778,87 @@ WalkSmem walk8_smem(const aiwcrf_forest *f, int row_words)
     return WalkSmem{tree_cap, 2 * tree_cap * 8 + xs_bytes};
 }
 
+// How a call's trees are split over CTAs (TreeParts), for tiles of 256 * kQPT queries and CTAs of
+// smem bytes of shared memory.
+//  - Fewer tiles than the chip holds CTAs: as many parts as fill it once, down to one tree each.
+//  - More: enough parts that the last wave of CTAs, nearly empty for an unlucky tile count, is a
+//    small share of the launch, while a part keeps kPartMinTrees trees to pay for staging its
+//    tile's codes again.
+// Measured per call (GB300; unsplit -> split): 2,220 queries x 128 trees 286 -> 119 us (5 CTAs ->
+// 640), 40,001 x 500 with the variance 927 -> 354 us (79 -> 1,264), 1,000,000 x 500 4.89 ->
+// 4.76 ms (1,954 CTAs in 2.1 waves -> 7,816).
+constexpr int64_t kPartMinTrees = 32;
+constexpr int64_t kPartWaves = 8;
+
+int tree_parts(int64_t tiles, int smem, int64_t T)
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t slots = (int64_t)sms * std::max(1, std::min(2048 / kPredThreads, 233472 / (smem + 1024)));
+    const int64_t fill = std::min<int64_t>((slots + tiles - 1) / tiles, T);
+    const int64_t smooth = std::min<int64_t>((kPartWaves * slots + tiles - 1) / tiles, T / kPartMinTrees);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::max(fill, smooth), 65535));
+}
+
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+// The walk's own scratch, one stream-ordered block: the queries' codes, the parts' partial sums
+// and the tickets of the split above. (Callers that bring code scratch walk unsplit.)
+struct WalkScratch {
+    void *block = nullptr;
+    cudaStream_t s = nullptr;
+    void *codes = nullptr;
+    TreeParts tp = {};
+    int parts = 1, tickets = 0;
+    ~WalkScratch() { if (block) cudaFreeAsync(block, s); }
+
+    cudaError_t init(int64_t Q, size_t code_bytes, int smem, int64_t T, bool var, void *codes_scratch, cudaStream_t st)
+    {
+        s = st;
+        const int64_t tiles = (Q + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
+        tp.per = (int)T;
+        if (codes_scratch) { codes = codes_scratch; return cudaSuccess; }
+        parts = tree_parts(tiles, smem, T);
+        tp.per = (int)((T + parts - 1) / parts);
+        parts = (int)((T + tp.per - 1) / tp.per);
+        tp.stride = tiles * kPredThreads * kQPT;
+        const size_t b_codes = up256(code_bytes);
+        const size_t b_sum = parts > 1 ? 8 * (size_t)parts * (size_t)tp.stride : 0, b_sq = var ? 2 * b_sum : 0;
+        tickets = parts > 1 ? (int)tiles : 0;
+        const cudaError_t e = cudaMallocAsync(&block, b_codes + b_sum + b_sq + 4 * (size_t)tickets, st);
+        if (e != cudaSuccess) { block = nullptr; return e; }
+        unsigned char *p = static_cast<unsigned char *>(block);
+        codes = p;
+        tp.sum = reinterpret_cast<int64_t *>(p + b_codes);
+        tp.sq = reinterpret_cast<uint64_t *>(p + b_codes + b_sum);
+        tp.ticket = reinterpret_cast<uint32_t *>(p + b_codes + b_sum + b_sq);
+        return cudaSuccess;
+    }
+};
+
 template <typename CT, bool VAR>
 int launch_predict(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t *d_sum, int64_t *d_pred,
                    uint64_t *d_var, int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *codes_scratch,
                    int64_t walk_T)
 {
     const int ld_words = code_row_words(f->F, (int)sizeof(CT));
-    CT *d_codes = static_cast<CT *>(codes_scratch);
-    cudaError_t e = cudaSuccess;
-    if (!d_codes && cudaMallocAsync(&d_codes, (size_t)Q * (size_t)ld_words * 4, s) != cudaSuccess)
-        return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
-    struct Free { CT *p; cudaStream_t s; ~Free() { if (p) cudaFreeAsync(p, s); } } fr{codes_scratch ? nullptr : d_codes, s};
-    if ((e = launch_code_queries<CT>(f, dXq, Q, d_codes, ld_words, s)) != cudaSuccess)
-        return cuda_fail(e, "code_queries_kernel launch");
     const WalkSmem ws = walk8_smem(f, ld_words);
     const int tree_cap = ws.tree_cap, smem = ws.bytes;
+    WalkScratch w;
+    cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
+    if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
+    CT *d_codes = static_cast<CT *>(w.codes);
+    if ((e = launch_code_queries<CT>(f, dXq, Q, d_codes, ld_words, s, w.tp.ticket, w.tickets)) != cudaSuccess)
+        return cuda_fail(e, "code_queries_kernel launch");
     auto kern = predict_kernel<CT, kQPT, VAR>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(predict_kernel)");
     const int64_t grid = (Q + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
     prof_begin(s, kProfWalk);
-    kern<<<(unsigned)grid, kPredThreads, smem, s>>>(f->d_cnodes, f->d_tree_off, (int)walk_T, d_codes, Q, ld_words,
-                                                    total_trees, tree_cap, d_sum, d_pred, d_var, d_err);
+    kern<<<dim3((unsigned)grid, (unsigned)w.parts), kPredThreads, smem, s>>>(
+        f->d_cnodes, f->d_tree_off, (int)walk_T, d_codes, Q, ld_words, total_trees, tree_cap, d_sum, d_pred, d_var,
+        d_err, w.tp);
     prof_end(s, kProfWalk);
     count_launches(1);
     e = cudaGetLastError();
@@ -761,13 +875,6 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const int ld_words = code_row_words(f->F, 1);
-    uint8_t *d_codes = static_cast<uint8_t *>(codes_scratch);
-    cudaError_t e = cudaSuccess;
-    if (!d_codes && cudaMallocAsync(&d_codes, (size_t)Q * (size_t)ld_words * 4, s) != cudaSuccess)
-        return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
-    struct Free { uint8_t *p; cudaStream_t s; ~Free() { if (p) cudaFreeAsync(p, s); } } fr{codes_scratch ? nullptr : d_codes, s};
-    if ((e = launch_code_queries<uint8_t>(f, dXq, Q, d_codes, ld_words, s)) != cudaSuccess)
-        return cuda_fail(e, "code_queries_kernel launch");
     // query code rows, then 256 bytes that a leaf's code read (feature field 255) may touch
     const int xs_bytes = kPredThreads * kQPT * ld_words * 4 + 256;
     // two tree slots of 4-byte nodes, sized to the largest tree up to 48 KB each
@@ -776,6 +883,12 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     tree_cap &= ~3;
     if (tree_cap < 4) tree_cap = 4;
     const int smem = 2 * tree_cap * 4 + xs_bytes;
+    WalkScratch w;
+    cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
+    if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
+    uint8_t *d_codes = static_cast<uint8_t *>(w.codes);
+    if ((e = launch_code_queries<uint8_t>(f, dXq, Q, d_codes, ld_words, s, w.tp.ticket, w.tickets)) != cudaSuccess)
+        return cuda_fail(e, "code_queries_kernel launch");
     // large batches walk in the order of their leading codes (own scratch only)
     const bool sorted = !codes_scratch && Q >= kSortMinQueries && Q < ((int64_t)1 << 32) && f->key_feats[0] >= 0;
     uint32_t *perm = nullptr;
@@ -799,9 +912,9 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(predict4_kernel)");
     const int64_t grid = (Q + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
     prof_begin(s, kProfWalk);
-    kern<<<(unsigned)grid, kPredThreads, smem, s>>>(f->d_c32, f->d_tree_off4, f->d_nodes, f->d_tree_off, (int)walk_T,
-                                                    d_codes, Q, ld_words, total_trees, tree_cap, d_sum, d_pred, d_var,
-                                                    d_err, perm);
+    kern<<<dim3((unsigned)grid, (unsigned)w.parts), kPredThreads, smem, s>>>(
+        f->d_c32, f->d_tree_off4, f->d_nodes, f->d_tree_off, (int)walk_T, d_codes, Q, ld_words, total_trees, tree_cap,
+        d_sum, d_pred, d_var, d_err, perm, w.tp);
     prof_end(s, kProfWalk);
     count_launches(1);
     e = cudaGetLastError();
@@ -1034,7 +1147,8 @@ int select_noalloc_ct(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, i
     const int64_t grid = (Qn + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
     kern<<<(unsigned)grid, kPredThreads, smem, s>>>(f->d_cnodes, f->d_tree_off, (int)f->T,
                                                     reinterpret_cast<const CT *>(d_codes), Qn, ld_words, f->T,
-                                                    tree_cap, nullptr, d_p, nullptr, d_err);
+                                                    tree_cap, nullptr, d_p, nullptr, d_err,
+                                                    TreeParts{(int)f->T, 0, nullptr, nullptr, nullptr});
     argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, d_dev, K, D, d_best, d_pred);
     count_launches(2);
     e = cudaGetLastError();
