@@ -66,6 +66,7 @@ cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s)
         f->max_tree4 = std::max(f->max_tree4, m4);
     }
     f->compact = f->max_card <= 255u && f->max_tree_nodes <= 65536 && f->F <= 128;
+    f->c32_shift = f->max_tree_nodes <= 16384 ? 2 : 0;
     f->num_c32 = f->compact ? off4[(size_t)f->T] : 0;
     const size_t nn = (size_t)std::max<int64_t>(f->num_nodes, 2);
     const size_t b_nodes = up(8 * nn), b_off = up(8 * (size_t)(f->T + 1));

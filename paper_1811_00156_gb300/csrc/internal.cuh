@@ -431,7 +431,8 @@ struct aiwcrf_forest {
     int64_t fstride = 0;
     uint32_t max_card = 0;
     // 4-byte coded nodes for the shared-memory walk, when every code fits a byte and every tree
-    // 65,536 nodes: bit 31 leaf; else bits 24..30 feature, 16..23 code, 0..15 left child.
+    // 65,536 nodes: bit 31 leaf; else bits 24..30 feature, 16..23 code, 0..15 left child, shifted
+    // left by c32_shift (2, a byte offset, when every tree has at most 16,384 nodes; else 0).
     // Trees padded to a multiple of four nodes (16-byte aligned copies); leaf values are read
     // from d_nodes at the same tree-relative index.
     // out-of-bag evaluation: per tree ceil(oob_rows / 32) words, bit r = training row r in-bag
@@ -439,6 +440,7 @@ struct aiwcrf_forest {
     int64_t inbag_words = 0;
     uint32_t *d_inbag = nullptr;
     bool compact = false;
+    int c32_shift = 0;
     uint32_t *d_c32 = nullptr;
     int64_t *d_tree_off4 = nullptr;       // T + 1 offsets into d_c32
     int64_t num_c32 = 0;

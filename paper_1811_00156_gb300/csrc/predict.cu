@@ -93,21 +93,49 @@ __device__ __forceinline__ void issue_tree(const uint64_t *nodes, const int64_t 
     }
 }
 
+// The tile's code rows (words 32-bit words, 16-byte aligned at both ends) into shared memory: whole
+// 16-byte units by one bulk copy that completes on bar, the rest by plain loads.
+__device__ __forceinline__ void stage_rows(uint32_t *dst, const uint32_t *src, int64_t words, uint64_t *bar)
+{
+    const int64_t whole = words & ~(int64_t)3;
+    if (threadIdx.x == 0) {
+        mbar_arrive_expect_tx(bar, (uint32_t)whole * 4u);
+        if (whole) bulk_g2s(dst, src, (uint32_t)whole * 4u, bar);
+    }
+    if (threadIdx.x < words - whole) dst[whole + threadIdx.x] = src[whole + threadIdx.x];
+}
+
+// Every thread of the CTA: wait for stage_rows' copy on bar[2]. On a wait that gives up, flag it,
+// give the first trees' copies (bar[0], bar[1]) a bounded chance to land, and return false.
+__device__ __forceinline__ bool rows_landed(uint64_t *bar, int T, uint32_t *err)
+{
+    bool ok = false;
+    for (uint32_t it = 0; it < kWaitLimit && !ok; ++it) ok = mbar_try_wait(&bar[2], 0);
+    if (!__syncthreads_or(!ok)) return true;
+    if (threadIdx.x == 0) atomicOr(err, kErrTimeout);
+    for (int b = 0; b < min(T, 2); ++b)
+        for (uint32_t it = 0; it < kWaitLimit; ++it)
+            if (mbar_try_wait(&bar[b], 0)) break;
+    return false;
+}
+
 __device__ __forceinline__ int64_t leaf_value(uint64_t nd)
 {
     return ((int64_t)(nd << 1)) >> 1;
 }
 
 // Rank codes of queries: c(x) = #{table values < x}; NaN goes right of every threshold
-// (c = table size). One thread per query codes all F features (a binary search of each value
-// table) into the query's row in shared memory; the CTA then writes its rows, which are
+// (c = table size). A CTA codes kCodeQueries queries into rows in shared memory, one lane per
+// query and kCodeWarps warps side by side over the features, then writes its rows, which are
 // contiguous in global memory, with 16-byte stores, so that every byte of the code matrix is
 // written once, whole sectors at a time. A row is row_words 4-byte words; its padding is zero.
-constexpr int kCodeThreads = 128;
-
-// The binary searches of kCodeGroup features run side by side (their table loads in flight
-// together), each for a fixed steps = bit width of the largest table: the same lower bound as
-// a search that stops early.
+// What bounds it is the searches' chain of dependent table loads (L1 hits: a warp's lanes search
+// one table). A thread searches kCodeGroup features side by side, so 32 features are one chain of
+// `steps` loads per thread; one thread per query walked eight such chains one after the other.
+// 2,220 queries 58 -> 11 us, 111,000 47 -> 23, 1,000,000 196 -> 177 (148 values per column; cold).
+constexpr int kCodeQueries = 32;
+constexpr int kCodeWarps = 8;
+constexpr int kCodeThreads = 32 * kCodeWarps;
 constexpr int kCodeGroup = 4;
 
 template <typename CT>
@@ -115,50 +143,48 @@ __global__ void __launch_bounds__(kCodeThreads) code_queries_kernel(const float 
                                                                    const float *__restrict__ fvals, int64_t fstride,
                                                                    const uint32_t *__restrict__ fcard,
                                                                    CT *__restrict__ codes, int row_words, int steps,
-                                                                   uint32_t *zero, int nzero)
+                                                                   unsigned long long *zero, int64_t nzero)
 {
-    extern __shared__ __align__(16) uint32_t code_rows[];         // kCodeThreads * row_words words
-    const int tid = threadIdx.x;
-    const int64_t q0 = (int64_t)blockIdx.x * kCodeThreads, q = q0 + tid;
-    if (q < nzero) zero[q] = 0u;                                   // the walk's tickets (fewer than Q)
-    uint32_t *row = code_rows + (size_t)tid * (size_t)row_words;   // odd row_words: distinct banks
-    for (int w = 0; w < row_words; ++w) row[w] = 0u;
+    extern __shared__ __align__(16) uint32_t code_rows[];         // kCodeQueries * row_words words
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t q0 = (int64_t)blockIdx.x * kCodeQueries, q = q0 + lane;
+    for (int64_t i = (int64_t)blockIdx.x * kCodeThreads + tid; i < nzero; i += (int64_t)gridDim.x * kCodeThreads)
+        zero[i] = 0ull;                                            // the walk's sums and tickets
+    CT *c = reinterpret_cast<CT *>(code_rows + (size_t)lane * (size_t)row_words);   // odd row_words: distinct banks
+    for (int f = F + warp; f < row_words * 4 / (int)sizeof(CT); f += kCodeWarps) c[f] = (CT)0;
     if (q < Q) {
-        CT *c = reinterpret_cast<CT *>(row);
-        for (int f0 = 0; f0 < F; f0 += kCodeGroup) {
+        for (int f0 = warp; f0 < F; f0 += kCodeWarps * kCodeGroup) {
             float x[kCodeGroup];
-            uint32_t lo[kCodeGroup], len[kCodeGroup];
+            uint32_t n[kCodeGroup], pos[kCodeGroup];
+            const float *tab[kCodeGroup];
 #pragma unroll
             for (int u = 0; u < kCodeGroup; ++u) {
-                const int f = f0 + u;
+                const int f = f0 + u * kCodeWarps;
                 // features are read once: streaming loads (evict first in L1 and L2) leave the
                 // codes written here resident in L2 for the key and walk kernels that read them
                 x[u] = f < F ? __ldcs(&Xq[(size_t)f * (size_t)Q + q]) : 0.0f;
-                const uint32_t n = f < F ? __ldg(&fcard[f]) : 0u;
-                lo[u] = x[u] != x[u] ? n : 0u;                      // NaN: past every value
-                len[u] = x[u] != x[u] ? 0u : n;
+                n[u] = f < F ? __ldg(&fcard[f]) : 0u;
+                tab[u] = fvals + (size_t)(f < F ? f : 0) * (size_t)fstride;
+                pos[u] = 0u;
             }
-            for (int it = 0; it < steps; ++it) {
+            // lower bound by halving powers of two: pos + bit values are below x if the last of
+            // them is (tables are sorted; a position past the table, or a NaN, never is)
+            for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
 #pragma unroll
                 for (int u = 0; u < kCodeGroup; ++u) {
-                    if (len[u]) {
-                        const uint32_t half = len[u] >> 1;
-                        if (__ldg(&fvals[(size_t)(f0 + u) * (size_t)fstride + lo[u] + half]) < x[u]) {
-                            lo[u] += half + 1u;
-                            len[u] -= half + 1u;
-                        } else {
-                            len[u] = half;
-                        }
-                    }
+                    const uint32_t at = pos[u] + bit;
+                    if (at <= n[u] && __ldg(&tab[u][at - 1]) < x[u]) pos[u] = at;
                 }
             }
 #pragma unroll
-            for (int u = 0; u < kCodeGroup; ++u)
-                if (f0 + u < F) c[f0 + u] = (CT)lo[u];
+            for (int u = 0; u < kCodeGroup; ++u) {
+                const int f = f0 + u * kCodeWarps;
+                if (f < F) c[f] = (CT)(x[u] != x[u] ? n[u] : pos[u]);
+            }
         }
     }
     __syncthreads();
-    const int64_t n = min((int64_t)kCodeThreads, Q - q0);
+    const int64_t n = min((int64_t)kCodeQueries, Q - q0);
     const int words = (int)n * row_words;
     uint32_t *dst = reinterpret_cast<uint32_t *>(codes) + (size_t)q0 * (size_t)row_words;
     const int vec = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0 ? words >> 2 : 0;
@@ -182,20 +208,15 @@ __host__ __forceinline__ int code_row_words(int F, int code_bytes)
     return w;
 }
 
-// codes of Q queries (row_words words per query) on the stream; zero: nzero <= Q words to clear
+// codes of Q queries (row_words words per query) on the stream; zero: nzero 8-byte words to clear
 template <typename CT>
 cudaError_t launch_code_queries(const aiwcrf_forest *f, const float *dXq, int64_t Q, CT *d_codes, int row_words,
-                                cudaStream_t s, uint32_t *zero = nullptr, int nzero = 0)
+                                cudaStream_t s, unsigned long long *zero = nullptr, int64_t nzero = 0)
 {
     if (Q == 0) return cudaSuccess;
-    const size_t smem = (size_t)kCodeThreads * (size_t)row_words * 4;        // <= 66 KB (F <= 128)
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(code_queries_kernel<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const size_t smem = (size_t)kCodeQueries * (size_t)row_words * 4;        // <= 16.5 KB (F <= 128)
     const int steps = 32 - __builtin_clz(f->max_card | 1u);               // bit width of the largest table
-    code_queries_kernel<CT><<<(unsigned)((Q + kCodeThreads - 1) / kCodeThreads), kCodeThreads, smem, s>>>(
+    code_queries_kernel<CT><<<(unsigned)((Q + kCodeQueries - 1) / kCodeQueries), kCodeThreads, smem, s>>>(
         dXq, Q, f->F, f->d_fvals, f->fstride, f->d_fcard, d_codes, row_words, steps, zero, nzero);
     count_launches(1);
     return cudaGetLastError();
@@ -233,15 +254,17 @@ __device__ __forceinline__ void walk_tree(NodePtr tn, const CT *const (&xr)[QPT]
 }
 
 // Split of the trees over CTAs. CTA (tile, part) walks trees [part * per, ...) for its tile of
-// queries; with more than one part, each CTA writes its queries' partial sums (and sums of
-// squares) to sum / sq at [part][tile position] and the last CTA of a tile to arrive (ticket)
-// adds the parts and writes the results: exact integers, so the order does not matter.
+// queries; with more than one part, each CTA adds its queries' partial sums (and sums of squares)
+// into sum / sq, and the last CTA of a tile to arrive (ticket) writes the results: exact integers,
+// so the order does not matter. sum, sq and ticket are zero on entry (the coding kernel clears
+// them). A square sum is kept as its low 32 bits' sum and the rest's, which 64 bits hold.
+// Adding costs the last CTA one read per query; summing the parts' separate sums there instead
+// took 35 us of a 2,220-query call with 128 parts.
 struct TreeParts {
     int per;                     // trees of one part
-    int64_t stride;              // queries, rounded up to whole tiles
-    int64_t *sum;                // parts x stride
-    uint64_t *sq;                // 2 words per entry of sum, for the variance
-    uint32_t *ticket;            // one per tile, zero on entry
+    unsigned long long *sum;     // one per query position (whole tiles)
+    unsigned long long *sq;      // two per query position, for the variance
+    uint32_t *ticket;            // one per tile
 };
 
 __device__ __forceinline__ void write_query(int64_t q, int64_t acc, u128_t sq, int64_t total_trees, int64_t *out_sum,
@@ -271,15 +294,13 @@ __device__ __forceinline__ void finish_tile(const TreeParts &tp, int64_t (&acc)[
     const int tid = threadIdx.x;
     if (gridDim.y > 1) {
         __shared__ uint32_t last;
-        int64_t *mine = tp.sum + (size_t)blockIdx.y * (size_t)tp.stride + (size_t)q0;
 #pragma unroll
         for (int i = 0; i < QPT; ++i) {
-            const int k = tid + i * kPredThreads;
-            mine[k] = acc[i];
+            const size_t k = (size_t)q0 + (size_t)(tid + i * kPredThreads);
+            atomicAdd(&tp.sum[k], (unsigned long long)acc[i]);
             if (VAR) {
-                uint64_t *m = tp.sq + 2 * ((size_t)blockIdx.y * (size_t)tp.stride + (size_t)q0 + (size_t)k);
-                m[0] = (uint64_t)sq[i];
-                m[1] = (uint64_t)(sq[i] >> 64);
+                atomicAdd(&tp.sq[2 * k], (unsigned long long)(uint32_t)sq[i]);
+                atomicAdd(&tp.sq[2 * k + 1], (unsigned long long)(sq[i] >> 32));
             }
         }
         __threadfence();
@@ -291,17 +312,8 @@ __device__ __forceinline__ void finish_tile(const TreeParts &tp, int64_t (&acc)[
 #pragma unroll
         for (int i = 0; i < QPT; ++i) {
             const size_t k = (size_t)q0 + (size_t)(tid + i * kPredThreads);
-            int64_t a = 0;
-            u128_t v = 0;
-            for (unsigned z = 0; z < gridDim.y; ++z) {
-                const size_t at = (size_t)z * (size_t)tp.stride + k;
-                a += __ldcg((const long long *)&tp.sum[at]);
-                if (VAR)
-                    v += (u128_t)__ldcg((const unsigned long long *)&tp.sq[2 * at]) |
-                         ((u128_t)__ldcg((const unsigned long long *)&tp.sq[2 * at + 1]) << 64);
-            }
-            acc[i] = a;
-            sq[i] = v;
+            acc[i] = (int64_t)__ldcg(&tp.sum[k]);
+            if (VAR) sq[i] = (u128_t)__ldcg(&tp.sq[2 * k]) + ((u128_t)__ldcg(&tp.sq[2 * k + 1]) << 32);
         }
     }
 #pragma unroll
@@ -324,7 +336,7 @@ __global__ void __launch_bounds__(kPredThreads) predict_kernel(
     const int t_first = (int)blockIdx.y * tp.per, T = min(tp.per, T_all - t_first);
     const int64_t *tree_off = tree_off_all + t_first;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bar[3];
     uint64_t *slot0 = reinterpret_cast<uint64_t *>(sm_raw);
     uint64_t *slot1 = slot0 + tree_cap;
     uint32_t *xw = reinterpret_cast<uint32_t *>(slot1 + tree_cap);
@@ -333,23 +345,16 @@ __global__ void __launch_bounds__(kPredThreads) predict_kernel(
     const int64_t q0 = (int64_t)blockIdx.x * QT;
 
     if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        for (int i = 0; i < 3; ++i) mbar_init(&bar[i], 1);
         fence_mbar_init();
-    }
-    // stage the tile's codes: global rows of ld_words words -> shared rows of ld_words words
-    {
-        const uint32_t *gw = reinterpret_cast<const uint32_t *>(codes);
-        const int64_t nq = min((int64_t)QT, Q - q0);
-        const int64_t words = nq * ld_words;
-        const uint32_t *src = gw + (size_t)q0 * (size_t)ld_words;
-        for (int64_t k = tid; k < words; k += kPredThreads) xw[k] = src[k];
-    }
-    __syncthreads();
-    if (tid == 0) {
         issue_tree(nodes, tree_off, 0, tree_cap, slot0, &bar[0]);
         if (T > 1) issue_tree(nodes, tree_off, 1, tree_cap, slot1, &bar[1]);
     }
+    // the tile's codes: global rows of ld_words words -> shared rows of ld_words words
+    stage_rows(xw, reinterpret_cast<const uint32_t *>(codes) + (size_t)q0 * (size_t)ld_words,
+               min((int64_t)QT, Q - q0) * ld_words, &bar[2]);
+    __syncthreads();
+    if (!rows_landed(bar, T, err)) return;
 
     const CT *xr[QPT];
 #pragma unroll
@@ -392,7 +397,7 @@ __global__ void __launch_bounds__(kPredThreads) predict_kernel(
 // compact 4-byte coded nodes (one CTA per tree)
 // ------------------------------------------------------------------------------------------
 __global__ void compact_nodes_kernel(const uint64_t *__restrict__ cnodes, const int64_t *__restrict__ tree_off,
-                                     const int64_t *__restrict__ tree_off4, uint32_t *__restrict__ c32)
+                                     const int64_t *__restrict__ tree_off4, uint32_t *__restrict__ c32, int shift)
 {
     const int t = blockIdx.x;
     const int64_t a = tree_off[t], m = tree_off[t + 1] - a;
@@ -400,14 +405,14 @@ __global__ void compact_nodes_kernel(const uint64_t *__restrict__ cnodes, const 
     for (int64_t j = threadIdx.x; j < m4; j += blockDim.x) {
         // a leaf (and a pad) is its own child: left = j, threshold 255 (no code exceeds it),
         // feature field 255 with the top bit as the leaf flag
-        uint32_t v = 0xFFFF0000u | (uint32_t)j;
+        uint32_t v = 0xFFFF0000u | (uint32_t)j << shift;
         if (j < m) {
             const uint64_t nd = cnodes[a + j];
             if (!(nd >> 63)) {
                 const uint32_t f = (uint32_t)(nd >> 56) & 0x7Fu;
                 const uint32_t lc = (uint32_t)(nd >> 32) & 0xFFFFFFu;
                 const uint32_t code = (uint32_t)nd & 0xFFFFFFu;
-                v = (f << 24) | (code << 16) | lc;
+                v = (f << 24) | (code << 16) | lc << shift;
             }
         }
         c32[a4 + j] = v;
@@ -433,8 +438,13 @@ __device__ __forceinline__ void issue_tree4(const uint32_t *c32, const int64_t *
 // leaf test, and the warp stops once the last node of every chain was a leaf. (A leaf's feature
 // field is 255: its code read lands in the padding after the query rows and is never above the
 // leaf's threshold 255.)
+// Instruction issue bounds the walk, so a step is as few as the node's layout allows. SCALED nodes
+// (trees of at most 16,384) hold the left child as a byte offset below the threshold byte: with
+// m = threshold * 65536 + left, code > threshold  <=>  code * 65536 > m, and the next offset is m, or
+// m + 4, without its upper half: no separate threshold or index arithmetic. 1,000,000 queries x 500
+// trees: walk 4.27 -> 4.00 ms; shared-memory wavefronts (997 M, 80 % of their peak rate) bound it now.
 constexpr int kWalkSteps = 2;
-template <int QPT, typename NodePtr>
+template <int QPT, bool SCALED, typename NodePtr>
 __device__ __forceinline__ void walk_tree4(NodePtr tn, const uint8_t *const (&xr)[QPT], uint32_t (&j)[QPT], uint32_t nn)
 {
     uint32_t nd[QPT];
@@ -445,9 +455,17 @@ __device__ __forceinline__ void walk_tree4(NodePtr tn, const uint8_t *const (&xr
         for (int u = 0; u < kWalkSteps; ++u) {
 #pragma unroll
             for (int i = 0; i < QPT; ++i) {
-                nd[i] = tn[j[i]];
-                const uint32_t c = (uint32_t)xr[i][nd[i] >> 24];
-                j[i] = AIWCRF_IDX((nd[i] & 0xFFFFu) + (c > ((nd[i] >> 16) & 0xFFu) ? 1u : 0u), nn, kBoundWalk);
+                if (SCALED) {
+                    nd[i] = *reinterpret_cast<NodePtr>(reinterpret_cast<const unsigned char *>(tn) + j[i]);
+                    const uint32_t c = (uint32_t)xr[i][nd[i] >> 24];
+                    uint32_t m = nd[i] & 0xFFFFFFu;
+                    if ((c << 16) > m) m += 4u;
+                    j[i] = AIWCRF_IDX(m & 0xFFFFu, 4u * nn, kBoundWalk);
+                } else {
+                    nd[i] = tn[j[i]];
+                    const uint32_t c = (uint32_t)xr[i][nd[i] >> 24];
+                    j[i] = AIWCRF_IDX((nd[i] & 0xFFFFu) + (c > ((nd[i] >> 16) & 0xFFu) ? 1u : 0u), nn, kBoundWalk);
+                }
             }
         }
         bool done = true;
@@ -455,11 +473,14 @@ __device__ __forceinline__ void walk_tree4(NodePtr tn, const uint8_t *const (&xr
         for (int i = 0; i < QPT; ++i) done = done && (int32_t)nd[i] < 0;
         if (__all_sync(kFull, done)) break;
     }
+#pragma unroll
+    for (int i = 0; i < QPT; ++i)
+        if (SCALED) j[i] >>= 2;
 }
 
 // The byte-code walk over compact trees. Leaf values are loaded from the 8-byte node array
 // (L2-resident) and added one tree later, so their latency overlaps the next walk.
-template <int QPT, bool VAR, bool PERM>
+template <int QPT, bool VAR, bool PERM, bool SCALED>
 __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
     const uint32_t *__restrict__ c32, const int64_t *__restrict__ tree_off4_all, const uint64_t *__restrict__ nodes,
     const int64_t *__restrict__ tree_off_all, int T_all, const uint8_t *__restrict__ codes, int64_t Q, int ld_words,
@@ -470,7 +491,7 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
     const int t_first = (int)blockIdx.y * tp.per, T = min(tp.per, T_all - t_first);
     const int64_t *tree_off4 = tree_off4_all + t_first, *tree_off = tree_off_all + t_first;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bar[3];
     uint32_t *slot0 = reinterpret_cast<uint32_t *>(sm_raw);
     uint32_t *slot1 = slot0 + tree_cap;
     uint32_t *xw = slot1 + tree_cap;
@@ -479,9 +500,10 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
     const int64_t q0 = (int64_t)blockIdx.x * QT;
 
     if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
+        for (int i = 0; i < 3; ++i) mbar_init(&bar[i], 1);
         fence_mbar_init();
+        issue_tree4(c32, tree_off4, 0, tree_cap, slot0, &bar[0]);
+        if (T > 1) issue_tree4(c32, tree_off4, 1, tree_cap, slot1, &bar[1]);
     }
     {
         // the tile's query codes; with PERM, tile position i holds query perm[q0 + i]
@@ -494,15 +516,11 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
                 xw[k] = gw[(size_t)perm[q0 + r] * (size_t)ld_words + (size_t)w];
             }
         } else {
-            const uint32_t *src = gw + (size_t)q0 * (size_t)ld_words;
-            for (int64_t k = tid; k < words; k += kPredThreads) xw[k] = src[k];
+            stage_rows(xw, gw + (size_t)q0 * (size_t)ld_words, words, &bar[2]);
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        issue_tree4(c32, tree_off4, 0, tree_cap, slot0, &bar[0]);
-        if (T > 1) issue_tree4(c32, tree_off4, 1, tree_cap, slot1, &bar[1]);
-    }
+    if (!PERM && !rows_landed(bar, T, err)) return;
 
     const uint8_t *xr[QPT];
 #pragma unroll
@@ -532,10 +550,10 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
         uint32_t j[QPT];
         const uint32_t nn4 = (uint32_t)(b4 - a4);
         if (b4 - a4 <= tree_cap) {
-            if (s) walk_tree4<QPT>(slot1, xr, j, nn4);
-            else walk_tree4<QPT>(slot0, xr, j, nn4);
+            if (s) walk_tree4<QPT, SCALED, const uint32_t *>(slot1, xr, j, nn4);
+            else walk_tree4<QPT, SCALED, const uint32_t *>(slot0, xr, j, nn4);
         } else {
-            walk_tree4<QPT>(c32 + a4, xr, j, nn4);
+            walk_tree4<QPT, SCALED, const uint32_t *>(c32 + a4, xr, j, nn4);
         }
         // add the previous tree's leaves, then start loading this tree's
         const uint64_t *tn = nodes + ta;
@@ -784,9 +802,9 @@ WalkSmem walk8_smem(const aiwcrf_forest *f, int row_words)
 //  - More: enough parts that the last wave of CTAs, nearly empty for an unlucky tile count, is a
 //    small share of the launch, while a part keeps kPartMinTrees trees to pay for staging its
 //    tile's codes again.
-// Measured per call (GB300; unsplit -> split): 2,220 queries x 128 trees 286 -> 119 us (5 CTAs ->
-// 640), 40,001 x 500 with the variance 927 -> 354 us (79 -> 1,264), 1,000,000 x 500 4.89 ->
-// 4.76 ms (1,954 CTAs in 2.1 waves -> 7,816).
+// Measured, the walk alone (GB300; unsplit -> split): 2,220 queries x 128 trees 243 -> 13 us (5 CTAs
+// -> 640), 40,001 x 500 with the variance 933 -> 264 us (79 -> 1,264), 1,000,000 x 500 4.34 ->
+// 4.22 ms (1,954 CTAs in 2.1 waves -> 7,816).
 constexpr int64_t kPartMinTrees = 32;
 constexpr int64_t kPartWaves = 8;
 
@@ -803,14 +821,16 @@ int tree_parts(int64_t tiles, int smem, int64_t T)
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// The walk's own scratch, one stream-ordered block: the queries' codes, the parts' partial sums
-// and the tickets of the split above. (Callers that bring code scratch walk unsplit.)
+// The walk's own scratch, one stream-ordered block: the queries' codes, and the sums and tickets
+// of the split above. (Callers that bring code scratch walk unsplit.)
 struct WalkScratch {
     void *block = nullptr;
     cudaStream_t s = nullptr;
     void *codes = nullptr;
     TreeParts tp = {};
-    int parts = 1, tickets = 0;
+    int parts = 1;
+    unsigned long long *zero = nullptr;     // what the coding kernel clears: zero_words words
+    int64_t zero_words = 0;
     ~WalkScratch() { if (block) cudaFreeAsync(block, s); }
 
     cudaError_t init(int64_t Q, size_t code_bytes, int smem, int64_t T, bool var, void *codes_scratch, cudaStream_t st)
@@ -822,17 +842,16 @@ struct WalkScratch {
         parts = tree_parts(tiles, smem, T);
         tp.per = (int)((T + parts - 1) / parts);
         parts = (int)((T + tp.per - 1) / tp.per);
-        tp.stride = tiles * kPredThreads * kQPT;
         const size_t b_codes = up256(code_bytes);
-        const size_t b_sum = parts > 1 ? 8 * (size_t)parts * (size_t)tp.stride : 0, b_sq = var ? 2 * b_sum : 0;
-        tickets = parts > 1 ? (int)tiles : 0;
-        const cudaError_t e = cudaMallocAsync(&block, b_codes + b_sum + b_sq + 4 * (size_t)tickets, st);
+        const int64_t n = parts > 1 ? tiles * kPredThreads * kQPT : 0;
+        zero_words = parts > 1 ? n * (var ? 3 : 1) + (tiles + 1) / 2 : 0;
+        const cudaError_t e = cudaMallocAsync(&block, b_codes + 8 * (size_t)zero_words, st);
         if (e != cudaSuccess) { block = nullptr; return e; }
-        unsigned char *p = static_cast<unsigned char *>(block);
-        codes = p;
-        tp.sum = reinterpret_cast<int64_t *>(p + b_codes);
-        tp.sq = reinterpret_cast<uint64_t *>(p + b_codes + b_sum);
-        tp.ticket = reinterpret_cast<uint32_t *>(p + b_codes + b_sum + b_sq);
+        codes = block;
+        zero = reinterpret_cast<unsigned long long *>(static_cast<unsigned char *>(block) + b_codes);
+        tp.sum = zero;
+        tp.sq = zero + n;
+        tp.ticket = reinterpret_cast<uint32_t *>(zero + n * (var ? 3 : 1));
         return cudaSuccess;
     }
 };
@@ -849,7 +868,7 @@ int launch_predict(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t 
     cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
     CT *d_codes = static_cast<CT *>(w.codes);
-    if ((e = launch_code_queries<CT>(f, dXq, Q, d_codes, ld_words, s, w.tp.ticket, w.tickets)) != cudaSuccess)
+    if ((e = launch_code_queries<CT>(f, dXq, Q, d_codes, ld_words, s, w.zero, w.zero_words)) != cudaSuccess)
         return cuda_fail(e, "code_queries_kernel launch");
     auto kern = predict_kernel<CT, kQPT, VAR>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -887,7 +906,7 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
     uint8_t *d_codes = static_cast<uint8_t *>(w.codes);
-    if ((e = launch_code_queries<uint8_t>(f, dXq, Q, d_codes, ld_words, s, w.tp.ticket, w.tickets)) != cudaSuccess)
+    if ((e = launch_code_queries<uint8_t>(f, dXq, Q, d_codes, ld_words, s, w.zero, w.zero_words)) != cudaSuccess)
         return cuda_fail(e, "code_queries_kernel launch");
     // large batches walk in the order of their leading codes (own scratch only)
     const bool sorted = !codes_scratch && Q >= kSortMinQueries && Q < ((int64_t)1 << 32) && f->key_feats[0] >= 0;
@@ -907,7 +926,8 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
         if (rc != AIWCRF_OK) return rc;
         perm = vA;
     }
-    auto kern = sorted ? predict4_kernel<kQPT, VAR, true> : predict4_kernel<kQPT, VAR, false>;
+    auto kern = f->c32_shift ? (sorted ? predict4_kernel<kQPT, VAR, true, true> : predict4_kernel<kQPT, VAR, false, true>)
+                             : (sorted ? predict4_kernel<kQPT, VAR, true, false> : predict4_kernel<kQPT, VAR, false, false>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(predict4_kernel)");
     const int64_t grid = (Q + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
@@ -1039,7 +1059,8 @@ int oob_launch(const aiwcrf_forest *f, const float *dX, int64_t N, int64_t *d_su
 int forest_build_compact(aiwcrf_forest *f, cudaStream_t s)
 {
     if (!f->compact) return AIWCRF_OK;
-    compact_nodes_kernel<<<(unsigned)f->T, 256, 0, s>>>(f->d_cnodes, f->d_tree_off, f->d_tree_off4, f->d_c32);
+    compact_nodes_kernel<<<(unsigned)f->T, 256, 0, s>>>(f->d_cnodes, f->d_tree_off, f->d_tree_off4, f->d_c32,
+                                                          f->c32_shift);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "compact_nodes_kernel launch");
@@ -1148,7 +1169,7 @@ int select_noalloc_ct(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, i
     kern<<<(unsigned)grid, kPredThreads, smem, s>>>(f->d_cnodes, f->d_tree_off, (int)f->T,
                                                     reinterpret_cast<const CT *>(d_codes), Qn, ld_words, f->T,
                                                     tree_cap, nullptr, d_p, nullptr, d_err,
-                                                    TreeParts{(int)f->T, 0, nullptr, nullptr, nullptr});
+                                                    TreeParts{(int)f->T, nullptr, nullptr, nullptr});
     argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, d_dev, K, D, d_best, d_pred);
     count_launches(2);
     e = cudaGetLastError();

@@ -85,13 +85,42 @@ __device__ __forceinline__ uint32_t serve_code(const uint32_t *kcode, uint32_t f
     return f == fd ? dc : kcode[f];
 }
 
+// What a selection walks: 8-byte nodes, compact nodes with the left child as an index, or (trees of
+// at most 16,384 nodes) as a byte offset (see compact_nodes_kernel).
+enum WalkNodes { kWalkWide = 0, kWalkCompact = 1, kWalkScaled = 2 };
+
+__host__ __forceinline__ int walk_nodes_of(const aiwcrf_forest *f)
+{
+    return !f->compact ? kWalkWide : f->c32_shift ? kWalkScaled : kWalkCompact;
+}
+
+// One step of a compact walk from node nd, whose feature's code is c: j is the node's index, or its
+// byte offset when scaled.
+template <int NODES>
+__device__ __forceinline__ uint32_t serve_step(uint32_t nd, uint32_t c, uint32_t nn)
+{
+    if (NODES == kWalkScaled) {
+        uint32_t m = nd & 0xFFFFFFu;
+        if ((c << 16) > m) m += 4u;
+        return AIWCRF_IDX(m & 0xFFFFu, 4u * nn, kBoundWalk);
+    }
+    return AIWCRF_IDX((nd & 0xFFFFu) + (c > ((nd >> 16) & 0xFFu) ? 1u : 0u), nn, kBoundWalk);
+}
+
+template <int NODES>
+__device__ __forceinline__ uint32_t serve_node(const uint32_t *tree, uint32_t j)
+{
+    if (NODES == kWalkScaled) return __ldg(reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(tree) + j));
+    return __ldg(tree + j);
+}
+
 // Two independent walks (trees t0, t1; -1 = none).
-template <bool COMPACT>
+template <int NODES>
 __device__ __forceinline__ int64_t serve_walk2(const ServeForest &sf, int t0, int t1, const uint32_t *kcode,
                                                uint32_t fd, uint32_t dc)
 {
     int64_t v = 0;
-    if (COMPACT) {
+    if (NODES != kWalkWide) {
         const uint32_t *n0 = sf.c32 + (t0 >= 0 ? sf.tree_off4[t0] : 0);
         const uint32_t *n1 = sf.c32 + (t1 >= 0 ? sf.tree_off4[t1] : 0);
 #ifdef AIWCRF_DEBUG_BOUNDS
@@ -101,17 +130,21 @@ __device__ __forceinline__ int64_t serve_walk2(const ServeForest &sf, int t0, in
         uint32_t j0 = 0, j1 = 0;
         bool l0 = t0 < 0, l1 = t1 < 0;
         while (!(l0 && l1)) {
-            const uint32_t a = __ldg(n0 + j0), b = __ldg(n1 + j1);
+            const uint32_t a = serve_node<NODES>(n0, j0), b = serve_node<NODES>(n1, j1);
             const bool la = l0 || (int32_t)a < 0, lb = l1 || (int32_t)b < 0;
             const uint32_t ca = serve_code(kcode, la ? 0u : (a >> 24), fd, dc);
             const uint32_t cb = serve_code(kcode, lb ? 0u : (b >> 24), fd, dc);
-            j0 = la ? j0 : AIWCRF_IDX((a & 0xFFFFu) + (ca > ((a >> 16) & 0xFFu) ? 1u : 0u), m0, kBoundWalk);
-            j1 = lb ? j1 : AIWCRF_IDX((b & 0xFFFFu) + (cb > ((b >> 16) & 0xFFu) ? 1u : 0u), m1, kBoundWalk);
+#ifndef AIWCRF_DEBUG_BOUNDS
+            const uint32_t m0 = 0u, m1 = 0u;               // only a debug build looks at the bounds
+#endif
+            j0 = la ? j0 : serve_step<NODES>(a, ca, m0);
+            j1 = lb ? j1 : serve_step<NODES>(b, cb, m1);
             l0 = la;
             l1 = lb;
         }
-        if (t0 >= 0) v += serve_leaf(__ldg(sf.nodes + sf.tree_off[t0] + j0));
-        if (t1 >= 0) v += serve_leaf(__ldg(sf.nodes + sf.tree_off[t1] + j1));
+        constexpr int kUnit = NODES == kWalkScaled ? 2 : 0;
+        if (t0 >= 0) v += serve_leaf(__ldg(sf.nodes + sf.tree_off[t0] + (j0 >> kUnit)));
+        if (t1 >= 0) v += serve_leaf(__ldg(sf.nodes + sf.tree_off[t1] + (j1 >> kUnit)));
     } else {
         const uint64_t *n0 = sf.cnodes + (t0 >= 0 ? sf.tree_off[t0] : 0);
         const uint64_t *n1 = sf.cnodes + (t1 >= 0 ? sf.tree_off[t1] : 0);
@@ -158,7 +191,7 @@ __device__ __forceinline__ uint32_t rank_code(const float *V, uint32_t card, flo
 // pred: Kb x D row-major predictions; best: Kb device ids. Kernels k < n_gated went through the
 // gate first: only those whose gate flag has kGateForest are answered here, and their
 // predictions are also written to fpred as float log10 seconds.
-template <bool COMPACT>
+template <int NODES>
 __global__ void __launch_bounds__(kServeThreads) serve_select_kernel(ServeForest sf, const float *__restrict__ kq,
                                                                      int Kb, const int32_t *__restrict__ dev, int D,
                                                                      int size_override, unsigned long long *sums,
@@ -187,7 +220,7 @@ __global__ void __launch_bounds__(kServeThreads) serve_select_kernel(ServeForest
     for (int jb = 0; jb < D; jb += kDevSlots) {
         const int j = jb + jl;
         int64_t v = 0;
-        if (j < D) v = serve_walk2<COMPACT>(sf, t0 < sf.T ? t0 : -1, t1 < sf.T ? t1 : -1, kcode, fd, dcode[j]);
+        if (j < D) v = serve_walk2<NODES>(sf, t0 < sf.T ? t0 : -1, t1 < sf.T ? t1 : -1, kcode, fd, dcode[j]);
         v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);             // the warp's two tree slots
         if (lane < kDevSlots) red[warp][lane] = v;
         __syncthreads();
@@ -279,12 +312,12 @@ int serve_launch(const aiwcrf_forest *f, const float *d_kq, int Kb, const int32_
     sf.F = f->F;
     const dim3 grid((unsigned)Kb, (unsigned)((f->T + kTreesPerBlock - 1) / kTreesPerBlock));
     prof_begin(s, kProfServe);
-    if (f->compact)
-        serve_select_kernel<true><<<grid, kServeThreads, 0, s>>>(sf, d_kq, Kb, d_dev, D, size_override, d_sum, d_cnt,
-                                                                 d_pred, d_best, d_only, n_gated, d_fpred);
-    else
-        serve_select_kernel<false><<<grid, kServeThreads, 0, s>>>(sf, d_kq, Kb, d_dev, D, size_override, d_sum, d_cnt,
-                                                                  d_pred, d_best, d_only, n_gated, d_fpred);
+    const int nodes = walk_nodes_of(f);
+    auto kern = nodes == kWalkScaled    ? serve_select_kernel<kWalkScaled>
+                : nodes == kWalkCompact ? serve_select_kernel<kWalkCompact>
+                                        : serve_select_kernel<kWalkWide>;
+    kern<<<grid, kServeThreads, 0, s>>>(sf, d_kq, Kb, d_dev, D, size_override, d_sum, d_cnt, d_pred, d_best, d_only,
+                                        n_gated, d_fpred);
     prof_end(s, kProfServe);
     count_launches(1);
     const cudaError_t e = cudaGetLastError();
@@ -1058,11 +1091,12 @@ int aiwcrf_server_create(const aiwcrf_server_params *params, const aiwcrf_fit_pa
     }
     s->arena.init(p.arena_bytes);
     s->st.arena_bytes = p.arena_bytes;
-    // load both walk variants now: a refit can switch between them, and a kernel's first
+    // load every walk variant now: a refit can switch between them, and a kernel's first
     // launch would otherwise load its code in the middle of serving
     cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, serve_select_kernel<true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, serve_select_kernel<false>);
+    e = cudaFuncGetAttributes(&fa, serve_select_kernel<kWalkScaled>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, serve_select_kernel<kWalkCompact>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, serve_select_kernel<kWalkWide>);
     if (e != cudaSuccess) {
         cuda_fail(e, "loading the selection kernels");
         return bail(AIWCRF_E_CUDA);
