@@ -381,11 +381,12 @@ struct GrowStats {        // device counters of one fit (field order is used by 
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
-// Stable LSD radix sort (four 8-bit passes) of S segments of n (key, value) u32 pairs, segment s
-// at offset s * stride. The result ends in (keys_a, vals_a); (keys_b, vals_b) is scratch.
-// hist needs S * 256 * ceil(n / 4096) + 1 words.
+// Stable LSD radix sort (8-bit passes) of S segments of n (key, value) u32 pairs by the keys' low
+// `bits` bits, segment s at offset s * stride. The result ends in (keys_a, vals_a), or with an odd
+// number of passes in (keys_b, vals_b): *in_b says which. The other pair is scratch.
+// hist needs radix_sort_hist_words(n, S) words.
 int radix_sort_segments(uint32_t *keys_a, uint32_t *vals_a, uint32_t *keys_b, uint32_t *vals_b, int64_t n,
-                        int S, int64_t stride, uint32_t *hist, cudaStream_t s);
+                        int S, int64_t stride, uint32_t *hist, cudaStream_t s, int bits = 32, bool *in_b = nullptr);
 size_t radix_sort_hist_words(int64_t n, int S);
 
 enum ProfClass {
@@ -448,6 +449,7 @@ struct aiwcrf_forest {
     // features whose codes order large query batches before a compact walk (most used in the
     // trees' top levels first; -1: none), so that a warp's queries take similar paths
     int32_t key_feats[4] = {-1, -1, -1, -1};
+    int32_t key_bits[4] = {0, 0, 0, 0};   // bits of each one's codes (0..its table size)
     std::vector<int64_t> tree_off;        // host copy
     aiwcrf_fit_stats stats = {};
 };

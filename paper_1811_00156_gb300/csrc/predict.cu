@@ -592,18 +592,19 @@ __global__ void top_features_kernel(const uint64_t *__restrict__ cnodes, const i
     }
 }
 
-// 32-bit sort key of a coded query: the one-byte codes of four features, most significant first
-__global__ void query_key_kernel(const uint8_t *__restrict__ codes, int ld_bytes, int64_t Q, int4 kf,
+// sort key of a coded query: the codes of up to four features, most significant first, each in
+// the bits its codes need (at most 32 in all)
+__global__ void query_key_kernel(const uint8_t *__restrict__ codes, int ld_bytes, int64_t Q, int4 kf, int4 kb,
                                  uint32_t *__restrict__ keys, uint32_t *__restrict__ idx)
 {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= Q) return;
     const uint8_t *c = codes + (size_t)q * (size_t)ld_bytes;
     uint32_t k = 0;
-    k |= kf.x >= 0 ? (uint32_t)c[kf.x] << 24 : 0u;
-    k |= kf.y >= 0 ? (uint32_t)c[kf.y] << 16 : 0u;
-    k |= kf.z >= 0 ? (uint32_t)c[kf.z] << 8 : 0u;
-    k |= kf.w >= 0 ? (uint32_t)c[kf.w] : 0u;
+    if (kf.x >= 0) k = (uint32_t)c[kf.x];
+    if (kf.y >= 0) k = (k << kb.y) | (uint32_t)c[kf.y];
+    if (kf.z >= 0) k = (k << kb.z) | (uint32_t)c[kf.z];
+    if (kf.w >= 0) k = (k << kb.w) | (uint32_t)c[kf.w];
     keys[q] = k;
     idx[q] = (uint32_t)q;
 }
@@ -920,11 +921,13 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
         fs.p = buf;
         uint32_t *kA = buf, *vA = buf + nq, *kB = buf + 2 * nq, *vB = buf + 3 * nq, *hist = buf + 4 * nq;
         const int4 kf = make_int4(f->key_feats[0], f->key_feats[1], f->key_feats[2], f->key_feats[3]);
-        query_key_kernel<<<(unsigned)((Q + 255) / 256), 256, 0, s>>>(d_codes, ld_words * 4, Q, kf, kA, vA);
+        const int4 kb = make_int4(f->key_bits[0], f->key_bits[1], f->key_bits[2], f->key_bits[3]);
+        query_key_kernel<<<(unsigned)((Q + 255) / 256), 256, 0, s>>>(d_codes, ld_words * 4, Q, kf, kb, kA, vA);
         count_launches(1);
-        int rc = radix_sort_segments(kA, vA, kB, vB, Q, 1, Q, hist, s);
+        bool in_b = false;
+        int rc = radix_sort_segments(kA, vA, kB, vB, Q, 1, Q, hist, s, kb.x + kb.y + kb.z + kb.w, &in_b);
         if (rc != AIWCRF_OK) return rc;
-        perm = vA;
+        perm = in_b ? vB : vA;
     }
     auto kern = f->c32_shift ? (sorted ? predict4_kernel<kQPT, VAR, true, true> : predict4_kernel<kQPT, VAR, false, true>)
                              : (sorted ? predict4_kernel<kQPT, VAR, true, false> : predict4_kernel<kQPT, VAR, false, false>);
@@ -1073,16 +1076,19 @@ int forest_build_compact(aiwcrf_forest *f, cudaStream_t s)
         count_launches(1);
         e = cudaGetLastError();
     }
-    std::vector<uint32_t> h((size_t)f->F, 0u);
+    std::vector<uint32_t> h((size_t)f->F, 0u), card((size_t)f->F, 0u);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), d_cnt, 4 * (size_t)f->F, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(card.data(), f->d_fcard, 4 * (size_t)f->F, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFreeAsync(d_cnt, s);
     if (e != cudaSuccess) return cuda_fail(e, "top split features");
     std::vector<int> order((size_t)f->F);
     for (int i = 0; i < f->F; ++i) order[(size_t)i] = i;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h[(size_t)x] > h[(size_t)y]; });
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k) {
         f->key_feats[k] = (k < f->F && h[(size_t)order[(size_t)k]] > 0) ? order[(size_t)k] : -1;
+        f->key_bits[k] = f->key_feats[k] < 0 ? 0 : 32 - __builtin_clz(card[(size_t)f->key_feats[k]] | 1u);
+    }
     return AIWCRF_OK;
 }
 
