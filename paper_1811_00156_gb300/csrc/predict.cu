@@ -641,11 +641,118 @@ __global__ void oob_kernel(const uint64_t *__restrict__ cnodes, const int64_t *_
     out_count[row] = cnt;
 }
 
+// The same for compact trees: CTA (tile of 256 * QPT rows, part of tp_per trees). As in
+// predict4_kernel the rows' codes sit in shared memory and the trees pass through two slots, here by
+// asynchronous copies of every thread (whose wait cannot run out, so that the call needs no error
+// flag). Every row is walked: the rows of one cell are alike and follow one path, and leaving a
+// tree's in-bag rows out would only idle their lanes; the in-bag words, one for a warp's 32 rows,
+// are read one tree ahead. With several parts the sums and counts, zero on entry, are added to.
+// What bounds it is instruction issue, as the walk of predict; the walk from global memory it
+// replaces waited for a load per node: 111,000 rows x 500 trees 1,072 -> 420 us.
+__device__ __forceinline__ void copy_tree4_async(const uint32_t *src, int64_t nodes, uint32_t *slot)
+{
+    for (int64_t i = threadIdx.x; i < nodes / 4; i += kPredThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + 4 * i)), "l"(src + 4 * i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int QPT, bool SCALED>
+__global__ void __launch_bounds__(kPredThreads) oob4_kernel(
+    const uint32_t *__restrict__ c32, const int64_t *__restrict__ tree_off4, const uint64_t *__restrict__ nodes,
+    const int64_t *__restrict__ tree_off, int T_all, int per, const uint32_t *__restrict__ codes, int64_t N, int ld_words,
+    int tree_cap, const uint32_t *__restrict__ inbag, int64_t inbag_words, int64_t *out_sum, int32_t *out_count)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    uint32_t *slot0 = reinterpret_cast<uint32_t *>(sm_raw);
+    uint32_t *slot1 = slot0 + tree_cap;
+    uint32_t *xw = slot1 + tree_cap;
+    const int tid = threadIdx.x;
+    const int64_t q0 = (int64_t)blockIdx.x * kPredThreads * QPT;
+    const int t_first = (int)blockIdx.y * per, t_end = min(T_all, t_first + per);
+    auto fetch = [&](int t) {                    // tree t's nodes into its slot, if they fit one
+        const int64_t a = tree_off4[t], nn = tree_off4[t + 1] - a;
+        copy_tree4_async(c32 + a, nn <= tree_cap ? nn : 0, (t - t_first) & 1 ? slot1 : slot0);
+    };
+    fetch(t_first);
+    {
+        const int64_t words = min((int64_t)kPredThreads * QPT, N - q0) * ld_words;
+        const uint32_t *src = codes + (size_t)q0 * (size_t)ld_words;
+        for (int64_t k = tid; k < words; k += kPredThreads) xw[k] = src[k];
+    }
+    const uint8_t *xr[QPT];
+    const uint32_t *bits[QPT];
+    uint32_t bag[QPT], count[QPT];
+    int64_t acc[QPT], pend[QPT];
+#pragma unroll
+    for (int i = 0; i < QPT; ++i) {
+        const int64_t row = q0 + tid + i * kPredThreads;
+        xr[i] = reinterpret_cast<const uint8_t *>(xw + (size_t)(tid + i * kPredThreads) * (size_t)ld_words);
+        // a row past the end is in every bag
+        bits[i] = row < N ? inbag + (size_t)t_first * (size_t)inbag_words + (size_t)(row >> 5) : nullptr;
+        bag[i] = bits[i] ? __ldg(bits[i]) : ~0u;
+        count[i] = 0u;
+        acc[i] = pend[i] = 0;
+    }
+    for (int t = t_first; t < t_end; ++t) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();                         // tree t has landed, and nobody walks tree t - 1 any more
+        if (t + 1 < t_end) fetch(t + 1);
+        uint32_t next[QPT];
+#pragma unroll
+        for (int i = 0; i < QPT; ++i) {
+            if (bits[i] && t + 1 < t_end) bits[i] += inbag_words;
+            next[i] = bits[i] ? __ldg(bits[i]) : ~0u;
+        }
+        const int64_t a = tree_off4[t];
+        const uint32_t nn = (uint32_t)(tree_off4[t + 1] - a);
+        const bool fits = nn <= (uint32_t)tree_cap;
+        uint32_t j[QPT];
+        if (!fits) walk_tree4<QPT, SCALED, const uint32_t *>(c32 + a, xr, j, nn);
+        else if ((t - t_first) & 1) walk_tree4<QPT, SCALED, const uint32_t *>(slot1, xr, j, nn);
+        else walk_tree4<QPT, SCALED, const uint32_t *>(slot0, xr, j, nn);
+        const uint64_t *tn = nodes + tree_off[t];
+#pragma unroll
+        for (int i = 0; i < QPT; ++i) {
+            const bool out = !((bag[i] >> (tid & 31)) & 1u);
+            acc[i] += pend[i];
+            count[i] += out ? 1u : 0u;
+            pend[i] = out ? leaf_value(__ldg(&tn[j[i]])) : 0;
+            bag[i] = next[i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < QPT; ++i) {
+        const int64_t row = q0 + tid + i * kPredThreads;
+        if (row >= N) continue;
+        acc[i] += pend[i];
+        if (gridDim.y > 1) {
+            atomicAdd(reinterpret_cast<unsigned long long *>(&out_sum[row]), (unsigned long long)acc[i]);
+            atomicAdd(&out_count[row], (int)count[i]);
+        } else {
+            out_sum[row] = acc[i];
+            out_count[row] = (int32_t)count[i];
+        }
+    }
+}
+
 // Out-of-bag error (Sec. III-B): per row with c > 0 out-of-bag trees its out-of-bag prediction
 // p = floor((2 s + c) / (2 c)) and the squared error (p - y)^2, exact in 128 bits; each CTA
 // writes the sum of its rows' squared errors and their number, oob_error_finish_kernel adds the
 // CTA sums in CTA order and divides once.
 constexpr int kOobErrThreads = 256;
+
+// the warp's sum of 128-bit values and counts, in every lane
+__device__ __forceinline__ void warp_add_part(unsigned long long &lo, unsigned long long &hi, unsigned long long &rows)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long olo = __shfl_xor_sync(kFull, lo, o), ohi = __shfl_xor_sync(kFull, hi, o);
+        const unsigned long long nlo = lo + olo;
+        hi += ohi + (nlo < lo ? 1ull : 0ull);
+        lo = nlo;
+        rows += __shfl_xor_sync(kFull, rows, o);
+    }
+}
 
 __global__ void __launch_bounds__(kOobErrThreads) oob_error_kernel(const int64_t *__restrict__ sum,
                                                                    const int32_t *__restrict__ cnt,
@@ -673,14 +780,7 @@ __global__ void __launch_bounds__(kOobErrThreads) oob_error_kernel(const int64_t
         }
         if (pred) pred[row] = p;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long olo = __shfl_xor_sync(kFull, lo, o), ohi = __shfl_xor_sync(kFull, hi, o);
-        const unsigned long long nlo = lo + olo;
-        hi += ohi + (nlo < lo ? 1ull : 0ull);
-        lo = nlo;
-        rows += __shfl_xor_sync(kFull, rows, o);
-    }
+    warp_add_part(lo, hi, rows);
     if (lane == 0) { red[warp].lo = lo; red[warp].hi = hi; red[warp].rows = rows; }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -695,15 +795,28 @@ __global__ void __launch_bounds__(kOobErrThreads) oob_error_kernel(const int64_t
     }
 }
 
-__global__ void oob_error_finish_kernel(const OobPart *part, int nparts, OobResult *res)
+// One CTA adds the CTA sums (exact, so in any order) and divides once. One thread adding them in
+// turn waited for a load per CTA: 434 of them took 50 us.
+__global__ void __launch_bounds__(kOobErrThreads) oob_error_finish_kernel(const OobPart *part, int nparts, OobResult *res)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ OobPart red[kOobErrThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long lo = 0ull, hi = 0ull, rows = 0ull;
-    for (int i = 0; i < nparts; ++i) {
+    for (int i = threadIdx.x; i < nparts; i += kOobErrThreads) {
         const unsigned long long nlo = lo + part[i].lo;
         hi += part[i].hi + (nlo < lo ? 1ull : 0ull);
         lo = nlo;
         rows += part[i].rows;
+    }
+    warp_add_part(lo, hi, rows);
+    if (lane == 0) { red[warp].lo = lo; red[warp].hi = hi; red[warp].rows = rows; }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kOobErrThreads / 32; ++w) {
+        const unsigned long long nlo = lo + red[w].lo;
+        hi += red[w].hi + (nlo < lo ? 1ull : 0ull);
+        lo = nlo;
+        rows += red[w].rows;
     }
     res->sq_lo = lo;
     res->sq_hi = hi;
@@ -718,7 +831,7 @@ int oob_error_launch(const int64_t *d_sum, const int32_t *d_count, const int64_t
 {
     const int nparts = (int)std::max<int64_t>(1, (N + kOobErrThreads - 1) / kOobErrThreads);
     oob_error_kernel<<<(unsigned)nparts, kOobErrThreads, 0, s>>>(d_sum, d_count, d_y, N, d_pred, d_parts, d_err);
-    oob_error_finish_kernel<<<1, 32, 0, s>>>(d_parts, nparts, d_res);
+    oob_error_finish_kernel<<<1, kOobErrThreads, 0, s>>>(d_parts, nparts, d_res);
     count_launches(2);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "oob_error launch");
@@ -795,6 +908,21 @@ WalkSmem walk8_smem(const aiwcrf_forest *f, int row_words)
     tree_cap &= ~1;
     if (tree_cap < 2) tree_cap = 2;
     return WalkSmem{tree_cap, 2 * tree_cap * 8 + xs_bytes};
+}
+
+// The same for the compact walks: query code rows, then 256 bytes that a leaf's code read (feature
+// field 255) may touch, and two slots of 4-byte nodes.
+WalkSmem walk4_smem(const aiwcrf_forest *f, int row_words)
+{
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const int xs_bytes = kPredThreads * kQPT * row_words * 4 + 256;
+    int tree_cap = std::min<int>((optin - xs_bytes - 1024) / 8, 12288);
+    if ((int64_t)tree_cap > f->max_tree4) tree_cap = (int)f->max_tree4;
+    tree_cap &= ~3;
+    if (tree_cap < 4) tree_cap = 4;
+    return WalkSmem{tree_cap, 2 * tree_cap * 4 + xs_bytes};
 }
 
 // How a call's trees are split over CTAs (TreeParts), for tiles of 256 * kQPT queries and CTAs of
@@ -891,18 +1019,9 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
                     uint64_t *d_var, int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *codes_scratch,
                     int64_t walk_T)
 {
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     const int ld_words = code_row_words(f->F, 1);
-    // query code rows, then 256 bytes that a leaf's code read (feature field 255) may touch
-    const int xs_bytes = kPredThreads * kQPT * ld_words * 4 + 256;
-    // two tree slots of 4-byte nodes, sized to the largest tree up to 48 KB each
-    int tree_cap = std::min<int>((optin - xs_bytes - 1024) / 8, 12288);
-    if ((int64_t)tree_cap > f->max_tree4) tree_cap = (int)f->max_tree4;
-    tree_cap &= ~3;
-    if (tree_cap < 4) tree_cap = 4;
-    const int smem = 2 * tree_cap * 4 + xs_bytes;
+    const WalkSmem ws = walk4_smem(f, ld_words);
+    const int tree_cap = ws.tree_cap, smem = ws.bytes;
     WalkScratch w;
     cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
@@ -1039,6 +1158,27 @@ int oob_ct(const aiwcrf_forest *f, const float *dX, int64_t N, int64_t *d_sum, i
     cudaError_t e = cudaMallocAsync(&d_codes, (size_t)N * (size_t)ld_words * 4, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the row codes failed");
     struct Free { CT *p; cudaStream_t s; ~Free() { cudaFreeAsync(p, s); } } fr{d_codes, s};
+    if (sizeof(CT) == 1 && f->compact) {
+        const WalkSmem ws = walk4_smem(f, ld_words);
+        const int64_t tiles = (N + (int64_t)kPredThreads * kQPT - 1) / ((int64_t)kPredThreads * kQPT);
+        const int want = tree_parts(tiles, ws.bytes, f->T);
+        const int per = (int)((f->T + want - 1) / want), parts = (int)((f->T + per - 1) / per);
+        if ((e = launch_code_queries<CT>(f, dX, N, d_codes, ld_words, s,
+                                         parts > 1 ? reinterpret_cast<unsigned long long *>(d_sum) : nullptr,
+                                         parts > 1 ? N : 0)) != cudaSuccess)
+            return cuda_fail(e, "code_queries_kernel launch");
+        if (parts > 1 && (e = cudaMemsetAsync(d_count, 0, sizeof(int32_t) * (size_t)N, s)) != cudaSuccess)
+            return cuda_fail(e, "out-of-bag counts");
+        auto kern = f->c32_shift ? oob4_kernel<kQPT, true> : oob4_kernel<kQPT, false>;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ws.bytes);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(oob4_kernel)");
+        kern<<<dim3((unsigned)tiles, (unsigned)parts), kPredThreads, ws.bytes, s>>>(
+            f->d_c32, f->d_tree_off4, f->d_nodes, f->d_tree_off, (int)f->T, per, reinterpret_cast<uint32_t *>(d_codes), N,
+            ld_words, ws.tree_cap, f->d_inbag, f->inbag_words, d_sum, d_count);
+        count_launches(1);
+        e = cudaGetLastError();
+        return e == cudaSuccess ? AIWCRF_OK : cuda_fail(e, "oob4_kernel launch");
+    }
     if ((e = launch_code_queries<CT>(f, dX, N, d_codes, ld_words, s)) != cudaSuccess)
         return cuda_fail(e, "code_queries_kernel launch");
     oob_kernel<CT><<<(unsigned)((N + 127) / 128), 128, 0, s>>>(f->d_cnodes, f->d_tree_off, (int)f->T, d_codes, ld, N,

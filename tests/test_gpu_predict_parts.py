@@ -66,3 +66,27 @@ def test_a_large_split_batch_equals_its_slices(var):
         if var:
             assert np.array_equal(gv[2 * a:2 * (a + 1000)], sv)
     assert np.array_equal(got[:1000], ref.predict(Xq[:, :1000])[0])
+
+
+# card 40 compact (three rows in a row alike, as repeated runs are), continuous: the 8-byte walk
+@pytest.mark.parametrize("card", [40, None])
+@pytest.mark.parametrize("n,T", [(1, 3), (31, 1), (511, 2), (512, 37), (513, 37), (1537, 5)])
+def test_out_of_bag_sums_equal_the_oracle(card, n, T):
+    wl = synth.small_case(77 + n, (n + 2) // 3, 32, card=card)
+    X = np.ascontiguousarray(np.repeat(wl.X, 3, axis=1)[:, :n])
+    y = np.ascontiguousarray(np.repeat(wl.y, 3)[:n])
+    forest = A.aiwcrf_fit(A.params(T, 10, 2, seed=9), torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda())
+    s = torch.full((n,), -7, dtype=torch.int64, device="cuda")
+    c = torch.full((n,), -7, dtype=torch.int32, device="cuda")
+    A.aiwcrf_oob(forest, torch.from_numpy(X).cuda(), s, c)
+    torch.cuda.synchronize()
+    ref = O.fit(X, y, T, 10, 2, seed=9)
+    rs, rc = ref.oob(X)
+    assert np.array_equal(s.cpu().numpy(), rs) and np.array_equal(c.cpu().numpy(), rc)
+    pred = torch.empty(n, dtype=torch.int64, device="cuda")
+    mse, rows = A.aiwcrf_oob_error(forest, torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda(), pred)
+    rp, _, rrows = ref.oob_error(X, y)
+    # the documented arithmetic: the exact sum of squares converted to double, divided once
+    sq = sum((int(p) - int(v)) ** 2 for p, v, k in zip(rp, y, rc) if k > 0)
+    exp = (float(sq >> 64) * 2.0 ** 64 + float(sq & (2 ** 64 - 1))) / rrows * 2.0 ** -64 if rrows else 0.0
+    assert np.array_equal(pred.cpu().numpy(), rp) and mse == exp and rows == rrows
