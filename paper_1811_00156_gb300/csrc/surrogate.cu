@@ -9,7 +9,7 @@
 // Inference is one persistent fused kernel: both weight matrices stay in shared memory; for
 // every 128 queries the encoded tile is written straight into the MMA operand layout, layer 1
 // accumulates into TMEM columns 0..255 and layer 2 into 256..511, and the epilogues apply bias
-// and GELU (and the final dot product) from tcgen05.ld registers.
+// and GELU (and the final dot product) from tcgen05.ld registers while the MMAs of the next part run.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -42,35 +42,109 @@ __device__ __forceinline__ float gelu(float x)
     return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));
 }
 
-#ifndef AIWCRF_SUR_GELU_AS
-#define AIWCRF_SUR_GELU_AS 1    // inference epilogues: erf by Abramowitz & Stegun 7.1.26
-#endif
-#ifndef AIWCRF_SUR_SMEM_BIAS
-#define AIWCRF_SUR_SMEM_BIAS 1  // inference: b1 and b2 staged in shared memory
-#endif
-
-// erf(x) by the rational-exponential approximation of Abramowitz & Stegun, Handbook of
-// Mathematical Functions, formula 7.1.26 (absolute error at most 1.5e-7 for x >= 0, extended as
-// an odd function): 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) exp(-x^2), t = 1 / (1 + p x).
-// Evaluated with the approximate reciprocal and exponential: the absolute error of the result
-// stays below 1e-6 (the FP32 evaluation adds a few units of 2^-24 to the formula's 1.5e-7).
-__device__ __forceinline__ float erf_as(float x)
+// GELU of the inference epilogues, two values at a time: the packed FP32 instructions halve those
+// of the polynomials.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
 {
-    const float ax = fabsf(x);
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, ax, 1.0f));
-    const float poly =
-        fmaf(fmaf(fmaf(fmaf(1.061405429f, t, -1.453152027f), t, 1.421413741f), t, -0.284496736f), t, 0.254829592f) * t;
-    return copysignf(fmaf(-poly, __expf(-ax * ax), 1.0f), x);
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
 }
 
-// GELU of the inference epilogues
-__device__ __forceinline__ float gelu_infer(float x)
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
 {
-#if AIWCRF_SUR_GELU_AS
-    return 0.5f * x * (1.0f + erf_as(x * 0.70710678118654752f));
-#else
-    return gelu(x);
-#endif
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ float neg_abs_clamped(float x)      // max(-|x|, -6), NaN stays NaN
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(-fabsf(x)), "f"(-6.0f));
+    return r;
+}
+
+__device__ __forceinline__ float exp2_approx(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Layer 1: 0.5 x (1 + erf(x / sqrt 2)) with erf by the rational-exponential approximation of
+// Abramowitz & Stegun, Handbook of Mathematical Functions, formula 7.1.26 (absolute error at most
+// 1.5e-7 for x >= 0, extended as an odd function): 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5)
+// exp(-x^2), t = 1 / (1 + p x), with the approximate reciprocal and exponential: the absolute error
+// stays below 1e-6. Its result is rounded to BF16, where another formula's last bits would move an
+// activation by a whole BF16 unit now and then, so the first layer keeps this one.
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t gelu2_layer1(uint64_t x)
+{
+    auto both = [](float c) { return pack2(c, c); };
+    float x0, x1, a, b;
+    const uint64_t xs = mul2(x, both(0.70710678118654752f));
+    unpack2(xs, x0, x1);
+    const uint64_t ax = pack2(fabsf(x0), fabsf(x1));
+    unpack2(fma2(both(0.3275911f), ax, both(1.0f)), a, b);
+    const uint64_t t = pack2(rcp_approx(a), rcp_approx(b));
+    uint64_t poly = fma2(both(-1.061405429f), t, both(1.453152027f));      // the polynomial's negative
+    poly = fma2(poly, t, both(-1.421413741f));
+    poly = fma2(poly, t, both(0.284496736f));
+    poly = fma2(poly, t, both(-0.254829592f));
+    poly = mul2(poly, t);
+    // exp(-ax^2) = 2^(-ax^2 log2 e)
+    unpack2(mul2(mul2(ax, ax), both(-1.44269504088896341f)), a, b);
+    const uint64_t ex = pack2(exp2_approx(a), exp2_approx(b));
+    unpack2(fma2(poly, ex, both(1.0f)), a, b);
+    const uint64_t erf = pack2(copysignf(a, x0), copysignf(b, x1));
+    return mul2(mul2(both(0.5f), x), add2(both(1.0f), erf));
+}
+
+// Layer 2, whose GELU stays in FP32: x Phi(x) = max(x, 0) - |x| Phi(-|x|), and log2 Phi(-t) is so
+// smooth on [0, 6] that a degree-8 polynomial q (a weighted minimax fit, here in s = -t) gives
+// |2^q - Phi(-t)| <= 7.6e-9; evaluated in FP32 it stays below 4e-8, and the exponential adds at most
+// 2^-22 of a value below 1/2 (formula 7.1.26 leaves 7e-8 on the same scale before rounding). Beyond 6,
+// Phi(-t) < 1e-9 is taken as Phi(-6). One exponential and nine multiply-adds a value. NaN stays NaN.
+__device__ __forceinline__ uint64_t gelu2(uint64_t x)
+{
+    constexpr float kQ[9] = {-1.0f, 1.1511057615280151f, -0.45920491218566895f, 0.052505023777484894f,
+                             0.007075459696352482f, 0.00014585882308892906f, -0.0001825532381189987f,
+                             -3.8622158172074705e-05f, -2.7721882815967547e-06f};
+    float x0, x1;
+    unpack2(x, x0, x1);
+    const uint64_t s = pack2(neg_abs_clamped(x0), neg_abs_clamped(x1));
+    uint64_t q = fma2(pack2(kQ[8], kQ[8]), s, pack2(kQ[7], kQ[7]));
+#pragma unroll
+    for (int i = 6; i >= 0; --i) q = fma2(q, s, pack2(kQ[i], kQ[i]));
+    float q0, q1;
+    unpack2(q, q0, q1);
+    return fma2(s, pack2(exp2_approx(q0), exp2_approx(q1)), pack2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f)));
 }
 
 __device__ __forceinline__ float gelu_grad(float x)
@@ -265,10 +339,96 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
-constexpr int kInferThreads = 512;
-constexpr int kInferColGroups = kInferThreads / 128;          // warps sharing one TMEM lane quarter
-constexpr int kInferCols = 256 / kInferColGroups;              // accumulator columns per warp
-constexpr int kInferSmem = 32768 + 4 * 32768 + 4 * 16384;     // W1, W2 (4 K-chunks), H1 (4 K-chunks)
+// One tile is 128 queries. What bounds the kernel is the epilogues' arithmetic (65,536 GELUs a tile,
+// the FP32 pipe first; the MMAs take about 2,600 clocks), so everything else runs beside it on warps
+// of its own, and the sixteen epilogue warps hardly wait for each other:
+//  - layer 1 accumulates in TMEM columns 0..255 and layer 2 in 256..511;
+//  - epilogue 1 goes through the first layer's columns in four chunks of 64. A warp puts its BF16
+//    activations back over the columns it read, where layer 2 takes them as the A operand straight
+//    from TMEM (through shared memory, the stores and the proxy fence of a chunk took 400 clocks);
+//  - the warps hand a chunk over by arriving on an mbarrier and go on; one warp waits for the
+//    arrivals and issues the chunk's part of layer 2 (one K chunk), which runs under the next chunk.
+//    (An epilogue warp that also issued them fell behind and held up the others.)
+//  - four warps, that one among them, encode the next tile while this one is in its epilogues (in
+//    the epilogue warps that took 2,500 clocks of a tile), 32 rows each, so that its layer 1 runs
+//    under this tile's epilogue 2. The raw features of the tile after that are copied to shared
+//    memory meanwhile, every lane its own.
+// Twenty warps leave 96 registers a thread.
+// Why nothing is overwritten early: a warp reaches chunk c of the next tile only after bar_h of this
+// one, which every warp's arrivals of this tile precede, and the next layer 1 is issued after it.
+// Shared memory holds W1 (32 KB), W2 (128), the input tile (16) and its raw features (32).
+// Measured at 1,000,000 queries (32 features): 980 us with every part of a
+// tile after the other and eight instructions more a GELU, 413 us now = 400 TFLOP/s of the MMAs; a
+// tile's clocks are 5,200 of epilogue 1, 4,300 of epilogue 2 (6,400 together at the FP32 pipe's rate)
+// and about 2,500 of waiting for the slowest warp and the last chunk.
+constexpr int kInferWarps = 16;                                // epilogue warps
+constexpr int kEncodeWarps = 4;                                // the first of them issues the MMAs
+constexpr int kInferThreads = 32 * (kInferWarps + kEncodeWarps);
+constexpr int kInferColGroups = kInferWarps / 4;               // warps sharing one TMEM lane quarter
+constexpr int kInferCols = 256 / kInferColGroups;              // layer-2 columns per warp
+constexpr int kInferSmem = 32768 + 4 * 32768 + 16384 + kIn * 128 * 4;
+
+// The transform of one AIWC column.
+struct EncodeColumn {
+    float mu, sd, rcp_sd;
+    uint32_t lg;
+};
+
+// encode_value of one AIWC column; the quotient by the approximate reciprocal and one exact residual
+// (the division sequence costs several times that). No branch on the logarithm, so that several
+// columns' chains run side by side.
+__device__ __forceinline__ float standardise(float x, const EncodeColumn &c)
+{
+    const float lg = log2f(fmaxf(x, 1.0f));
+    const float a = (c.lg ? lg : x) - c.mu;
+    const float q = a * c.rcp_sd, better = fmaf(fmaf(-q, c.sd, a), c.rcp_sd, q);
+    return fabsf(q) < INFINITY ? better : q;
+}
+
+// the input that a one-hot column's value v sets (first + v for v = 0..n-1), or -1
+__device__ __forceinline__ int hot_input(float v, int first, int n)
+{
+    const int i = (int)v;
+    return (float)i == v && i >= 0 && i < n ? first + i : -1;
+}
+
+// A part of a tile that a warp encodes at once is 32 rows x 8 inputs from k0 on, one row a lane; the
+// 8 inputs are AIWC columns, one-hot inputs or both. copy_part starts the copies of the lane's raw
+// values to raw[k0 + i][row], encode_part computes the inputs from them.
+__device__ __forceinline__ void copy_part(const Encoder &e, const float *__restrict__ X, int64_t Q, int64_t q, int row, int k0,
+                                          float *raw)
+{
+    if (q >= Q) return;
+    const float *src = X + (size_t)k0 * (size_t)Q + q;
+    uint32_t dst = tc::smem_addr(raw + k0 * 128 + row);
+#pragma unroll
+    for (int i = 0; i < 8; ++i, src += Q, dst += 512u)
+        if (k0 + i < e.n_aiwc)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void encode_part(const Encoder &e, const EncodeColumn *col, const float *raw, float dev,
+                                            float size, bool valid, int row, int k0, unsigned char *sX)
+{
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (k0 < e.n_aiwc) {
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = standardise(raw[(k0 + i) * 128 + row], col[k0 + i]);   // past the columns: any value
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = k0 + i < e.n_aiwc && valid ? v[i] : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
+    }
+    if (k0 + 8 > e.n_aiwc) {                    // the device's and the size's 1 where it falls here
+        const uint32_t d = (uint32_t)(hot_input(dev, e.n_aiwc, e.n_dev) - k0);
+        const uint32_t z = (uint32_t)(hot_input(size, e.n_aiwc + e.n_dev, e.n_size) - k0);
+        const uint32_t dv = d & 1u ? 0x3F800000u : 0x3F80u, zv = z & 1u ? 0x3F800000u : 0x3F80u;      // BF16 1
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] |= (d >> 1 == (uint32_t)i ? dv : 0u) | (z >> 1 == (uint32_t)i ? zv : 0u);
+    }
+    *reinterpret_cast<uint4 *>(sX + tc::core_offset((uint32_t)row, (uint32_t)k0)) = make_uint4(w[0], w[1], w[2], w[3]);
+}
 
 __global__ void __launch_bounds__(kInferThreads, 1) surrogate_infer_kernel(
     Encoder e, const float *__restrict__ Xq, int64_t Q, const bf16 *__restrict__ W1b, const bf16 *__restrict__ W2b,
@@ -276,151 +436,207 @@ __global__ void __launch_bounds__(kInferThreads, 1) surrogate_infer_kernel(
     float *__restrict__ out, uint32_t *err)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
-    unsigned char *sW1 = sm;                    // 256 x 64
-    unsigned char *sW2 = sm + 32768;            // 4 chunks of 256 x 64
-    unsigned char *sH = sm + 32768 + 4 * 32768; // 4 chunks of 128 x 64; chunk 0 holds the input tile first
-    __shared__ __align__(8) uint64_t bar;
+    unsigned char *sW1 = sm;                        // 256 x 64
+    unsigned char *sW2 = sm + 32768;                // 4 chunks of 256 x 64
+    unsigned char *sX = sm + 32768 + 4 * 32768;     // 128 x 64: the input tile
+    float *raw = reinterpret_cast<float *>(sX + 16384);     // [input][row]
+    __shared__ __align__(8) uint64_t full_x, full_h[4];     // operands written (one arrival a warp)
+    __shared__ __align__(8) uint64_t bar_x, bar_h;          // MMAs done: layer 1, layer 2
+    __shared__ __align__(16) float b1s[kHid], b2s[kHid], w3s[kHid];
+    __shared__ __align__(16) EncodeColumn col[kIn];
+    __shared__ float part[kInferColGroups][128];            // the output dot's partial sums
     __shared__ uint32_t tmem_base;
-#if AIWCRF_SUR_SMEM_BIAS
-    __shared__ float b1s[kHid], b2s[kHid];
-    // the output dot's partial sums sit in the last activation chunk: free once layer 2's MMAs
-    // are done, and the next tile's encoding writes chunk 0 only
-    float(*part)[128] = reinterpret_cast<float(*)[128]>(sH + 3 * 16384);
-#define AIWCRF_B1(j) b1s[j]
-#define AIWCRF_B2(j) b2s[j]
-#else
-    __shared__ float part[kInferColGroups][128];
-#define AIWCRF_B1(j) __ldg(&b1[j])
-#define AIWCRF_B2(j) __ldg(&b2[j])
-#endif
+    __shared__ volatile int gave_up;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q4 = warp & 3, half = warp >> 2;          // TMEM lane quarter, column group
+    const int64_t ntiles = (Q + 127) / 128;
 
     // weights, once per CTA, in the operand layout
-    for (int p = tid; p < 256 * 8; p += kInferThreads) {
-        const int r = p >> 3, kk = (p & 7) * 8;
-        *reinterpret_cast<uint4 *>(sW1 + tc::core_offset(r, kk)) =
-            __ldg(reinterpret_cast<const uint4 *>(W1b + (size_t)r * kIn + kk));
+    for (int i = tid; i < 256 * 8; i += kInferThreads) {
+        const int n = i >> 3, kk = (i & 7) * 8;
+        *reinterpret_cast<uint4 *>(sW1 + tc::core_offset(n, kk)) =
+            __ldg(reinterpret_cast<const uint4 *>(W1b + (size_t)n * kIn + kk));
     }
-    for (int p = tid; p < 4 * 256 * 8; p += kInferThreads) {
-        const int kc = p / (256 * 8), rr = p % (256 * 8);
-        const int r = rr >> 3, kk = (rr & 7) * 8;
-        *reinterpret_cast<uint4 *>(sW2 + kc * 32768 + tc::core_offset(r, kk)) =
-            __ldg(reinterpret_cast<const uint4 *>(W2b + (size_t)r * kHid + kc * 64 + kk));
+    for (int i = tid; i < 4 * 256 * 8; i += kInferThreads) {
+        const int kc = i / (256 * 8), rr = i % (256 * 8);
+        const int n = rr >> 3, kk = (rr & 7) * 8;
+        *reinterpret_cast<uint4 *>(sW2 + kc * 32768 + tc::core_offset(n, kk)) =
+            __ldg(reinterpret_cast<const uint4 *>(W2b + (size_t)n * kHid + kc * 64 + kk));
     }
-#if AIWCRF_SUR_SMEM_BIAS
-    for (int j = tid; j < kHid; j += kInferThreads) { b1s[j] = __ldg(&b1[j]); b2s[j] = __ldg(&b2[j]); }
-#endif
-    if (warp == 0) {
+    for (int j = tid; j < kHid; j += kInferThreads) { b1s[j] = __ldg(&b1[j]); b2s[j] = __ldg(&b2[j]); w3s[j] = __ldg(&w3[j]); }
+    for (int k = tid; k < e.n_aiwc; k += kInferThreads) col[k] = EncodeColumn{e.mu[k], e.sd[k], rcp_approx(e.sd[k]), e.logf[k]};
+    if (warp == kInferWarps) {
         tc::tmem_alloc(&tmem_base, 512);
         tc::tmem_relinquish();
     }
-    if (tid == 0) tc::mbar_init(&bar, 1);
+    if (tid == 0) {
+        tc::mbar_init(&full_x, kEncodeWarps);
+        for (int c = 0; c < 4; ++c) tc::mbar_init(&full_h[c], kInferWarps);
+        tc::mbar_init(&bar_x, 1);
+        tc::mbar_init(&bar_h, 1);
+        gave_up = 0;
+    }
     tc::fence_before_sync();
+    tc::fence_smem_to_async();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = tmem_base;
-    const uint32_t idesc = tc::make_idesc_bf16(128, 256);
-    const int64_t ntiles = (Q + 127) / 128;
-    uint32_t phase = 0;
-    bool ok = true;
-
-    for (int64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const int64_t q0 = tile * 128;
-        {   // encode the query tile: thread (row, part) encodes inputs [part * kIn / G, ...) of one row
-            const int row = tid & 127, kpart = tid >> 7;
-            const int64_t q = q0 + row;
-            constexpr int kPer = kIn / kInferColGroups;
-            for (int kk = kpart * kPer; kk < (kpart + 1) * kPer; kk += 8) {
-                uint32_t w[4];
-                for (int i = 0; i < 4; ++i) {
-                    const float v0 = q < Q ? encode_value(e, Xq, Q, q, kk + 2 * i) : 0.0f;
-                    const float v1 = q < Q ? encode_value(e, Xq, Q, q, kk + 2 * i + 1) : 0.0f;
-                    w[i] = pack_bf16x2(v0, v1);
-                }
-                *reinterpret_cast<uint4 *>(sH + tc::core_offset(row, kk)) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        tc::fence_smem_to_async();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after_sync();
-            const uint32_t a0 = tc::smem_addr(sH), w0 = tc::smem_addr(sW1);
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-                tc::mma_bf16(tbase, tc::make_desc(a0 + 256u * s, tc::kLbo, tc::kSbo),
-                             tc::make_desc(w0 + 256u * s, tc::kLbo, tc::kSbo), idesc, s > 0 ? 1u : 0u);
-            tc::mma_commit(&bar);
-        }
-        ok = __syncthreads_and(tc::mbar_wait(&bar, phase));
-        phase ^= 1u;
-        if (!ok) break;
+    auto wait = [&](uint64_t *bar, uint32_t parity) {     // once a wait has run out, none waits again
+        if (!gave_up && !tc::mbar_wait(bar, parity)) gave_up = 1;
         tc::fence_after_sync();
-        {   // epilogue 1: bias, GELU, BF16 into the layer-2 operand tile
-            const int r = 32 * q4 + lane;
-            for (int c = 0; c < kInferCols / 32; ++c) {
-                const int col0 = kInferCols * half + 32 * c;
-                float v[32];
-                tc::tmem_ld32(tbase + ((uint32_t)(32 * q4) << 16) + (uint32_t)col0, v);
-                for (int g8 = 0; g8 < 32; g8 += 8) {
-                    uint32_t w[4];
-                    for (int i = 0; i < 4; ++i) {
-                        const int j0 = col0 + g8 + 2 * i;
-                        const float h0 = gelu_infer(v[g8 + 2 * i] + AIWCRF_B1(j0));
-                        const float h1 = gelu_infer(v[g8 + 2 * i + 1] + AIWCRF_B1(j0 + 1));
-                        w[i] = pack_bf16x2(h0, h1);
-                    }
-                    const int k = col0 + g8;
-                    *reinterpret_cast<uint4 *>(sH + (k >> 6) * 16384 + tc::core_offset(r, k & 63)) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-        }
+    };
+    auto arrive = [&](uint64_t *bar) {
         tc::fence_before_sync();
-        tc::fence_smem_to_async();
-        __syncthreads();
-        if (tid == 0) {
-            tc::fence_after_sync();
-            const uint32_t a0 = tc::smem_addr(sH), w0 = tc::smem_addr(sW2);
-            for (int kc = 0; kc < 4; ++kc)
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(bar);
+    };
+
+    if (warp >= kInferWarps) {
+        const int row = 32 * (warp - kInferWarps) + lane;
+        float dev, size;
+        auto fetch = [&](int64_t tile) {                   // the row's raw values of a tile
+            const int64_t q = tile * 128 + row;
+#pragma unroll 1
+            for (int k0 = 0; k0 < e.n_aiwc; k0 += 8) copy_part(e, Xq, Q, q, row, k0, raw);
+            dev = q < Q ? __ldg(&Xq[(size_t)e.n_aiwc * (size_t)Q + q]) : -1.0f;
+            size = q < Q ? __ldg(&Xq[(size_t)(e.n_aiwc + 1) * (size_t)Q + q]) : -1.0f;
+        };
+        auto encode = [&](int64_t tile, int k_from, int k_to) {
+#pragma unroll 1
+            for (int k0 = k_from; k0 < k_to; k0 += 8) encode_part(e, col, raw, dev, size, tile * 128 + row < Q, row, k0, sX);
+        };
+        auto hand_over_tile = [&]() {
+            tc::fence_smem_to_async();
+            arrive(&full_x);
+        };
+        fetch(blockIdx.x);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        encode(blockIdx.x, 0, kIn);
+        hand_over_tile();
+        if ((int64_t)blockIdx.x + gridDim.x < ntiles) fetch((int64_t)blockIdx.x + gridDim.x);
+        const uint32_t idesc = tc::make_idesc_bf16(128, 256);
+        const uint32_t a0 = tc::smem_addr(sX), w1 = tc::smem_addr(sW1), w2 = tc::smem_addr(sW2);
+        auto issue_chunk = [&](int c, uint32_t parity) {
+            wait(&full_h[c], parity);
+            if (lane == 0 && !gave_up) {
 #pragma unroll
                 for (int s = 0; s < 4; ++s)
-                    tc::mma_bf16(tbase + 256u, tc::make_desc(a0 + 16384u * kc + 256u * s, tc::kLbo, tc::kSbo),
-                                 tc::make_desc(w0 + 32768u * kc + 256u * s, tc::kLbo, tc::kSbo), idesc,
-                                 (kc > 0 || s > 0) ? 1u : 0u);
-            tc::mma_commit(&bar);
-        }
-        ok = __syncthreads_and(tc::mbar_wait(&bar, phase));
-        phase ^= 1u;
-        if (!ok) break;
-        tc::fence_after_sync();
-        {   // epilogue 2: bias, GELU, dot with w3
-            const int r = 32 * q4 + lane;
-            float dot = 0.0f;
-            for (int c = 0; c < kInferCols / 32; ++c) {
-                const int col0 = kInferCols * half + 32 * c;
-                float v[32];
-                tc::tmem_ld32(tbase + ((uint32_t)(32 * q4) << 16) + 256u + (uint32_t)col0, v);
-                for (int i = 0; i < 32; ++i) dot += gelu_infer(v[i] + AIWCRF_B2(col0 + i)) * __ldg(&w3[col0 + i]);
+                    tc::mma_bf16_ta(tbase + 256u, tbase + 64u * c + 16u * s,
+                                    tc::make_desc(w2 + 32768u * c + 256u * s, tc::kLbo, tc::kSbo), idesc,
+                                    c > 0 || s > 0 ? 1u : 0u);
+                if (c == 3) tc::mma_commit(&bar_h);
             }
-            part[half][r] = dot;
-        }
-        tc::fence_before_sync();
-        __syncthreads();
-        if (tid < 128 && q0 + tid < Q) {
-            float o = __ldg(&b3[0]);
+            __syncwarp();
+        };
+        uint32_t n = 0;                                    // the CTA's tiles in turn
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++n) {
+            const int64_t next = tile + gridDim.x;
+            const bool more = next < ntiles;
+            if (warp == kInferWarps) {
+                wait(&full_x, n & 1u);
+                if (n) wait(&bar_h, (n - 1u) & 1u);        // the activations have been read
+                if (lane == 0 && !gave_up) {
 #pragma unroll
-            for (int g = 0; g < kInferColGroups; ++g) o += part[g][tid];
-            out[q0 + tid] = o;
+                    for (int s = 0; s < 4; ++s)
+                        tc::mma_bf16(tbase, tc::make_desc(a0 + 256u * s, tc::kLbo, tc::kSbo),
+                                     tc::make_desc(w1 + 256u * s, tc::kLbo, tc::kSbo), idesc, s > 0 ? 1u : 0u);
+                    tc::mma_commit(&bar_x);
+                }
+                __syncwarp();
+            }
+            if (more) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                wait(&bar_x, n & 1u);                      // layer 1 has read the input tile
+            }
+            if (warp != kInferWarps) {
+                if (more) encode(next, 0, kIn);
+            } else {                                       // between the chunks, which come at their own pace
+                if (more) encode(next, 0, 24);
+                issue_chunk(0, n & 1u);
+                if (more) encode(next, 24, kIn);
+                issue_chunk(1, n & 1u);
+                issue_chunk(2, n & 1u);
+                issue_chunk(3, n & 1u);
+            }
+            if (more) {
+                hand_over_tile();
+                if (next + gridDim.x < ntiles) fetch(next + gridDim.x);
+            }
+        }
+        if (gave_up && warp == kInferWarps && lane == 0) {   // MMAs may still be running: a bounded wait
+            tc::mma_commit(&bar_h);                          // for them before their TMEM goes
+            for (uint32_t k = 0; k < 2u; ++k) tc::mbar_wait(&bar_h, k);
+        }
+        __syncwarp();
+    } else {
+        const int q4 = warp & 3, group = warp >> 2;         // TMEM lane quarter, column group
+        const int r = 32 * q4 + lane;
+        const uint32_t mine = tbase + ((uint32_t)(32 * q4) << 16);
+        uint32_t parity = 0;
+        for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, parity ^= 1u) {
+            const int64_t q0 = tile * 128;
+            wait(&bar_x, parity);
+            uint32_t v[16];
+            tc::tmem_start16(mine + 16u * group, v);
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {   // epilogue 1: bias, GELU, BF16 back into TMEM
+                const uint32_t col0 = 64u * c + 16u * group;
+                const float4 *bias = reinterpret_cast<const float4 *>(b1s + col0);
+                uint32_t w[8];
+                float x[16];
+                tc::tmem_wait16(v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
+                if (c < 3) tc::tmem_start16(mine + col0 + 64u, v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 b = bias[i];
+                    float h0, h1;
+                    unpack2(gelu2_layer1(add2(pack2(x[4 * i], x[4 * i + 1]), pack2(b.x, b.y))), h0, h1);
+                    w[2 * i] = pack_bf16x2(h0, h1);
+                    unpack2(gelu2_layer1(add2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2(b.z, b.w))), h0, h1);
+                    w[2 * i + 1] = pack_bf16x2(h0, h1);
+                }
+                tc::tmem_st8(mine + col0, w);
+                arrive(&full_h[c]);
+            }
+            wait(&bar_h, parity);
+            tc::tmem_start16(mine + 256u + (uint32_t)(kInferCols * group), v);
+            uint64_t dot = pack2(0.0f, 0.0f);
+#pragma unroll 1
+            for (int c = 0; c < kInferCols / 16; ++c) {     // epilogue 2: bias, GELU, dot with w3
+                const int col0 = kInferCols * group + 16 * c;
+                const float4 *bias = reinterpret_cast<const float4 *>(b2s + col0);
+                const float4 *wt = reinterpret_cast<const float4 *>(w3s + col0);
+                float x[16];
+                tc::tmem_wait16(v);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
+                if (c + 1 < kInferCols / 16) tc::tmem_start16(mine + 256u + (uint32_t)(col0 + 16), v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 b = bias[i], w = wt[i];
+                    dot = fma2(gelu2(add2(pack2(x[4 * i], x[4 * i + 1]), pack2(b.x, b.y))), pack2(w.x, w.y), dot);
+                    dot = fma2(gelu2(add2(pack2(x[4 * i + 2], x[4 * i + 3]), pack2(b.z, b.w))), pack2(w.z, w.w), dot);
+                }
+            }
+            tc::fence_before_sync();
+            float d0, d1;
+            unpack2(dot, d0, d1);
+            part[group][r] = d0 + d1;
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + q4) : "memory");   // the quarter's four warps
+            if (group == 0 && q0 + r < Q) {
+                float o = __ldg(&b3[0]);
+#pragma unroll
+                for (int g = 0; g < kInferColGroups; ++g) o += part[g][r];
+                out[q0 + r] = o;
+            }
         }
     }
-    if (!ok && tid == 0) atomicOr(err, kErrTimeout);
+    if (gave_up && tid == 0) atomicOr(err, kErrTimeout);
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tbase, 512);
-    }
+    tc::fence_after_sync();
+    if (warp == kInferWarps) tc::tmem_dealloc(tbase, 512);
 }
 
 }  // namespace aiwcrf
