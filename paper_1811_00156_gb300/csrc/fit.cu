@@ -1573,9 +1573,6 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) level_list_kerne
 // tie-breaks and leaf values.
 // ------------------------------------------------------------------------------------------
 // build-time tuning of the tree kernel (the forest does not depend on them)
-#ifndef AIWCRF_TREE_THREADS
-#define AIWCRF_TREE_THREADS 256        // threads per CTA
-#endif
 #ifndef AIWCRF_TREE_UNROLL
 #define AIWCRF_TREE_UNROLL 0           // 1: small-node sort and scan unrolled per segment width
 #endif
@@ -1585,9 +1582,9 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) level_list_kerne
 #ifndef AIWCRF_TREE_DYN
 #define AIWCRF_TREE_DYN 1              // 1: phase-A items handed out by a shared counter
 #endif
-constexpr int kTreeThreads = AIWCRF_TREE_THREADS;
-constexpr int kTreeWarps = kTreeThreads / 32;
-constexpr int kTreeCtasPerSm = 4;      // resident CTAs per SM the tree kernel is compiled for
+// The tree kernel is compiled for 8, 16 and 32 warps a tree, at 4, 2 and 1 CTAs per SM (64 registers
+// a thread each): see tree_warps.
+constexpr int kTreeSmWarps = 32;       // resident warps per SM it is compiled for
 constexpr int kTreeIlp = 8;            // rank loads in flight per lane in a histogram pass
 
 struct TNode {            // an active node of a CTA's tree at the current depth
@@ -1630,11 +1627,11 @@ struct TreeArgs {
     uint32_t *levels;             // the deepest tree's depth count (atomicMax)
 };
 
-size_t tree_smem_bytes(int ecap, int bins, int big_cap)
+size_t tree_smem_bytes(int ecap, int bins, int big_cap, int warps)
 {
     const size_t e = (size_t)ecap;
     return 8 * e + 4 * e + ((2 * e + 15) & ~(size_t)15) + 2 * ((2 * e + 15) & ~(size_t)15) + ((e + 15) & ~(size_t)15) +
-           (size_t)kTreeWarps * (size_t)bins * 12 + 2 * (((size_t)big_cap * 2 + 15) & ~(size_t)15);
+           (size_t)warps * (size_t)bins * 12 + 2 * (((size_t)big_cap * 2 + 15) & ~(size_t)15);
 }
 
 struct TreeSmem {
@@ -1648,7 +1645,7 @@ struct TreeSmem {
     uint32_t *big_mask;      // tried features of the depth's big nodes (aliases flag)
 };
 
-__device__ __forceinline__ TreeSmem tree_smem(unsigned char *base, const TreeArgs &a)
+__device__ __forceinline__ TreeSmem tree_smem(unsigned char *base, const TreeArgs &a, int warps)
 {
     const size_t e = (size_t)a.ecap;
     TreeSmem m;
@@ -1659,7 +1656,7 @@ __device__ __forceinline__ TreeSmem tree_smem(unsigned char *base, const TreeArg
     m.ix[0] = reinterpret_cast<uint16_t *>(p); p += (2 * e + 15) & ~(size_t)15;
     m.ix[1] = reinterpret_cast<uint16_t *>(p); p += (2 * e + 15) & ~(size_t)15;
     m.flag = p; p += (e + 15) & ~(size_t)15;
-    m.bins = reinterpret_cast<uint32_t *>(p); p += (size_t)kTreeWarps * (size_t)a.bins * 12;
+    m.bins = reinterpret_cast<uint32_t *>(p); p += (size_t)warps * (size_t)a.bins * 12;
     m.big[0] = reinterpret_cast<uint16_t *>(p); p += ((size_t)a.big_cap * 2 + 15) & ~(size_t)15;
     m.big[1] = reinterpret_cast<uint16_t *>(p);
     // the big nodes' masks are read in phase A only, the partition flags written in phase B only:
@@ -1987,6 +1984,7 @@ __device__ __forceinline__ void tree_big_split(const TreeArgs &a, const TreeSmem
 // in shared memory across one CTA barrier, and each writes its chunk's entries after the left
 // (or right) entries of the chunks before it: the same stable partition as one warp's.
 // Every warp of the CTA calls this once (it holds the depth's one barrier).
+template <int kTreeWarps>
 __device__ __forceinline__ void tree_big_split_w(const TreeArgs &a, const TreeSmem &sm, const uint16_t *ix, uint16_t *ox,
                                                  const TNode *cn, const uint16_t *big, uint32_t nb, int m,
                                                  const Cand *cands, SplitRes *res, uint32_t *counts, int warp, int lane)
@@ -2063,14 +2061,16 @@ __device__ __forceinline__ void tree_big_split_w(const TreeArgs &a, const TreeSm
     }
 }
 
-__global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm) tree_grow_kernel(TreeArgs a)
+template <int kTreeWarps>
+__global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tree_grow_kernel(TreeArgs a)
 {
+    constexpr int kTreeThreads = 32 * kTreeWarps;
     extern __shared__ __align__(16) unsigned char tree_sm[];
     __shared__ uint32_t warp_tmp[32];
     __shared__ unsigned long long red[6][kTreeWarps];
     __shared__ uint32_t s_nb[2];
     __shared__ uint32_t s_next;                                 // the next phase-A item to hand out
-    const TreeSmem sm = tree_smem(tree_sm, a);
+    const TreeSmem sm = tree_smem(tree_sm, a, kTreeWarps);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     TNode *const nodes0 = a.nodes + (size_t)blockIdx.x * 2 * (size_t)a.ecap;
     TNode *const nodes1 = nodes0 + a.ecap;
@@ -2152,7 +2152,7 @@ __global__ void __launch_bounds__(kTreeThreads, kTreeCtasPerSm) tree_grow_kernel
             // B: big nodes' decisions and partitions (a node per warp, or several warps per
             // node when the depth has fewer big nodes than warps)
             if (nb > 0u && nb < (uint32_t)kTreeWarps) {
-                tree_big_split_w(a, sm, ix, ox, cn, big, nb, m, cands, res, warp_tmp, warp, lane);
+                tree_big_split_w<kTreeWarps>(a, sm, ix, ox, cn, big, nb, m, cands, res, warp_tmp, warp, lane);
             } else {
                 for (uint32_t bi = (uint32_t)warp; bi < nb; bi += kTreeWarps) {
                     const uint32_t i = AIWCRF_IDX(big[bi], a.ecap, kBoundNode);
@@ -2249,6 +2249,22 @@ __global__ void group_records_kernel(const uint8_t *__restrict__ Rr, int F, cons
     const uint8_t r = (int)f < F ? Rr[(size_t)grp_rows[grp_off[g]] * (size_t)F + f] : (uint8_t)0;
     Rg[i] = r;
     if ((int)f < F) RgT[(size_t)f * G + g] = r;
+}
+
+using TreeKernel = void (*)(TreeArgs);
+
+TreeKernel tree_kernel(int warps)
+{
+    return warps == 32 ? tree_grow_kernel<32> : warps == 16 ? tree_grow_kernel<16> : tree_grow_kernel<8>;
+}
+
+// Warps per tree: as many as leave every tree a place on the chip at once, since a tree is a serial
+// chain of depths that more warps shorten, while trees side by side fill an SM as well with 8 warps
+// each. Measured, tree kernel at 8 / 16 / 32 warps: 128 trees of 2,220 rows 1,235 / 828 / 695 us; 500
+// trees of 2,220 groups 2,750 / 3,010 / 3,640 us.
+int tree_warps(int64_t T, int sms)
+{
+    return T <= sms ? 32 : T <= 2 * (int64_t)sms ? 16 : 8;
 }
 
 // copy each tree's nodes from its output slot into the forest (and pad an odd count)
@@ -3000,7 +3016,13 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
     const int tree_bins = (int)std::max<uint32_t>(max_card, 1u);
     const int tree_ecap = (int)std::max<int64_t>(row_cap, 1);
     const int tree_big_cap = tree_ecap / (kSmallNodeRows + 1) + 1;
-    const size_t tree_smem = tree_smem_bytes(tree_ecap, tree_bins, tree_big_cap);
+    int tree_sms = 0;
+    AIWCRF_CUDA(cudaDeviceGetAttribute(&tree_sms, cudaDevAttrMultiProcessorCount, device));
+    // a background fit keeps to small CTAs; so does a fit whose histograms for more warps do not fit
+    int n_tree_warps = p.ctas_per_sm > 0 ? 8 : tree_warps(T, tree_sms);
+    auto tree_bytes = [&](int warps) { return tree_smem_bytes(tree_ecap, tree_bins, tree_big_cap, warps); };
+    while (n_tree_warps > 8 && tree_bytes(n_tree_warps) + 1024 > (size_t)max_smem_optin) n_tree_warps /= 2;
+    const size_t tree_smem = tree_bytes(n_tree_warps);
     const bool tree_fits = rank8 && F <= 32 && n_groups <= 65535u && row_cap <= 65535 &&
                            tree_smem + 1024 <= (size_t)max_smem_optin;
     if (gmode == AIWCRF_GROWER_TREE && !tree_fits)
@@ -3164,12 +3186,13 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
 
     if (use_tree) {
         // one CTA per tree at a time, as many as fit (a background fit: at most ctas_per_sm per SM)
-        AIWCRF_CUDA(cudaFuncSetAttribute(tree_grow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tree_smem));
+        const TreeKernel kern = tree_kernel(n_tree_warps);
+        AIWCRF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tree_smem));
         // shared memory over L1: the occupancy (and one wave of trees) depends on it
-        AIWCRF_CUDA(cudaFuncSetAttribute(tree_grow_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+        AIWCRF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared));
         int occ = 0;
-        AIWCRF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tree_grow_kernel, kTreeThreads, tree_smem));
+        AIWCRF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * n_tree_warps, tree_smem));
         if (occ < 1) return fail(AIWCRF_E_LIMIT, "tree-resident growth: no CTA fits on an SM");
         if (p.ctas_per_sm > 0) occ = std::min<int>(occ, p.ctas_per_sm);
         const int64_t grid = std::min<int64_t>(T, (int64_t)occ * dev_sms);
@@ -3192,7 +3215,7 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
         ta.out_nodes = slot_nodes; ta.out_cnodes = slot_cnodes; ta.node_cap = node_cap; ta.out_count = counts;
         ta.stats = d_stats; ta.levels = levels;
         prof_begin(s, kProfTree);
-        tree_grow_kernel<<<(unsigned)grid, kTreeThreads, tree_smem, s>>>(ta);
+        kern<<<(unsigned)grid, 32 * n_tree_warps, tree_smem, s>>>(ta);
         AIWCRF_LAUNCH_CHECK("tree_grow_kernel");
         prof_end(s, kProfTree);
         // the error flags are read with the tree sizes (one wait instead of two)
