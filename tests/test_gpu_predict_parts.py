@@ -68,13 +68,14 @@ def test_a_large_split_batch_equals_its_slices(var):
     assert np.array_equal(got[:1000], ref.predict(Xq[:, :1000])[0])
 
 
-# card 40 compact (three rows in a row alike, as repeated runs are), continuous: the 8-byte walk
-@pytest.mark.parametrize("card", [40, None])
-@pytest.mark.parametrize("n,T", [(1, 3), (31, 1), (511, 2), (512, 37), (513, 37), (1537, 5)])
-def test_out_of_bag_sums_equal_the_oracle(card, n, T):
-    wl = synth.small_case(77 + n, (n + 2) // 3, 32, card=card)
-    X = np.ascontiguousarray(np.repeat(wl.X, 3, axis=1)[:, :n])
-    y = np.ascontiguousarray(np.repeat(wl.y, 3)[:n])
+# card 40 compact, continuous: the 8-byte walk; runs of alike rows as repeated measurements make them:
+# a tile of 512 rows holds at most 128 different ones (so they alone are walked) from 4 in a row on
+@pytest.mark.parametrize("card,runs", [(40, 1), (40, 3), (40, 4), (40, 50), (None, 3)])
+@pytest.mark.parametrize("n,T", [(1, 3), (31, 1), (511, 2), (512, 37), (513, 37), (1537, 5), (1024, 400)])
+def test_out_of_bag_sums_equal_the_oracle(card, runs, n, T):
+    wl = synth.small_case(77 + n, (n + runs - 1) // runs, 32, card=card)
+    X = np.ascontiguousarray(np.repeat(wl.X, runs, axis=1)[:, :n])
+    y = np.ascontiguousarray(np.repeat(wl.y, runs)[:n])
     forest = A.aiwcrf_fit(A.params(T, 10, 2, seed=9), torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda())
     s = torch.full((n,), -7, dtype=torch.int64, device="cuda")
     c = torch.full((n,), -7, dtype=torch.int32, device="cuda")
