@@ -664,24 +664,21 @@ int aiwcrf_select_device(const aiwcrf_forest *forest, const float *kfeat, int32_
     InArg ak, ad;
     OutArg ob, op;
     if ((rc = stage_in(ak, kfeat, sizeof(float) * (size_t)(forest->F - 2) * (size_t)n_kernels, dev, s, "kfeat"))) return rc;
-    if ((rc = stage_in(ad, device_ids, sizeof(int32_t) * (size_t)n_devices, dev, s, "device_ids"))) return rc;
+    // a host array of a few ids travels with the launches
+    DeviceIds ids;
+    if (n_devices <= kSelectMaxDevices && classify(device_ids, dev) == kPtrHost) {
+        std::memcpy(ids.id, device_ids, sizeof(int32_t) * (size_t)n_devices);
+    } else {
+        if ((rc = stage_in(ad, device_ids, sizeof(int32_t) * (size_t)n_devices, dev, s, "device_ids"))) return rc;
+        ids.dev = (const int32_t *)ad.dev;
+    }
     if ((rc = stage_out(ob, out_best, sizeof(int32_t) * (size_t)n_kernels, dev, s, "out_best"))) return rc;
     if ((rc = stage_out(op, out_pred, sizeof(int64_t) * (size_t)Qn, dev, s, "out_pred"))) return rc;
-    float *d_q = nullptr;
-    int64_t *d_p = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_q, sizeof(float) * (size_t)forest->F * (size_t)Qn, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&d_p, sizeof(int64_t) * (size_t)Qn, s);
-    if (e != cudaSuccess) {
-        if (d_q) cudaFreeAsync(d_q, s);
-        return fail(AIWCRF_E_OOM, "select_device scratch");
-    }
-    rc = select_launch(forest, (const float *)ak.dev, n_kernels, size_class, (const int32_t *)ad.dev, n_devices,
-                       (int32_t *)ob.dev, (int64_t *)op.dev, d_q, d_p, s);
-    cudaFreeAsync(d_q, s);
-    cudaFreeAsync(d_p, s);
-    if (rc) return rc;
+    if ((rc = select_launch(forest, (const float *)ak.dev, n_kernels, size_class, ids, n_devices, (int32_t *)ob.dev,
+                            (int64_t *)op.dev, s)))
+        return rc;
     if ((rc = finish_out(ob)) || (rc = finish_out(op))) return rc;
-    // device_ids is usually a host array: its staged copy must be consumed before returning
+    // a staged copy of device_ids must be consumed before returning
     return sync_if(true, s);
 }
 

@@ -501,11 +501,19 @@ int predict_enqueue(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
 // fused surrogate inference on the stream, timeouts flagged in d_err (no allocation, no sync)
 int surrogate_predict_enqueue(const aiwcrf_surrogate *sg, const float *dXq, int64_t Q, float *d_out, uint32_t *d_err,
                               cudaStream_t s);
+// The device ids of a selection: device memory, or (at most kSelectMaxDevices of them, dev null) the
+// ids themselves, which then travel with the launch.
+constexpr int kSelectMaxDevices = 64;
+struct DeviceIds {
+    const int32_t *dev = nullptr;
+    int32_t id[kSelectMaxDevices] = {};
+    __device__ __forceinline__ int32_t operator[](int j) const { return dev ? dev[j] : id[j]; }
+};
 // Device selection by the tree-parallel kernel (one CTA per kernel and 32 trees): d_kfeat is
 // (F-2) x K, d_sum (K * D) and d_cnt (K) zero on entry and left zero, d_pred K x D; needs
 // D <= 64 and size_class >= 0. Same integer results as predict + argmin.
 int select_small_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class,
-                        const int32_t *d_dev, int32_t D, int32_t *d_best, int64_t *d_pred, unsigned long long *d_sum,
+                        const DeviceIds &ids, int32_t D, int32_t *d_best, int64_t *d_pred, unsigned long long *d_sum,
                         uint32_t *d_cnt, cudaStream_t s);
 // exact ensemble variance numerators of the first n_trees trees (2 u64 words per query)
 int predict_prefix_var_enqueue(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t n_trees,
@@ -563,9 +571,9 @@ int predict_launch(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t 
                    int64_t *d_pred, uint64_t *d_var, int64_t total_trees, cudaStream_t s);
 int round_mean_launch(const int64_t *d_sum, int64_t Q, int64_t total_trees, int64_t *d_out,
                       cudaStream_t s);
-int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class,
-                  const int32_t *d_dev, int32_t D, int32_t *d_best, int64_t *d_pred,
-                  float *d_scratch_q, int64_t *d_scratch_p, cudaStream_t s);
+// device selection; with more than kSelectMaxDevices devices ids.dev is given
+int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class, const DeviceIds &ids,
+                  int32_t D, int32_t *d_best, int64_t *d_pred, cudaStream_t s);
 size_t select_noalloc_bytes(const aiwcrf_forest *f, int32_t K, int32_t D);
 int select_launch_noalloc(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class,
                           const int32_t *h_dev, int32_t D, int32_t *d_best, int64_t *d_pred, unsigned char *scratch,

@@ -74,8 +74,8 @@ __device__ __forceinline__ void fence_mbar_init()
 }
 
 constexpr int kPredThreads = 256;
-// device selections with at most this many queries use the tree-parallel kernel
-constexpr int64_t kTreeParallelMaxQueries = 1 << 18;
+// device selections with at most this many walks use the tree-parallel kernel (select_launch)
+constexpr int64_t kTreeParallelMaxWalks = 1 << 21;
 constexpr uint32_t kWaitLimit = 1u << 24;     // try_wait polls before giving up
 
 // stage tree t into slot (or just complete the phase if it does not fit)
@@ -138,6 +138,40 @@ constexpr int kCodeWarps = 8;
 constexpr int kCodeThreads = 32 * kCodeWarps;
 constexpr int kCodeGroup = 4;
 
+// this lane's codes c[f] of the features f < nf that are its warp's, x(f) their values
+template <typename CT, typename Value>
+__device__ __forceinline__ void code_columns(int nf, const float *__restrict__ fvals, int64_t fstride,
+                                             const uint32_t *__restrict__ fcard, int steps, int warp, CT *c, const Value &value)
+{
+    for (int f0 = warp; f0 < nf; f0 += kCodeWarps * kCodeGroup) {
+        float x[kCodeGroup];
+        uint32_t n[kCodeGroup], pos[kCodeGroup];
+        const float *tab[kCodeGroup];
+#pragma unroll
+        for (int u = 0; u < kCodeGroup; ++u) {
+            const int f = f0 + u * kCodeWarps;
+            x[u] = f < nf ? value(f) : 0.0f;
+            n[u] = f < nf ? __ldg(&fcard[f]) : 0u;
+            tab[u] = fvals + (size_t)(f < nf ? f : 0) * (size_t)fstride;
+            pos[u] = 0u;
+        }
+        // lower bound by halving powers of two: pos + bit values are below x if the last of
+        // them is (tables are sorted; a position past the table, or a NaN, never is)
+        for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
+#pragma unroll
+            for (int u = 0; u < kCodeGroup; ++u) {
+                const uint32_t at = pos[u] + bit;
+                if (at <= n[u] && __ldg(&tab[u][at - 1]) < x[u]) pos[u] = at;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kCodeGroup; ++u) {
+            const int f = f0 + u * kCodeWarps;
+            if (f < nf) c[f] = (CT)(x[u] != x[u] ? n[u] : pos[u]);
+        }
+    }
+}
+
 template <typename CT>
 __global__ void __launch_bounds__(kCodeThreads) code_queries_kernel(const float *__restrict__ Xq, int64_t Q, int F,
                                                                    const float *__restrict__ fvals, int64_t fstride,
@@ -152,37 +186,11 @@ __global__ void __launch_bounds__(kCodeThreads) code_queries_kernel(const float 
         zero[i] = 0ull;                                            // the walk's sums and tickets
     CT *c = reinterpret_cast<CT *>(code_rows + (size_t)lane * (size_t)row_words);   // odd row_words: distinct banks
     for (int f = F + warp; f < row_words * 4 / (int)sizeof(CT); f += kCodeWarps) c[f] = (CT)0;
-    if (q < Q) {
-        for (int f0 = warp; f0 < F; f0 += kCodeWarps * kCodeGroup) {
-            float x[kCodeGroup];
-            uint32_t n[kCodeGroup], pos[kCodeGroup];
-            const float *tab[kCodeGroup];
-#pragma unroll
-            for (int u = 0; u < kCodeGroup; ++u) {
-                const int f = f0 + u * kCodeWarps;
-                // features are read once: streaming loads (evict first in L1 and L2) leave the
-                // codes written here resident in L2 for the key and walk kernels that read them
-                x[u] = f < F ? __ldcs(&Xq[(size_t)f * (size_t)Q + q]) : 0.0f;
-                n[u] = f < F ? __ldg(&fcard[f]) : 0u;
-                tab[u] = fvals + (size_t)(f < F ? f : 0) * (size_t)fstride;
-                pos[u] = 0u;
-            }
-            // lower bound by halving powers of two: pos + bit values are below x if the last of
-            // them is (tables are sorted; a position past the table, or a NaN, never is)
-            for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
-#pragma unroll
-                for (int u = 0; u < kCodeGroup; ++u) {
-                    const uint32_t at = pos[u] + bit;
-                    if (at <= n[u] && __ldg(&tab[u][at - 1]) < x[u]) pos[u] = at;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kCodeGroup; ++u) {
-                const int f = f0 + u * kCodeWarps;
-                if (f < F) c[f] = (CT)(x[u] != x[u] ? n[u] : pos[u]);
-            }
-        }
-    }
+    // features are read once: streaming loads (evict first in L1 and L2) leave the codes written here
+    // resident in L2 for the key and walk kernels that read them
+    if (q < Q)
+        code_columns<CT>(F, fvals, fstride, fcard, steps, warp, c,
+                         [&](int f) { return __ldcs(&Xq[(size_t)f * (size_t)Q + q]); });
     __syncthreads();
     const int64_t n = min((int64_t)kCodeQueries, Q - q0);
     const int words = (int)n * row_words;
@@ -191,6 +199,56 @@ __global__ void __launch_bounds__(kCodeThreads) code_queries_kernel(const float 
     for (int i = tid; i < vec; i += kCodeThreads)
         reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(code_rows)[i];
     for (int i = 4 * vec + tid; i < words; i += kCodeThreads) dst[i] = code_rows[i];
+}
+
+// Rank codes of a device selection's queries (k, j) = kernel k's features, device ids[j], one size
+// class: a CTA codes the features of kCodeQueries kernels as above, the devices and the size once,
+// and writes every kernel's row for every device. (Expanding the queries first read and searched
+// every feature once per device.)
+template <typename CT>
+__device__ __forceinline__ CT code_of(float x, const float *__restrict__ tab, uint32_t n, int steps)
+{
+    uint32_t pos = 0u;
+    for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
+        const uint32_t at = pos + bit;
+        if (at <= n && __ldg(&tab[at - 1]) < x) pos = at;
+    }
+    return (CT)(x != x ? n : pos);
+}
+
+template <typename CT>
+__global__ void __launch_bounds__(kCodeThreads) code_selection_kernel(
+    const float *__restrict__ kfeat, int32_t K, int32_t size_class, DeviceIds ids, int32_t D, int F,
+    const float *__restrict__ fvals, int64_t fstride, const uint32_t *__restrict__ fcard, CT *__restrict__ codes,
+    int row_words, int steps, unsigned long long *zero, int64_t nzero)
+{
+    extern __shared__ __align__(16) uint32_t code_rows[];         // kCodeQueries kernels' rows
+    __shared__ uint32_t dcode[kSelectMaxDevices];
+    __shared__ uint32_t scode;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t k0 = (int64_t)blockIdx.x * kCodeQueries, k = k0 + lane;
+    for (int64_t i = (int64_t)blockIdx.x * kCodeThreads + tid; i < nzero; i += (int64_t)gridDim.x * kCodeThreads) zero[i] = 0ull;
+    CT *c = reinterpret_cast<CT *>(code_rows + (size_t)lane * (size_t)row_words);
+    // the device's and the size's places and the padding: zero here, put in as the rows are written
+    for (int f = F - 2 + warp; f < row_words * 4 / (int)sizeof(CT); f += kCodeWarps) c[f] = (CT)0;
+    code_columns<CT>(F - 2, fvals, fstride, fcard, steps, warp, c,
+                     [&](int f) { return k < K ? __ldg(&kfeat[(size_t)f * (size_t)K + k]) : 0.0f; });
+    if (tid < D) dcode[tid] = code_of<CT>((float)ids[tid], fvals + (size_t)(F - 2) * (size_t)fstride, __ldg(&fcard[F - 2]), steps);
+    if (tid == kCodeThreads - 1)
+        scode = code_of<CT>((float)size_class, fvals + (size_t)(F - 1) * (size_t)fstride, __ldg(&fcard[F - 1]), steps);
+    __syncthreads();
+    constexpr int kPer = 4 / (int)sizeof(CT);
+    const int dw = (F - 2) / kPer, ds = (F - 2) % kPer * 8 * (int)sizeof(CT);
+    const int sw = (F - 1) / kPer, ss = (F - 1) % kPer * 8 * (int)sizeof(CT);
+    const int rows = (int)min((int64_t)kCodeQueries, K - k0) * D, words = rows * row_words;
+    uint32_t *dst = reinterpret_cast<uint32_t *>(codes) + (size_t)k0 * (size_t)D * (size_t)row_words;
+    for (int i = tid; i < words; i += kCodeThreads) {
+        const int r = i / row_words, w = i - r * row_words, kk = r / D, j = r - kk * D;
+        uint32_t v = code_rows[kk * row_words + w];
+        if (w == dw) v |= dcode[j] << ds;
+        if (w == sw) v |= scode << ss;
+        dst[i] = v;
+    }
 }
 
 // bytes of one feature's code for a forest: one when every value table has at most 255 values
@@ -272,10 +330,14 @@ __device__ __forceinline__ void write_query(int64_t q, int64_t acc, u128_t sq, i
 {
     if (out_sum) out_sum[q] = acc;
     if (out_pred) {
-        const i128_t num = (i128_t)2 * acc + total_trees, den = (i128_t)2 * total_trees;
-        i128_t d = num / den;
-        if (num % den != 0 && num < 0) d -= 1;
-        out_pred[q] = (int64_t)d;
+        if (total_trees <= 0xFFFFFFFFll) {
+            out_pred[q] = round_mean(acc, (uint32_t)total_trees);
+        } else {
+            const i128_t num = (i128_t)2 * acc + total_trees, den = (i128_t)2 * total_trees;
+            i128_t d = num / den;
+            if (num % den != 0 && num < 0) d -= 1;
+            out_pred[q] = (int64_t)d;
+        }
     }
     if (out_var) {
         const u128_t V = (u128_t)total_trees * sq - (u128_t)((i128_t)acc * (i128_t)acc);
@@ -958,7 +1020,7 @@ __global__ void expand_queries_kernel(const float *kfeat, int32_t K, int64_t ld,
 }
 
 // argmin over devices per kernel; ties to the lower device id
-__global__ void argmin_kernel(const int64_t *pred, const int32_t *dev, int32_t K, int32_t D, int32_t *best,
+__global__ void argmin_kernel(const int64_t *pred, DeviceIds dev, int32_t K, int32_t D, int32_t *best,
                               int64_t *out_pred)
 {
     const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1074,8 +1136,10 @@ struct WalkScratch {
     }
 };
 
-template <typename CT, bool VAR>
-int launch_predict(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t *d_sum, int64_t *d_pred,
+// Coding and walk of Q queries. code(codes, row_words, zero, zero_words) enqueues the kernel that
+// writes their code rows and clears zero_words 8-byte words.
+template <typename CT, bool VAR, typename Code>
+int launch_predict(const aiwcrf_forest *f, const Code &code, int64_t Q, int64_t *d_sum, int64_t *d_pred,
                    uint64_t *d_var, int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *codes_scratch,
                    int64_t walk_T)
 {
@@ -1086,8 +1150,7 @@ int launch_predict(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t 
     cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
     CT *d_codes = static_cast<CT *>(w.codes);
-    if ((e = launch_code_queries<CT>(f, dXq, Q, d_codes, ld_words, s, w.zero, w.zero_words)) != cudaSuccess)
-        return cuda_fail(e, "code_queries_kernel launch");
+    if ((e = code(d_codes, ld_words, w.zero, w.zero_words)) != cudaSuccess) return cuda_fail(e, "query coding launch");
     auto kern = predict_kernel<CT, kQPT, VAR>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(predict_kernel)");
@@ -1103,8 +1166,8 @@ int launch_predict(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t 
     return AIWCRF_OK;
 }
 
-template <bool VAR>
-int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t *d_sum, int64_t *d_pred,
+template <bool VAR, typename Code>
+int launch_predict4(const aiwcrf_forest *f, const Code &code, int64_t Q, int64_t *d_sum, int64_t *d_pred,
                     uint64_t *d_var, int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *codes_scratch,
                     int64_t walk_T)
 {
@@ -1115,8 +1178,7 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     cudaError_t e = w.init(Q, (size_t)Q * (size_t)ld_words * 4, smem, walk_T, VAR, codes_scratch, s);
     if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "device allocation of the query codes failed");
     uint8_t *d_codes = static_cast<uint8_t *>(w.codes);
-    if ((e = launch_code_queries<uint8_t>(f, dXq, Q, d_codes, ld_words, s, w.zero, w.zero_words)) != cudaSuccess)
-        return cuda_fail(e, "code_queries_kernel launch");
+    if ((e = code(d_codes, ld_words, w.zero, w.zero_words)) != cudaSuccess) return cuda_fail(e, "query coding launch");
     // large batches walk in the order of their leading codes (own scratch only)
     const bool sorted = !codes_scratch && Q >= kSortMinQueries && Q < ((int64_t)1 << 32) && f->key_feats[0] >= 0;
     uint32_t *perm = nullptr;
@@ -1153,17 +1215,45 @@ int launch_predict4(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t
     return AIWCRF_OK;
 }
 
+template <typename CT, typename Code>
+int launch_coded(const aiwcrf_forest *f, const Code &code, int64_t Q, int64_t *d_sum, int64_t *d_pred, uint64_t *d_var,
+                 int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *scratch, int64_t walk_T)
+{
+    if constexpr (sizeof(CT) == 1) {
+        if (f->compact)
+            return d_var ? launch_predict4<true>(f, code, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T)
+                         : launch_predict4<false>(f, code, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T);
+    }
+    return d_var ? launch_predict<CT, true>(f, code, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T)
+                 : launch_predict<CT, false>(f, code, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T);
+}
+
 template <typename CT>
 int launch_predict_ct(const aiwcrf_forest *f, const float *dXq, int64_t Q, int64_t *d_sum, int64_t *d_pred,
                       uint64_t *d_var, int64_t total_trees, cudaStream_t s, uint32_t *d_err, void *scratch = nullptr,
                       int64_t walk_T = -1)
 {
-    if (walk_T < 0) walk_T = f->T;
-    if (f->compact)
-        return d_var ? launch_predict4<true>(f, dXq, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T)
-                     : launch_predict4<false>(f, dXq, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T);
-    return d_var ? launch_predict<CT, true>(f, dXq, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T)
-                 : launch_predict<CT, false>(f, dXq, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T);
+    auto code = [&](CT *codes, int row_words, unsigned long long *zero, int64_t nzero) {
+        return launch_code_queries<CT>(f, dXq, Q, codes, row_words, s, zero, nzero);
+    };
+    return launch_coded<CT>(f, code, Q, d_sum, d_pred, d_var, total_trees, s, d_err, scratch, walk_T < 0 ? f->T : walk_T);
+}
+
+// the same for the K x D queries of a device selection (query k * D + j), D <= kSelectMaxDevices
+template <typename CT>
+int launch_select_ct(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class, const DeviceIds &ids,
+                     int32_t D, int64_t *d_pred, cudaStream_t s, uint32_t *d_err)
+{
+    const int64_t Q = (int64_t)K * D;
+    auto code = [&](CT *codes, int row_words, unsigned long long *zero, int64_t nzero) {
+        const size_t smem = (size_t)kCodeQueries * (size_t)row_words * 4;
+        const int steps = 32 - __builtin_clz(f->max_card | 1u);
+        code_selection_kernel<CT><<<(unsigned)((K + kCodeQueries - 1) / kCodeQueries), kCodeThreads, smem, s>>>(
+            d_kfeat, K, size_class, ids, D, f->F, f->d_fvals, f->fstride, f->d_fcard, codes, row_words, steps, zero, nzero);
+        count_launches(1);
+        return cudaGetLastError();
+    };
+    return launch_coded<CT>(f, code, Q, nullptr, d_pred, nullptr, f->T, s, d_err, nullptr, f->T);
 }
 
 }  // namespace
@@ -1331,40 +1421,66 @@ int round_mean_launch(const int64_t *d_sum, int64_t Q, int64_t total_trees, int6
     return AIWCRF_OK;
 }
 
-int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class,
-                  const int32_t *d_dev, int32_t D, int32_t *d_best, int64_t *d_pred, float *d_q,
-                  int64_t *d_p, cudaStream_t s)
+// Which kernels answer a device selection of K kernels x D devices:
+//  - D <= 64 and at most kTreeParallelMaxWalks walks (queries x trees): the tree-parallel kernel;
+//  - D <= 64 beyond that: the walk of predict, whose trees pass through shared memory once for 512
+//    queries, on rows coded once per kernel;
+//  - more devices: the queries written out, and predict.
+// Measured per call (us), tree-parallel / shared-memory walk, x 15 devices: 256 kernels x 500 trees 80 /
+// 90, 512 143 / 94, 1,024 250 / 130, 4,096 856 / 290; 1,024 x 50 64 / 75, 2,048 76 / 77, 4,096 149 / 95;
+// 8,192 x 16 118 / 160.
+int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class, const DeviceIds &ids,
+                  int32_t D, int32_t *d_best, int64_t *d_pred, cudaStream_t s)
 {
     const int64_t Qn = (int64_t)K * D;
-    if (D <= 64 && Qn <= kTreeParallelMaxQueries && size_class >= 0) {
-        // few queries: spread the trees over CTAs instead of the queries; the query scratch
-        // (F * Qn floats) holds the kernel's zeroed sums and counters
-        unsigned long long *d_sum = reinterpret_cast<unsigned long long *>(d_q);
-        uint32_t *d_cnt = reinterpret_cast<uint32_t *>(d_sum + Qn);
-        const cudaError_t e = cudaMemsetAsync(d_sum, 0, 8 * (size_t)Qn + 4 * (size_t)K, s);
-        if (e != cudaSuccess) return cuda_fail(e, "select scratch");
+    keep_pool_memory(f->device);
+    // one block of scratch: sums and counters of the tree-parallel kernel, or an error flag; the
+    // predictions if the caller wants none; the queries where they are written out
+    const bool tree_parallel = D <= kSelectMaxDevices && Qn * f->T <= kTreeParallelMaxWalks && size_class >= 0;
+    const bool expand = D > kSelectMaxDevices;
+    const size_t b_cnt = tree_parallel ? up256(8 * (size_t)Qn + 4 * (size_t)K) : 256;
+    const size_t b_pred = d_pred ? 0 : up256(8 * (size_t)Qn), b_q = expand ? up256(4 * (size_t)f->F * (size_t)Qn) : 0;
+    unsigned char *block = nullptr;
+    cudaError_t e = cudaMallocAsync(&block, b_cnt + b_pred + b_q, s);
+    if (e != cudaSuccess) return fail(AIWCRF_E_OOM, "select_device scratch");
+    struct Free { void *p; cudaStream_t s; ~Free() { cudaFreeAsync(p, s); } } fr{block, s};
+    int64_t *d_p = d_pred ? d_pred : reinterpret_cast<int64_t *>(block + b_cnt);
+    if ((e = cudaMemsetAsync(block, 0, tree_parallel ? 8 * (size_t)Qn + 4 * (size_t)K : 4, s)) != cudaSuccess)
+        return cuda_fail(e, "select scratch");
+    if (tree_parallel) {
+        unsigned long long *d_sum = reinterpret_cast<unsigned long long *>(block);
         prof_begin(s, kProfSelect);
-        const int rc = select_small_launch(f, d_kfeat, K, size_class, d_dev, D, d_best, d_pred ? d_pred : d_p, d_sum,
-                                           d_cnt, s);
+        const int rc = select_small_launch(f, d_kfeat, K, size_class, ids, D, d_best, d_p, d_sum,
+                                           reinterpret_cast<uint32_t *>(d_sum + Qn), s);
         prof_end(s, kProfSelect);
         return rc;
     }
-    prof_begin(s, kProfSelect);
-    expand_queries_kernel<<<(unsigned)((Qn + 255) / 256), 256, 0, s>>>(d_kfeat, K, (int64_t)K, size_class, nullptr, d_dev, D,
-                                                                        f->F,
-                                                                        d_q);
-    count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "expand_queries_kernel launch");
-    prof_end(s, kProfSelect);
-    int rc = predict_launch(f, d_q, Qn, nullptr, d_p, nullptr, f->T, s);
+    uint32_t *d_err = reinterpret_cast<uint32_t *>(block);
+    int rc = AIWCRF_OK;
+    if (expand) {
+        float *d_q = reinterpret_cast<float *>(block + b_cnt + b_pred);
+        prof_begin(s, kProfSelect);
+        rc = expand_launch(d_kfeat, K, (int64_t)K, size_class, nullptr, ids.dev, D, f->F, d_q, s);
+        prof_end(s, kProfSelect);
+        if (rc == AIWCRF_OK) rc = predict_launch(f, d_q, Qn, nullptr, d_p, nullptr, f->T, s);
+    } else {
+        prof_begin(s, kProfPredict);
+        if (f->max_card <= 255u) rc = launch_select_ct<uint8_t>(f, d_kfeat, K, size_class, ids, D, d_p, s, d_err);
+        else if (f->max_card <= 65535u) rc = launch_select_ct<uint16_t>(f, d_kfeat, K, size_class, ids, D, d_p, s, d_err);
+        else rc = launch_select_ct<uint32_t>(f, d_kfeat, K, size_class, ids, D, d_p, s, d_err);
+        prof_end(s, kProfPredict);
+    }
     if (rc != AIWCRF_OK) return rc;
     prof_begin(s, kProfSelect);
-    argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, d_dev, K, D, d_best, d_pred);
+    argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, ids, K, D, d_best, nullptr);
     count_launches(1);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "argmin_kernel launch");
     prof_end(s, kProfSelect);
+    uint32_t h_err = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(e, "select_device");
+    if (h_err & kErrTimeout) return fail(AIWCRF_E_TIMEOUT, "a bounded device wait gave up");
     return AIWCRF_OK;
 }
 
@@ -1405,7 +1521,7 @@ int select_noalloc_ct(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, i
                                                     reinterpret_cast<const CT *>(d_codes), Qn, ld_words, f->T,
                                                     tree_cap, nullptr, d_p, nullptr, d_err,
                                                     TreeParts{(int)f->T, nullptr, nullptr, nullptr});
-    argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, d_dev, K, D, d_best, d_pred);
+    argmin_kernel<<<(unsigned)((K + 127) / 128), 128, 0, s>>>(d_p, DeviceIds{d_dev}, K, D, d_best, d_pred);
     count_launches(2);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "select_device launch");

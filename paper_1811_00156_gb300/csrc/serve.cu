@@ -71,7 +71,7 @@ constexpr int kServeThreads = 256;
 constexpr int kDevSlots = 16;                             // threads of one tree slot: devices
 constexpr int kTreeSlots = kServeThreads / kDevSlots;    // 16 tree slots
 constexpr int kTreesPerBlock = 2 * kTreeSlots;            // each thread walks two trees
-constexpr int kServeMaxDevices = 64;
+constexpr int kServeMaxDevices = kSelectMaxDevices;
 
 __device__ __forceinline__ int64_t serve_leaf(uint64_t nd)
 {
@@ -193,7 +193,7 @@ __device__ __forceinline__ uint32_t rank_code(const float *V, uint32_t card, flo
 // predictions are also written to fpred as float log10 seconds.
 template <int NODES>
 __global__ void __launch_bounds__(kServeThreads) serve_select_kernel(ServeForest sf, const float *__restrict__ kq,
-                                                                     int Kb, const int32_t *__restrict__ dev, int D,
+                                                                     int Kb, DeviceIds dev, int D,
                                                                      int size_override, unsigned long long *sums,
                                                                      uint32_t *cnt, int64_t *pred, int32_t *best,
                                                                      const uint8_t *__restrict__ only, int n_gated,
@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(kServeThreads) serve_select_kernel(ServeForest
             kcode[f] = rank_code(sf.fvals + (size_t)f * (size_t)sf.fstride, sf.fcard[f],
                                  (f == sf.F - 1 && size_override >= 0) ? (float)size_override
                                                                        : kq[(size_t)f * (size_t)Kb + (size_t)k]);
-    for (int j = tid; j < D; j += kServeThreads)
+    // the devices' codes by the last warps, beside the features'
+    for (int j = kServeThreads - 1 - tid; j < D; j += kServeThreads)
         dcode[j] = rank_code(sf.fvals + (size_t)fd * (size_t)sf.fstride, sf.fcard[fd], (float)dev[j]);
     __syncthreads();
     const int t0 = g * kTreesPerBlock + ts, t1 = t0 + kTreeSlots;
@@ -242,10 +243,7 @@ __global__ void __launch_bounds__(kServeThreads) serve_select_kernel(ServeForest
     int32_t bd = INT_MAX;
     for (int j = lane; j < D; j += 32) {
         const int64_t s = (int64_t)atomicExch(&sums[(size_t)k * (size_t)D + (size_t)j], 0ull);
-        const i128_t num = (i128_t)2 * s + sf.T, den = (i128_t)2 * sf.T;
-        i128_t d = num / den;
-        if (num % den != 0 && num < 0) d -= 1;
-        const int64_t p = (int64_t)d;
+        const int64_t p = round_mean(s, (uint32_t)sf.T);
         pred[(size_t)k * (size_t)D + (size_t)j] = p;
         if (k < n_gated) fpred[(size_t)k * (size_t)D + (size_t)j] = (float)((double)p * 0x1p-32);
         const int32_t id = dev[j];
@@ -295,7 +293,7 @@ size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 constexpr int64_t kIdlePollNs = 200000;   // the dispatcher polls this long before sleeping
 
-int serve_launch(const aiwcrf_forest *f, const float *d_kq, int Kb, const int32_t *d_dev, int D, int size_override,
+int serve_launch(const aiwcrf_forest *f, const float *d_kq, int Kb, const DeviceIds &ids, int D, int size_override,
                  unsigned long long *d_sum, uint32_t *d_cnt, int64_t *d_pred, int32_t *d_best, cudaStream_t s,
                  const uint8_t *d_only = nullptr, int n_gated = 0, float *d_fpred = nullptr)
 {
@@ -316,7 +314,7 @@ int serve_launch(const aiwcrf_forest *f, const float *d_kq, int Kb, const int32_
     auto kern = nodes == kWalkScaled    ? serve_select_kernel<kWalkScaled>
                 : nodes == kWalkCompact ? serve_select_kernel<kWalkCompact>
                                         : serve_select_kernel<kWalkWide>;
-    kern<<<grid, kServeThreads, 0, s>>>(sf, d_kq, Kb, d_dev, D, size_override, d_sum, d_cnt, d_pred, d_best, d_only,
+    kern<<<grid, kServeThreads, 0, s>>>(sf, d_kq, Kb, ids, D, size_override, d_sum, d_cnt, d_pred, d_best, d_only,
                                         n_gated, d_fpred);
     prof_end(s, kProfServe);
     count_launches(1);
@@ -328,12 +326,12 @@ int serve_launch(const aiwcrf_forest *f, const float *d_kq, int Kb, const int32_
 }  // namespace
 
 int select_small_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class,
-                        const int32_t *d_dev, int32_t D, int32_t *d_best, int64_t *d_pred, unsigned long long *d_sum,
+                        const DeviceIds &ids, int32_t D, int32_t *d_best, int64_t *d_pred, unsigned long long *d_sum,
                         uint32_t *d_cnt, cudaStream_t s)
 {
     if (D > kServeMaxDevices || f->F > AIWCRF_MAX_FEATURES || size_class < 0)
         return fail(AIWCRF_E_INVALID_ARG, "select_small_launch: unsupported shape");
-    return serve_launch(f, d_kfeat, K, d_dev, D, size_class, d_sum, d_cnt, d_pred, d_best, s);
+    return serve_launch(f, d_kfeat, K, ids, D, size_class, d_sum, d_cnt, d_pred, d_best, s);
 }
 
 namespace {
@@ -756,7 +754,7 @@ struct aiwcrf_server {
                                                  sl.s) != AIWCRF_OK)
                 e = cudaErrorLaunchFailure;
         }
-        if (e == cudaSuccess && serve_launch(sl.model->f, d_in, sl.Kb, d_dev, D, -1, sl.d_sum, sl.d_cnt, d_pred, d_best,
+        if (e == cudaSuccess && serve_launch(sl.model->f, d_in, sl.Kb, DeviceIds{d_dev}, D, -1, sl.d_sum, sl.d_cnt, d_pred, d_best,
                                              sl.s, d_flag, sl.Kg, d_fpred) != AIWCRF_OK)
             e = cudaErrorLaunchFailure;
         if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_out, d_out, L.out_bytes, cudaMemcpyDeviceToHost, sl.s);
