@@ -53,7 +53,7 @@ void forest_release_async(aiwcrf_forest *f, cudaStream_t s)
     delete f;
 }
 
-cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s)
+cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s, bool upload)
 {
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     // compact layout: trees padded to a multiple of four nodes
@@ -90,7 +90,7 @@ cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s)
         unsigned char *q = c + 2 * b_nodes + b_off + b_vals + b_card;
         f->d_tree_off4 = reinterpret_cast<int64_t *>(q);
         f->d_c32 = reinterpret_cast<uint32_t *>(q + b_off);
-        e = cudaMemcpyAsync(f->d_tree_off4, off4.data(), 8 * (size_t)(f->T + 1), cudaMemcpyHostToDevice, s);
+        if (upload) e = cudaMemcpyAsync(f->d_tree_off4, off4.data(), 8 * (size_t)(f->T + 1), cudaMemcpyHostToDevice, s);
     }
     return e;
 }

@@ -2267,17 +2267,64 @@ int tree_warps(int64_t T, int sms)
     return T <= sms ? 32 : T <= 2 * (int64_t)sms ? 16 : 8;
 }
 
-// copy each tree's nodes from its output slot into the forest (and pad an odd count)
-__global__ void tree_place_kernel(const uint64_t *slot_nodes, const uint64_t *slot_cnodes, int64_t node_cap,
-                                  const uint32_t *counts, uint64_t *const *tree_dst, uint64_t *const *tree_cdst)
+// A forest's device arrays, as the packaging kernels write them.
+struct ForestPtrs {
+    uint64_t *nodes, *cnodes;
+    int64_t *off, *off4;         // off4 and c32: null without a compact form
+    uint32_t *c32;
+    float *fvals;
+    uint32_t *fcard;
+    int shift;                   // c32_shift
+};
+
+// Packaging, one CTA per tree of the batch (forest t / Tper, its tree t % Tper): the tree's nodes from
+// its output slot into the forest (slot_nodes null: they are there already), an odd count padded by
+// a never-reached leaf of value 0, the compact nodes, the tree's offsets (offs: two per tree, host
+// computed) and the split features of its top nodes (top: F counts per forest, zero on entry).
+__global__ void forest_place_kernel(const ForestPtrs *__restrict__ fp, const int64_t *__restrict__ offs, uint32_t Tper,
+                                    const uint64_t *slot_nodes, const uint64_t *slot_cnodes, int64_t node_cap,
+                                    const uint32_t *__restrict__ counts, int F, uint32_t *top)
 {
-    const int t = blockIdx.x;
-    const uint32_t c = (uint32_t)AIWCRF_IDX(counts[t], (uint64_t)node_cap, kBoundOut);
-    const uint64_t *sn = slot_nodes + (size_t)t * (size_t)node_cap, *sc = slot_cnodes + (size_t)t * (size_t)node_cap;
-    uint64_t *dn = tree_dst[t], *dc = tree_cdst[t];
-    for (uint32_t i = threadIdx.x; i < c; i += blockDim.x) { dn[i] = sn[i]; dc[i] = sc[i]; }
-    if (threadIdx.x == 0 && (c & 1u)) { dn[c] = 1ull << 63; dc[c] = 1ull << 63; }
+    const uint32_t t = blockIdx.x, g = t / Tper, k = t - g * Tper;
+    const ForestPtrs p = fp[g];
+    const uint32_t c = slot_nodes ? (uint32_t)AIWCRF_IDX(counts[t], (uint64_t)node_cap, kBoundOut) : counts[t];
+    const int64_t a = offs[2 * (size_t)t], a4 = offs[2 * (size_t)t + 1];
+    const uint32_t even = (c + 1u) & ~1u, four = (even + 3u) & ~3u;
+    uint64_t *dn = p.nodes + a, *dc = p.cnodes + a;
+    const uint64_t *sn = slot_nodes ? slot_nodes + (size_t)t * (size_t)node_cap : dn;
+    const uint64_t *sc = slot_nodes ? slot_cnodes + (size_t)t * (size_t)node_cap : dc;
+    for (uint32_t i = threadIdx.x; i < four; i += blockDim.x) {
+        const uint64_t nd = i < c ? sc[i] : 1ull << 63;
+        if (i < even && (slot_nodes || i >= c)) {
+            dc[i] = nd;
+            dn[i] = i < c ? sn[i] : nd;
+        }
+        if (p.c32) p.c32[a4 + i] = compact_node(nd, i, p.shift);
+        if (p.c32 && i < (uint32_t)kTopNodes && !(nd >> 63)) atomicAdd(&top[(size_t)g * F + ((nd >> 56) & 0x7Fu)], 1u);
+    }
+    if (threadIdx.x == 0) {
+        p.off[k] = a;
+        if (k == Tper - 1) p.off[Tper] = a + even;
+        if (p.off4) {
+            p.off4[k] = a4;
+            if (k == Tper - 1) p.off4[Tper] = a4 + four;
+        }
+    }
 }
+
+// every forest's value tables (max_card values of each feature, leading dimension N -> fstride)
+__global__ void forest_values_kernel(const ForestPtrs *__restrict__ fp, int G, int F, const float *__restrict__ vals, int64_t N,
+                                     const uint32_t *__restrict__ card, uint32_t max_card, int64_t fstride)
+{
+    const int64_t per = (int64_t)F * max_card, n = per * G;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < n; i += step) {
+        const int64_t g = i / per, r = i - g * per, f = r / max_card, v = r - f * max_card;
+        fp[g].fvals[f * fstride + v] = vals[f * N + v];
+    }
+    for (int64_t i = i0; i < (int64_t)G * F; i += step) fp[i / F].fcard[i % F] = card[i % F];
+}
+
 
 // ------------------------------------------------------------------------------------------
 // exclusive scans of flag arrays (the grouping of identical feature vectors)
@@ -2516,22 +2563,16 @@ __global__ void iota_kernel(uint32_t *v, int n)
     if (i <= n) v[i] = (uint32_t)i;
 }
 
-__global__ void pack_kernel(const PackedRec *packed, int64_t n, uint64_t *const *tree_dst, uint64_t *const *tree_cdst)
+__global__ void pack_kernel(const PackedRec *packed, int64_t n, const ForestPtrs *__restrict__ fp,
+                            const int64_t *__restrict__ offs, uint32_t Tper)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const PackedRec p = packed[i];
-    tree_dst[p.tree][p.pos] = p.node;
-    tree_cdst[p.tree][p.pos] = p.cnode;
-}
-
-// a tree with an odd node count is padded by one never-reached leaf of value 0
-__global__ void pad_kernel(const uint32_t *counts, int64_t T, uint64_t *const *tree_dst, uint64_t *const *tree_cdst)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= T) return;
-    const uint32_t c = counts[t];
-    if (c & 1u) { tree_dst[t][c] = 1ull << 63; tree_cdst[t][c] = 1ull << 63; }
+    const ForestPtrs f = fp[p.tree / Tper];
+    const int64_t at = offs[2 * (size_t)p.tree] + p.pos;
+    f.nodes[at] = p.node;
+    f.cnodes[at] = p.cnode;
 }
 
 __global__ void check_y_kernel(const int64_t *y, int64_t n, uint32_t *err)
@@ -2711,7 +2752,7 @@ struct PackIn {
 };
 
 // One forest per tree group, trees padded to an even node count (16-byte aligned); nodes placed
-// by pack_kernel, padding by pad_kernel, compact copies built. Enqueued on s; the caller
+// by pack_kernel (or taken from the tree slots), padding, compact copies and tables written. Enqueued on s; the caller
 // synchronises before using the forests.
 int package_forests(const PackIn &in, cudaStream_t s, std::vector<aiwcrf_forest *> &out)
 {
@@ -2741,7 +2782,11 @@ int package_forests(const PackIn &in, cudaStream_t s, std::vector<aiwcrf_forest 
             for (auto f : *v) forest_release(f);
         }
     } guard{&forests};
-    std::vector<uint64_t *> h_dst((size_t)T), h_cdst((size_t)T);
+    // what the packaging kernels read, uploaded at once: the forests' arrays, then every tree's offsets
+    const size_t b_ptrs = (sizeof(ForestPtrs) * (size_t)G + 15) & ~(size_t)15;
+    std::vector<unsigned char> up(b_ptrs + 16 * (size_t)T);
+    ForestPtrs *h_ptrs = reinterpret_cast<ForestPtrs *>(up.data());
+    int64_t *h_offs = reinterpret_cast<int64_t *>(up.data() + b_ptrs);
     for (int32_t g = 0; g < G; ++g) {
         aiwcrf_forest *fr = new aiwcrf_forest();
         forests[(size_t)g] = fr;
@@ -2757,19 +2802,17 @@ int package_forests(const PackIn &in, cudaStream_t s, std::vector<aiwcrf_forest 
         fr->max_card = in.max_card;
         fr->fstride = std::max<int64_t>(in.max_card, 1);
         if (in.d_inbag) { fr->oob_rows = in.N; fr->inbag_words = in.inbag_words; }
-        AIWCRF_CUDA(forest_alloc(fr, s));
+        AIWCRF_CUDA(forest_alloc(fr, s, false));
         if (in.d_inbag)
             AIWCRF_CUDA(cudaMemcpyAsync(fr->d_inbag, in.d_inbag + (size_t)g * (size_t)Tper * (size_t)in.inbag_words,
                                         sizeof(uint32_t) * (size_t)Tper * (size_t)in.inbag_words, cudaMemcpyDeviceToDevice, s));
-        AIWCRF_CUDA(cudaMemcpy2DAsync(fr->d_fvals, sizeof(float) * (size_t)fr->fstride, in.d_vals,
-                                      sizeof(float) * (size_t)in.N, sizeof(float) * (size_t)in.max_card, (size_t)F,
-                                      cudaMemcpyDeviceToDevice, s));
-        AIWCRF_CUDA(cudaMemcpyAsync(fr->d_fcard, in.d_card, sizeof(uint32_t) * (size_t)F, cudaMemcpyDeviceToDevice, s));
-        AIWCRF_CUDA(cudaMemcpyAsync(fr->d_tree_off, fr->tree_off.data(), sizeof(int64_t) * (size_t)(Tper + 1),
-                                    cudaMemcpyHostToDevice, s));
+        h_ptrs[g] = ForestPtrs{fr->d_nodes, fr->d_cnodes, fr->d_tree_off, fr->compact ? fr->d_tree_off4 : nullptr,
+                               fr->compact ? fr->d_c32 : nullptr, fr->d_fvals, fr->d_fcard, fr->c32_shift};
+        int64_t off4 = 0;
         for (int64_t k = 0; k < Tper; ++k) {
-            h_dst[(size_t)(g * Tper + k)] = fr->d_nodes + fr->tree_off[(size_t)k];
-            h_cdst[(size_t)(g * Tper + k)] = fr->d_cnodes + fr->tree_off[(size_t)k];
+            h_offs[2 * (g * Tper + k)] = fr->tree_off[(size_t)k];
+            h_offs[2 * (g * Tper + k) + 1] = off4;
+            off4 += (fr->tree_off[(size_t)k + 1] - fr->tree_off[(size_t)k] + 3) & ~(int64_t)3;
         }
         fr->stats.num_trees = Tper;
         fr->stats.total_nodes = 0;
@@ -2790,23 +2833,35 @@ int package_forests(const PackIn &in, cudaStream_t s, std::vector<aiwcrf_forest 
         }
     }
     Scratch sc(s);
-    uint64_t **d_dst = sc.get<uint64_t *>(2 * (size_t)T, &rc); if (rc) return rc;
-    AIWCRF_CUDA(cudaMemcpyAsync(d_dst, h_dst.data(), sizeof(uint64_t *) * (size_t)T, cudaMemcpyHostToDevice, s));
-    AIWCRF_CUDA(cudaMemcpyAsync(d_dst + T, h_cdst.data(), sizeof(uint64_t *) * (size_t)T, cudaMemcpyHostToDevice, s));
+    unsigned char *d_up = sc.get<unsigned char>(up.size(), &rc); if (rc) return rc;
+    uint32_t *d_top = sc.get<uint32_t>((size_t)G * (size_t)F, &rc); if (rc) return rc;
+    const ForestPtrs *d_ptrs = reinterpret_cast<const ForestPtrs *>(d_up);
+    const int64_t *d_offs = reinterpret_cast<const int64_t *>(d_up + b_ptrs);
+    AIWCRF_CUDA(cudaMemcpyAsync(d_up, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+    AIWCRF_CUDA(cudaMemsetAsync(d_top, 0, sizeof(uint32_t) * (size_t)G * (size_t)F, s));
     prof_begin(s, kProfPack);
-    if (in.slot_nodes) {
-        tree_place_kernel<<<(unsigned)T, 256, 0, s>>>(in.slot_nodes, in.slot_cnodes, in.slot_cap, in.tree_base, d_dst,
-                                                      d_dst + T);
-        AIWCRF_LAUNCH_CHECK("tree_place_kernel");
-    } else {
-        pack_kernel<<<(unsigned)((in.packed_n + 255) / 256), 256, 0, s>>>(in.packed, (int64_t)in.packed_n, d_dst, d_dst + T);
+    if (!in.slot_nodes) {
+        pack_kernel<<<(unsigned)((in.packed_n + 255) / 256), 256, 0, s>>>(in.packed, (int64_t)in.packed_n, d_ptrs, d_offs,
+                                                                         (uint32_t)Tper);
         AIWCRF_LAUNCH_CHECK("pack_kernel");
-        pad_kernel<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(in.tree_base, T, d_dst, d_dst + T);
-        AIWCRF_LAUNCH_CHECK("pad_kernel");
     }
+    forest_place_kernel<<<(unsigned)T, 256, 0, s>>>(d_ptrs, d_offs, (uint32_t)Tper, in.slot_nodes, in.slot_cnodes, in.slot_cap,
+                                                    in.tree_base, F, d_top);
+    AIWCRF_LAUNCH_CHECK("forest_place_kernel");
+    const int64_t values = (int64_t)G * F * std::max<int64_t>(in.max_card, 1);
+    forest_values_kernel<<<(unsigned)std::min<int64_t>((values + 255) / 256, 4096), 256, 0, s>>>(
+        d_ptrs, G, F, in.d_vals, in.N, in.d_card, in.max_card, std::max<int64_t>(in.max_card, 1));
+    AIWCRF_LAUNCH_CHECK("forest_values_kernel");
     prof_end(s, kProfPack);
-    for (auto fr : forests)
-        if ((rc = forest_build_compact(fr, s)) != AIWCRF_OK) return rc;
+    std::vector<uint32_t> h_top((size_t)G * (size_t)F), h_card((size_t)F);
+    {
+        HostReads hr;              // its wait also ends the reads of the uploaded host copy
+        hr.add(h_top.data(), d_top, sizeof(uint32_t) * h_top.size());
+        hr.add(h_card.data(), in.d_card, sizeof(uint32_t) * h_card.size());
+        if ((rc = hr.run(s)) != AIWCRF_OK) return rc;
+    }
+    for (int32_t g = 0; g < G; ++g)
+        if (forests[(size_t)g]->compact) forest_set_key_feats(forests[(size_t)g], h_top.data() + (size_t)g * (size_t)F, h_card.data());
     guard.keep = true;
     out = forests;
     return AIWCRF_OK;

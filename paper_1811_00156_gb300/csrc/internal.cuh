@@ -364,6 +364,18 @@ __device__ __forceinline__ uint64_t encode_split(int f, uint32_t left, uint32_t 
     return ((uint64_t)(uint32_t)f << 56) | ((uint64_t)left << 32) | (uint64_t)thr_bits;
 }
 
+// Compact 4-byte form of coded node nd at index j of its tree (see aiwcrf_forest::d_c32). A leaf (and
+// a pad) is its own child: left = j, threshold 255 (no code exceeds it), feature field 255 with the
+// top bit as the leaf flag.
+__device__ __forceinline__ uint32_t compact_node(uint64_t nd, uint32_t j, int shift)
+{
+    if (nd >> 63) return 0xFFFF0000u | j << shift;
+    return ((uint32_t)(nd >> 56) & 0x7Fu) << 24 | ((uint32_t)nd & 0xFFu) << 16 | ((uint32_t)(nd >> 32) & 0xFFFFFFu) << shift;
+}
+// nodes at the head of a tree (breadth first: its top levels) whose split features order large
+// query batches
+constexpr int kTopNodes = 7;
+
 __device__ __forceinline__ uint64_t encode_leaf(int64_t v)
 {
     return (1ull << 63) | ((uint64_t)v & 0x7FFFFFFFFFFFFFFFull);
@@ -473,8 +485,11 @@ void forest_release(aiwcrf_forest *f);
 void forest_release_async(aiwcrf_forest *f, cudaStream_t s);
 // one stream-ordered device allocation on s for the forest's arrays (nodes, coded nodes, tree
 // offsets, value tables, compact nodes); sets the compact layout's host fields from tree_off
-// and max_card
-cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s);
+// and max_card; with upload the compact layout's offsets are copied to the device)
+cudaError_t forest_alloc(aiwcrf_forest *f, cudaStream_t s, bool upload = true);
+// sets the features that order large query batches from how often the trees' first kTopNodes nodes
+// split on each feature, and the tables' sizes
+void forest_set_key_feats(aiwcrf_forest *f, const uint32_t *top_counts, const uint32_t *card);
 // fills the compact 4-byte node array from d_cnodes (after d_cnodes and d_tree_off are written)
 int forest_build_compact(aiwcrf_forest *f, cudaStream_t s);
 // keep freed stream-ordered allocations cached in the device's default pool (once per device)

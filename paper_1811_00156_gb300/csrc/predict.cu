@@ -465,18 +465,7 @@ __global__ void compact_nodes_kernel(const uint64_t *__restrict__ cnodes, const 
     const int64_t a = tree_off[t], m = tree_off[t + 1] - a;
     const int64_t a4 = tree_off4[t], m4 = tree_off4[t + 1] - a4;
     for (int64_t j = threadIdx.x; j < m4; j += blockDim.x) {
-        // a leaf (and a pad) is its own child: left = j, threshold 255 (no code exceeds it),
-        // feature field 255 with the top bit as the leaf flag
-        uint32_t v = 0xFFFF0000u | (uint32_t)j << shift;
-        if (j < m) {
-            const uint64_t nd = cnodes[a + j];
-            if (!(nd >> 63)) {
-                const uint32_t f = (uint32_t)(nd >> 56) & 0x7Fu;
-                const uint32_t lc = (uint32_t)(nd >> 32) & 0xFFFFFFu;
-                const uint32_t code = (uint32_t)nd & 0xFFFFFFu;
-                v = (f << 24) | (code << 16) | lc << shift;
-            }
-        }
+        const uint32_t v = compact_node(j < m ? cnodes[a + j] : 1ull << 63, (uint32_t)j, shift);
         c32[a4 + j] = v;
     }
 }
@@ -641,7 +630,6 @@ __global__ void __launch_bounds__(kPredThreads) predict4_kernel(
 }
 
 // Split features of every tree's first kTopNodes nodes (breadth-first: the top levels).
-constexpr int kTopNodes = 7;
 __global__ void top_features_kernel(const uint64_t *__restrict__ cnodes, const int64_t *__restrict__ tree_off, int T,
                                     uint32_t *counts)
 {
@@ -1401,14 +1389,19 @@ int forest_build_compact(aiwcrf_forest *f, cudaStream_t s)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cudaFreeAsync(d_cnt, s);
     if (e != cudaSuccess) return cuda_fail(e, "top split features");
+    forest_set_key_feats(f, h.data(), card.data());
+    return AIWCRF_OK;
+}
+
+void forest_set_key_feats(aiwcrf_forest *f, const uint32_t *top_counts, const uint32_t *card)
+{
     std::vector<int> order((size_t)f->F);
     for (int i = 0; i < f->F; ++i) order[(size_t)i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return h[(size_t)x] > h[(size_t)y]; });
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return top_counts[x] > top_counts[y]; });
     for (int k = 0; k < 4; ++k) {
-        f->key_feats[k] = (k < f->F && h[(size_t)order[(size_t)k]] > 0) ? order[(size_t)k] : -1;
-        f->key_bits[k] = f->key_feats[k] < 0 ? 0 : 32 - __builtin_clz(card[(size_t)f->key_feats[k]] | 1u);
+        f->key_feats[k] = (k < f->F && top_counts[order[(size_t)k]] > 0) ? order[(size_t)k] : -1;
+        f->key_bits[k] = f->key_feats[k] < 0 ? 0 : 32 - __builtin_clz(card[f->key_feats[k]] | 1u);
     }
-    return AIWCRF_OK;
 }
 
 int round_mean_launch(const int64_t *d_sum, int64_t Q, int64_t total_trees, int64_t *d_out, cudaStream_t s)
