@@ -2,8 +2,8 @@
 // of the learned surrogate's training and inference kernels.
 //
 // tc_gemm_kernel: C = A * B^T with A (M x K) and B (N x K) in BF16; one CTA owns 128 rows of C
-// and a range of K. Every 64-wide K chunk of A and B is staged into shared memory in the
-// K-major core-matrix layout (transposing on the way when an operand is stored K x M), one
+// and a range of K. Every 64-wide K chunk of A and B is staged into shared memory in core matrices
+// (K-major, or MN-major when an operand is stored K x M), one
 // thread issues four 128 x N x 16 MMAs into the TMEM accumulator and commits them to an
 // mbarrier; four warps then read the accumulator rows with tcgen05.ld. K ranges of several
 // CTAs (split K) are summed afterwards in a fixed order.
@@ -22,51 +22,34 @@ using bf16 = __nv_bfloat16;
 
 constexpr int kGemmThreads = 128;
 
-// Stage rows [r0, r0 + rows) x K-elements [k0, k0 + 64) of an operand into a core-matrix tile.
-// Element (r, k) of the operand is G[r * ld + k] (stored row by row) or G[k * ld + r] (stored
-// K x rows, TRANS). Outside [0, rmax) x [0, K) the tile holds zeros. ld is a multiple of 8 and
-// G 16-byte aligned.
+// Stage rows [r0, r0 + rows) x K-elements [k0, k0 + 64) of an operand into a tile of 8 x 8 core
+// matrices. Element (r, k) of the operand is G[r * ld + k] (stored row by row): 16 bytes of a core
+// matrix are 8 K-elements of a row (K-major). Or G[k * ld + r] (stored K x rows, TRANS): 16 bytes are 8
+// rows at one k (MN-major), which the MMA reads transposed, so that both kinds go from 16-byte loads
+// to 16-byte stores. Outside [0, rmax) x [0, K) the tile holds zeros. ld is a multiple of 8 and G
+// 16-byte aligned.
 template <bool TRANS>
 __device__ __forceinline__ void stage_tile(unsigned char *tile, const bf16 *__restrict__ G, int ld, int r0, int rows,
                                            int rmax, int k0, int K)
 {
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    if (!TRANS) {
-        for (int p = threadIdx.x; p < rows * 8; p += blockDim.x) {
-            const int r = p >> 3, kk = (p & 7) * 8;
-            const int gr = r0 + r, gk = k0 + kk;
-            uint4 v = zero;
-            if (gr < rmax) {
-                if (gk + 8 <= K) {
-                    v = __ldg(reinterpret_cast<const uint4 *>(G + (size_t)gr * (size_t)ld + gk));
-                } else if (gk < K) {
-                    uint16_t h[8];
-                    for (int i = 0; i < 8; ++i)
-                        h[i] = gk + i < K ? __bfloat16_as_ushort(G[(size_t)gr * (size_t)ld + gk + i]) : (uint16_t)0;
-                    v = make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
-                                   h[6] | (uint32_t)h[7] << 16);
-                }
-            }
-            *reinterpret_cast<uint4 *>(tile + tc::core_offset((uint32_t)r, (uint32_t)kk)) = v;
-        }
-    } else {
-        const int rgroups = rows >> 3;
-        for (int p = threadIdx.x; p < rgroups * 64; p += blockDim.x) {
-            const int k = p / rgroups, rg = p % rgroups;
-            const int gk = k0 + k, gr = r0 + rg * 8;
+    // a run: 8 elements that are adjacent in memory, along K or along the rows
+    const int rgroups = rows >> 3;
+    for (int p = threadIdx.x; p < rows * 8; p += blockDim.x) {
+        const int r = TRANS ? (p % rgroups) * 8 : p >> 3, kk = TRANS ? p / rgroups : (p & 7) * 8;
+        const int gr = r0 + r, gk = k0 + kk;
+        const bf16 *src = TRANS ? G + (size_t)gk * (size_t)ld + gr : G + (size_t)gr * (size_t)ld + gk;
+        const int in = (TRANS ? gk < K : gr < rmax) ? (TRANS ? rmax - gr : K - gk) : 0;     // elements that exist
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (in >= 8) {
+            v = __ldg(reinterpret_cast<const uint4 *>(src));
+        } else if (in > 0) {
             uint16_t h[8];
-            if (gk < K && gr + 8 <= rmax) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(G + (size_t)gk * (size_t)ld + gr));
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-                for (int i = 0; i < 4; ++i) { h[2 * i] = (uint16_t)w[i]; h[2 * i + 1] = (uint16_t)(w[i] >> 16); }
-            } else {
-                for (int i = 0; i < 8; ++i)
-                    h[i] = (gk < K && gr + i < rmax) ? __bfloat16_as_ushort(G[(size_t)gk * (size_t)ld + gr + i])
-                                                     : (uint16_t)0;
-            }
-            for (int i = 0; i < 8; ++i)
-                *reinterpret_cast<uint16_t *>(tile + tc::core_offset((uint32_t)(rg * 8 + i), (uint32_t)k)) = h[i];
+            for (int i = 0; i < 8; ++i) h[i] = i < in ? __bfloat16_as_ushort(src[i]) : (uint16_t)0;
+            v = make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
+                           h[6] | (uint32_t)h[7] << 16);
         }
+        const uint32_t at = TRANS ? tc::core_offset_mn((uint32_t)r, (uint32_t)kk) : tc::core_offset((uint32_t)r, (uint32_t)kk);
+        *reinterpret_cast<uint4 *>(tile + at) = v;
     }
 }
 
@@ -102,7 +85,7 @@ __global__ void __launch_bounds__(kGemmThreads) tc_gemm_kernel(const bf16 *__res
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = tmem_base;
-    const uint32_t idesc = tc::make_idesc_bf16(128, (uint32_t)NT);
+    const uint32_t idesc = tc::make_idesc_bf16(128, (uint32_t)NT, AT, BT);
 
     bool ok = true;
     uint32_t phase = 0;

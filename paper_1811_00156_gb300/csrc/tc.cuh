@@ -40,10 +40,19 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo, uint
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
 
-// instruction descriptor of kind::f16: D = F32, A = B = BF16, both K-major, M x N
-__host__ __device__ constexpr uint32_t make_idesc_bf16(uint32_t M, uint32_t N)
+// the same for a tile whose core matrices are MN-major: 8 K-rows of 16 bytes, each 8 elements along
+// M/N. The core matrices lie as above (adjacent along K kLbo apart, along M/N kSbo), so that the
+// descriptor's strides are the same.
+__device__ __forceinline__ uint32_t core_offset_mn(uint32_t r, uint32_t k)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+    return ((r >> 3) * 8u + (k >> 3)) * kCoreBytes + (k & 7u) * 16u + (r & 7u) * 2u;
+}
+
+// instruction descriptor of kind::f16: D = F32, A = B = BF16, M x N; each operand K-major or MN-major
+__host__ __device__ constexpr uint32_t make_idesc_bf16(uint32_t M, uint32_t N, bool a_mn = false, bool b_mn = false)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u) | ((N >> 3) << 17) |
+           ((M >> 4) << 24);
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t *smem_dst, uint32_t ncols)
