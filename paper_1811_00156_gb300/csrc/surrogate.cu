@@ -3,9 +3,9 @@
 // for columns spanning orders of magnitude), one-hot device and size class, padded to 64;
 // layers 64 -> 256 -> 256 -> 1 with GELU; BF16 weights and activations, FP32 accumulation.
 //
-// Training (Adam, MSE on the forest's log10-time predictions) runs as a stream of kernels per
-// batch: encode, two tensor-core GEMMs forward, three backward (weight gradients with the batch
-// as K, split over CTAs), fixed-order column sums for the biases, Adam, and BF16 weight copies.
+// Training (Adam, MSE on the forest's log10-time predictions) runs five kernels per batch: encoding
+// with layer 1, layer 2, the backward pass to both pre-activations, the weight gradients (the batch
+// as K, split over CTAs), and fixed-order sums with Adam and the BF16 weight copies.
 // Inference is one persistent fused kernel: both weight matrices stay in shared memory; for
 // every 128 queries the encoded tile is written straight into the MMA operand layout, layer 1
 // accumulates into TMEM columns 0..255 and layer 2 into 256..511, and the epilogues apply bias
@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <random>
@@ -36,11 +37,6 @@ constexpr int ob2 = oW2 + kHid * kHid;
 constexpr int ow3 = ob2 + kHid;
 constexpr int ob3 = ow3 + kHid;
 constexpr int kParams = ob3 + 1;
-
-__device__ __forceinline__ float gelu(float x)
-{
-    return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f));
-}
 
 // GELU of the inference epilogues, two values at a time: the packed FP32 instructions halve those
 // of the polynomials.
@@ -147,9 +143,11 @@ __device__ __forceinline__ uint64_t gelu2(uint64_t x)
     return fma2(s, pack2(exp2_approx(q0), exp2_approx(q1)), pack2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f)));
 }
 
-__device__ __forceinline__ float gelu_grad(float x)
+// two floats as BF16 (round to nearest even) in one word, the first in the low half
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
-    return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
 }
 
 struct Encoder {
@@ -180,134 +178,484 @@ __device__ __forceinline__ float encode_value(const Encoder &e, const float *X, 
 // ------------------------------------------------------------------------------------------
 // training kernels
 // ------------------------------------------------------------------------------------------
-// step: when set, the batch starts at row (*step mod spe) * B of the permutation instead of r0
-// (a replayed training step reads its place in the epoch from the device step counter)
-__global__ void encode_batch_kernel(Encoder e, const float *__restrict__ X, int64_t ld, const uint32_t *__restrict__ perm,
-                                    int64_t r0, int B, const float *__restrict__ yall, bf16 *__restrict__ xin,
-                                    float *__restrict__ yb, const int64_t *step, int64_t spe)
+// One step (forward, backward, gradient sums) is five kernels. A tile is 128 rows of the batch; its
+// BF16 matrices (inputs, activations, pre-activation gradients) live in global memory in the core
+// matrix order of the MMA operands, so that the next kernel fetches a tile with bulk copies and reads
+// it as it lies: by rows as a K-major operand, or transposed as an MN-major one for the weight
+// gradients. What bounds a step at 4,096 rows is latency: 2 GFLOP are a microsecond of the tensor
+// cores, and as twenty kernels (a GEMM, its elementwise work and every sum apart) it took 209 us of
+// device time and a 4,096-row gradient 223 us; this takes 53 (cold caches) and 77, the launches and
+// the wait now about half of it.
+// FP32 values per row and column are stored [tile][column][row]: a warp's lanes are 32 rows.
+constexpr int kTrainThreads = 512;               // 16 warps: four per TMEM lane quarter, 16 columns each
+constexpr int kSlices = 4;                       // CTAs of a tile, 64 of the 256 columns each
+constexpr int kSliceCols = kHid / kSlices;
+constexpr int kTileX = 128 * kIn * 2, kTileH = 128 * kHid * 2;      // bytes of a tile's matrices
+constexpr int kMaxSplits = 64;                   // of the batch's tiles, for the weight gradients
+
+// byte offset of element (row, col) of a 128 x C tile
+template <int C>
+__host__ __device__ constexpr uint32_t tile_offset(uint32_t row, uint32_t col)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B * kIn) return;
-    if (step) r0 = (*step % spe) * (int64_t)B;
-    const int b = i / kIn, k = i % kIn;
-    const int64_t row = perm ? (int64_t)perm[r0 + b] : r0 + b;
-    xin[i] = __float2bfloat16_rn(encode_value(e, X, ld, row, k));
-    if (k == 0 && yb) yb[b] = yall[row];
+    return ((row >> 3) * (uint32_t)(C / 8) + (col >> 3)) * tc::kCoreBytes + (row & 7u) * 16u + (col & 7u) * 2u;
 }
 
-// z1 += b1 (kept for the backward pass); h1 = BF16(GELU(z1))
-__global__ void act1_kernel(float *__restrict__ z1, const float *__restrict__ b1, bf16 *__restrict__ h1, int n)
+struct TrainArgs {
+    Encoder e;
+    const float *X;              // F x ld inputs
+    int64_t ld;
+    const uint32_t *perm;        // row order, or null
+    int64_t r0;
+    const float *yall;
+    const int64_t *step;         // when set, the batch starts at row (*step mod spe) * B of the order
+    int64_t spe;
+    int B;
+    const float *P;              // parameters
+    const bf16 *W1b, *W2b;
+    unsigned char *xt, *ht, *dz2t, *dz1t;        // BF16 tiles: inputs, layer-1 activations, gradients
+    float *yb;                   // B targets
+    float *g1, *g2, *h2;         // GELU'(z1), GELU'(z2), GELU(z2): [tile][column][row]
+    float *dots;                 // B x 32 partial sums of the output dot
+    float *db1, *db2, *dw3;      // [tile][column] sums over the tile's rows
+    float *dloss;                // [tile][2]: sums of dout and of the loss
+    float *w2part, *w1part;      // [split][256][256], [split][256][64]
+    int splits;
+    uint32_t *err;
+};
+
+__device__ __forceinline__ void gelu_both(float x, float &h, float &g)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float z = z1[i] + b1[i % kHid];
-    z1[i] = z;
-    h1[i] = __float2bfloat16_rn(gelu(z));
+    const float e = erff(x * 0.70710678118654752f);
+    h = 0.5f * x * (1.0f + e);
+    g = 0.5f * (1.0f + e) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// one warp per row: z2 += b2, h2 = GELU(z2), out = h2 . w3 + b3, dout = (out - y) / B
-__global__ void act2_out_kernel(float *__restrict__ z2, const float *__restrict__ b2, const float *__restrict__ w3,
-                                const float *__restrict__ b3, float *__restrict__ h2, const float *__restrict__ y, int B,
-                                float *__restrict__ out, float *__restrict__ dout, float *__restrict__ loss_rows)
+// What the training kernels share: an mbarrier for copies and one for MMAs, an accumulator of ncols
+// TMEM columns, and an orderly end when a bounded wait runs out.
+__device__ __forceinline__ void train_begin(uint64_t *bar_c, uint64_t *bar_m, uint32_t *tmem_base, uint32_t ncols)
 {
-    const int b = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (b >= B) return;
-    float dot = 0.0f;
-    for (int j = lane; j < kHid; j += 32) {
-        const float z = z2[(size_t)b * kHid + j] + b2[j];
-        z2[(size_t)b * kHid + j] = z;
-        const float h = gelu(z);
-        h2[(size_t)b * kHid + j] = h;
-        dot += h * w3[j];
+    if (threadIdx.x < 32) {
+        tc::tmem_alloc(tmem_base, ncols);
+        tc::tmem_relinquish();
     }
+    if (threadIdx.x == 0) {
+        tc::mbar_init(bar_c, 1);
+        tc::mbar_init(bar_m, 1);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+}
+
+__device__ __forceinline__ void train_end(bool ok, uint32_t tbase, uint32_t ncols, uint32_t *err)
+{
+    if (!ok && threadIdx.x == 0) atomicOr(err, kErrTimeout);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (threadIdx.x < 32) tc::tmem_dealloc(tbase, ncols);
+}
+
+// every thread: the barrier's phase is complete (false for the whole CTA if a wait ran out)
+__device__ __forceinline__ bool train_wait(uint64_t *bar, uint32_t phase)
+{
+    bool ok = __syncthreads_and(tc::mbar_wait(bar, phase));
+    if (!ok) tc::mbar_wait(bar, phase);         // once more for what is still in flight, then give up
+    tc::fence_after_sync();
+    return ok;
+}
+
+// rows of a weight matrix stored [n][ld] as a K-major tile of 64 n x K (n of tile row r is row_of(r))
+template <int K, typename RowOf>
+__device__ __forceinline__ void stage_weights(unsigned char *dst, const bf16 *__restrict__ W, int ld, const RowOf &row_of)
+{
+    for (int i = threadIdx.x; i < kSliceCols * (K / 8); i += kTrainThreads) {
+        const int r = i / (K / 8), k = (i % (K / 8)) * 8;
+        *reinterpret_cast<uint4 *>(dst + tile_offset<K>((uint32_t)r, (uint32_t)k)) =
+            __ldg(reinterpret_cast<const uint4 *>(W + (size_t)row_of(r) * (size_t)ld + k));
+    }
+}
+
+// the tile's 128 x 64 accumulator columns [16 group, 16 group + 16) of this thread's row
+__device__ __forceinline__ void train_acc(uint32_t tbase, int q4, int group, float (&x)[16])
+{
+    uint32_t v[16];
+    tc::tmem_start16(tbase + ((uint32_t)(32 * q4) << 16) + 16u * group, v);
+    tc::tmem_wait16(v);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(kFull, dot, o);
-    if (lane == 0) {
-        const float o = dot + b3[0];
-        if (out) out[b] = o;
-        if (y) {
-            const float d = o - y[b];
-            dout[b] = d / (float)B;
-            loss_rows[b] = 0.5f * d * d;
+    for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
+}
+
+// CTA (slice, tile): encode the tile's rows, layer 1's columns [64 slice, ...): activations and GELU'.
+__global__ void __launch_bounds__(kTrainThreads) train_layer1_kernel(TrainArgs a)
+{
+    __shared__ __align__(1024) unsigned char sX[kTileX];
+    __shared__ __align__(1024) unsigned char sW[kSliceCols * kIn * 2];
+    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
+    const int64_t tile = blockIdx.y;
+    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    {   // thread (row, part) encodes inputs [8 part, 8 part + 8) and [32 + 8 part, ...) of one row; the
+        // row's values are loaded together before any is used
+        const int row = tid & 127, part = tid >> 7;
+        const int64_t r0 = a.step ? (*a.step % a.spe) * (int64_t)a.B : a.r0, at = r0 + tile * 128 + row;
+        const int64_t src = a.perm ? (int64_t)a.perm[at] : at;
+        float x[16], mu[16], sd[16];
+        bool lg[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = (i < 8 ? 0 : 24) + 8 * part + i;
+            x[i] = k < a.e.n_aiwc ? __ldg(&a.X[(size_t)k * (size_t)a.ld + src]) : 0.0f;
+            mu[i] = k < a.e.n_aiwc ? __ldg(&a.e.mu[k]) : 0.0f;
+            sd[i] = k < a.e.n_aiwc ? __ldg(&a.e.sd[k]) : 1.0f;
+            lg[i] = k < a.e.n_aiwc && __ldg(&a.e.logf[k]);
+        }
+        const float dev = __ldg(&a.X[(size_t)a.e.n_aiwc * (size_t)a.ld + src]);
+        const float size = __ldg(&a.X[(size_t)(a.e.n_aiwc + 1) * (size_t)a.ld + src]);
+        if (slice == 0 && part == 0) a.yb[tile * 128 + row] = a.yall[src];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = (i < 8 ? 0 : 24) + 8 * part + i, d = k - a.e.n_aiwc, z = d - a.e.n_dev;
+            if (d < 0) x[i] = ((lg[i] ? log2f(fmaxf(x[i], 1.0f)) : x[i]) - mu[i]) / sd[i];
+            else x[i] = z < 0 ? (dev == (float)d ? 1.0f : 0.0f) : z < a.e.n_size && size == (float)z ? 1.0f : 0.0f;
+        }
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const uint32_t off = tile_offset<kIn>((uint32_t)row, (uint32_t)(32 * g + 8 * part));
+            const float *v = x + 8 * g;
+            const uint4 w = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
+                                       pack_bf16x2(v[6], v[7]));
+            *reinterpret_cast<uint4 *>(sX + off) = w;
+            if (slice == 0) *reinterpret_cast<uint4 *>(a.xt + (size_t)tile * kTileX + off) = w;
         }
     }
-}
-
-// dz2 = dout * w3 * GELU'(z2)
-__global__ void back2_kernel(const float *__restrict__ z2, const float *__restrict__ w3, const float *__restrict__ dout,
-                             bf16 *__restrict__ dz2b, float *__restrict__ dz2f, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int b = i / kHid, j = i % kHid;
-    const float d = dout[b] * w3[j] * gelu_grad(z2[i]);
-    dz2f[i] = d;
-    dz2b[i] = __float2bfloat16_rn(d);
-}
-
-// dz1 = dh1 * GELU'(z1)
-__global__ void back1_kernel(const float *__restrict__ dh1, const float *__restrict__ z1, bf16 *__restrict__ dz1b,
-                             float *__restrict__ dz1f, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float d = dh1[i] * gelu_grad(z1[i]);
-    dz1f[i] = d;
-    dz1b[i] = __float2bfloat16_rn(d);
-}
-
-// dst[j] = sum_b v[b][j] (* w[b]) for the kHid columns of v (leading dimension kHid), in two
-// fixed-order passes with coalesced reads: block (g, c) sums columns [32 g, 32 g + 32) over the
-// c-th of kColChunks row ranges (eight row lanes, then the lanes in order) into part; then
-// colsum_finish_kernel adds the kColChunks partial sums of each column in order.
-constexpr int kColChunks = 16;
-
-__global__ void __launch_bounds__(256) colsum_part_kernel(const float *__restrict__ v, int rows,
-                                                          const float *__restrict__ w, float *__restrict__ part)
-{
-    __shared__ float red[8][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + tx;
-    const int per = (rows + kColChunks - 1) / kColChunks;
-    const int r0 = blockIdx.y * per, r1 = min(rows, r0 + per);
-    float s = 0.0f;
-    for (int b = r0 + ty; b < r1; b += 8) s += v[(size_t)b * kHid + c] * (w ? w[b] : 1.0f);
-    red[ty][tx] = s;
+    stage_weights<kIn>(sW, a.W1b + (size_t)slice * kSliceCols * kIn, kIn, [](int r) { return r; });
+    tc::fence_smem_to_async();
     __syncthreads();
-    if (ty == 0) {
-        float t = 0.0f;
+    const uint32_t tbase = tmem_base;
+    if (tid == 0) {
+        tc::fence_after_sync();
+        const uint32_t a0 = tc::smem_addr(sX), w0 = tc::smem_addr(sW), idesc = tc::make_idesc_bf16(128, kSliceCols);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) t += red[k][tx];
-        part[blockIdx.y * kHid + c] = t;
+        for (int s = 0; s < kIn / 16; ++s)
+            tc::mma_bf16(tbase, tc::make_desc(a0 + 256u * s, 128u, kIn / 8 * 128u), tc::make_desc(w0 + 256u * s, 128u, kIn / 8 * 128u),
+                         idesc, s > 0 ? 1u : 0u);
+        tc::mma_commit(&bar_m);
     }
+    const bool ok = train_wait(&bar_m, 0u);
+    if (ok) {
+        const int q4 = warp & 3, group = warp >> 2, row = 32 * q4 + lane, col0 = kSliceCols * slice + 16 * group;
+        float x[16], h[16];
+        train_acc(tbase, q4, group, x);
+        float *g1 = a.g1 + ((size_t)tile * kHid + col0) * 128 + row;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            float g;
+            gelu_both(x[i] + __ldg(&a.P[ob1 + col0 + i]), h[i], g);
+            g1[(size_t)i * 128] = g;
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+            *reinterpret_cast<uint4 *>(a.ht + (size_t)tile * kTileH + tile_offset<kHid>((uint32_t)row, (uint32_t)(col0 + 8 * p))) =
+                make_uint4(pack_bf16x2(h[8 * p], h[8 * p + 1]), pack_bf16x2(h[8 * p + 2], h[8 * p + 3]),
+                           pack_bf16x2(h[8 * p + 4], h[8 * p + 5]), pack_bf16x2(h[8 * p + 6], h[8 * p + 7]));
+    }
+    train_end(ok, tbase, 64, a.err);
 }
 
-__global__ void colsum_finish_kernel(const float *__restrict__ part, float *__restrict__ dst)
+// CTA (slice, tile): layer 2's columns n = 32 m + 8 slice + i (m, i < 8), in the order 8 i + m: GELU,
+// GELU' and, for each 8 slice + i, the sum over m of GELU(z2) w3: one of the 32 partial sums of the output,
+// in a fixed order.
+constexpr int kLayer2Smem = kTileH + kSliceCols * kHid * 2;
+__global__ void __launch_bounds__(kTrainThreads) train_layer2_kernel(TrainArgs a)
 {
-    const int j = threadIdx.x;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *sH = sm, *sW = sm + kTileH;
+    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
+    const int64_t tile = blockIdx.y;
+    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    if (tid == 0) {
+        tc::mbar_expect(&bar_c, kTileH);
+        tc::bulk_load(sH, a.ht + (size_t)tile * kTileH, kTileH, &bar_c);
+    }
+    stage_weights<kHid>(sW, a.W2b, kHid, [slice](int r) { return 32 * (r & 7) + 8 * slice + (r >> 3); });
+    tc::fence_smem_to_async();
+    const uint32_t tbase = tmem_base;
+    bool ok = train_wait(&bar_c, 0u);
+    if (ok) {
+        if (tid == 0) {
+            const uint32_t a0 = tc::smem_addr(sH), w0 = tc::smem_addr(sW), idesc = tc::make_idesc_bf16(128, kSliceCols);
+#pragma unroll
+            for (int s = 0; s < kHid / 16; ++s)
+                tc::mma_bf16(tbase, tc::make_desc(a0 + 256u * s, 128u, kHid / 8 * 128u),
+                             tc::make_desc(w0 + 256u * s, 128u, kHid / 8 * 128u), idesc, s > 0 ? 1u : 0u);
+            tc::mma_commit(&bar_m);
+        }
+        ok = train_wait(&bar_m, 0u);
+    }
+    if (ok) {
+        const int q4 = warp & 3, group = warp >> 2, row = 32 * q4 + lane;
+        float x[16];
+        train_acc(tbase, q4, group, x);
+        float *dots = a.dots + ((size_t)tile * 128 + row) * 32 + 8 * slice + 2 * group;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float dot = 0.0f;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const int n = 32 * m + 8 * slice + 2 * group + i;
+                float h, g;
+                gelu_both(x[8 * i + m] + __ldg(&a.P[ob2 + n]), h, g);
+                dot += h * __ldg(&a.P[ow3 + n]);
+                const size_t at = ((size_t)tile * kHid + n) * 128 + row;
+                a.h2[at] = h;
+                a.g2[at] = g;
+            }
+            dots[i] = dot;
+        }
+    }
+    train_end(ok, tbase, 64, a.err);
+}
+
+// sum of a tile column's 128 values v(row), by one warp
+template <typename Value>
+__device__ __forceinline__ float column_sum(int lane, const Value &v)
+{
     float s = 0.0f;
-    for (int y = 0; y < kColChunks; ++y) s += part[y * kHid + j];
-    dst[j] = s;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += v(32 * k + lane);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    return s;
 }
 
-// c12: when set, the bias corrections of step *step are c12[2 * step] and c12[2 * step + 1]
-// (computed on the host for every step, as c1 and c2 are otherwise)
-__global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, int n, float lr, float beta1, float beta2, float eps, float c1, float c2,
-                            const float *__restrict__ c12, const int64_t *step)
+// CTA (slice, tile): the outputs and their errors, dz2 = dout w3 GELU'(z2) of the whole tile, and the
+// columns k of [64 slice, ...) of dh1 = dz2 W2 and dz1 = dh1 GELU'(z1); sums over the tile's rows of dz2,
+// GELU(z2) dout and dz1 for the slice's columns.
+constexpr int kBackSmem = kTileH + kSliceCols * kHid * 2;
+__global__ void __launch_bounds__(kTrainThreads) train_back_kernel(TrainArgs a)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (c12) { c1 = c12[2 * *step]; c2 = c12[2 * *step + 1]; }
-    const float gi = g[i];
-    const float mi = beta1 * m[i] + (1.0f - beta1) * gi;
-    const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *sZ = sm, *sW = sm + kTileH;       // dz2 (later dz1's columns in FP32), W2's columns
+    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ uint32_t tmem_base;
+    __shared__ float dout_s[128], w3s[kHid];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
+    const int64_t tile = blockIdx.y;
+    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    // thread (row, part) computes dz2 of one row's columns [64 part, ...): half of GELU' loaded ahead
+    const int zrow = tid & 127, part = tid >> 7;
+    const float *g2z = a.g2 + ((size_t)tile * kHid + kSliceCols * part) * 128 + zrow;
+    float gz[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) gz[i] = __ldg(&g2z[(size_t)i * 128]);
+    if (tid < 128) {
+        // the 32 partial sums in the order of a warp's butterfly
+        const float4 *d4 = reinterpret_cast<const float4 *>(a.dots + ((size_t)tile * 128 + tid) * 32);
+        float s[32];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 v = d4[i];
+            s[4 * i] = v.x; s[4 * i + 1] = v.y; s[4 * i + 2] = v.z; s[4 * i + 3] = v.w;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; ++i) s[i] += s[i + o];
+        const float d = s[0] + a.P[ob3] - a.yb[tile * 128 + tid];
+        dout_s[tid] = d / (float)a.B;
+        if (slice == 0) {
+            float sd = d / (float)a.B, sl = 0.5f * d * d;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sd += __shfl_xor_sync(kFull, sd, o);
+                sl += __shfl_xor_sync(kFull, sl, o);
+            }
+            if (lane == 0) { a.dloss[8 * tile + 2 * warp] = sd; a.dloss[8 * tile + 2 * warp + 1] = sl; }
+        }
+    } else if (tid - 128 < kHid) {
+        w3s[tid - 128] = a.P[ow3 + tid - 128];
+    }
+    // W2[n][64 slice + c] with K = n: 16 bytes are 8 columns of one n
+    for (int i = tid; i < kHid * (kSliceCols / 8); i += kTrainThreads) {
+        const int n = i / (kSliceCols / 8), c = (i % (kSliceCols / 8)) * 8;
+        *reinterpret_cast<uint4 *>(sW + tile_offset<kSliceCols>((uint32_t)n, (uint32_t)c)) =
+            __ldg(reinterpret_cast<const uint4 *>(a.W2b + (size_t)n * kHid + kSliceCols * slice + c));
+    }
+    __syncthreads();
+    {
+        const float dout = dout_s[zrow];
+#pragma unroll
+        for (int c = 0; c < kSliceCols; c += 8) {
+            float d[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                d[i] = dout * w3s[kSliceCols * part + c + i] * gz[(c + i) & 31];
+                if (c < 32) gz[c + i] = __ldg(&g2z[(size_t)(32 + c + i) * 128]);
+            }
+            const uint4 v = make_uint4(pack_bf16x2(d[0], d[1]), pack_bf16x2(d[2], d[3]), pack_bf16x2(d[4], d[5]),
+                                       pack_bf16x2(d[6], d[7]));
+            const uint32_t off = tile_offset<kHid>((uint32_t)zrow, (uint32_t)(kSliceCols * part + c));
+            *reinterpret_cast<uint4 *>(sZ + off) = v;
+            if (part == slice) *reinterpret_cast<uint4 *>(a.dz2t + (size_t)tile * kTileH + off) = v;
+        }
+    }
+    tc::fence_smem_to_async();
+    __syncthreads();
+    const uint32_t tbase = tmem_base;
+    if (tid == 0) {
+        tc::fence_after_sync();
+        const uint32_t a0 = tc::smem_addr(sZ), w0 = tc::smem_addr(sW), idesc = tc::make_idesc_bf16(128, kSliceCols, false, true);
+#pragma unroll
+        for (int s = 0; s < kHid / 16; ++s)
+            tc::mma_bf16(tbase, tc::make_desc(a0 + 256u * s, 128u, kHid / 8 * 128u),
+                         tc::make_desc(w0 + 2u * (kSliceCols / 8 * 128u) * s, kSliceCols / 8 * 128u, 128u), idesc, s > 0 ? 1u : 0u);
+        tc::mma_commit(&bar_m);
+    }
+    const int q4 = warp & 3, group = warp >> 2, row = 32 * q4 + lane, col0 = kSliceCols * slice + 16 * group;
+    const float *g1 = a.g1 + ((size_t)tile * kHid + col0) * 128 + row;
+    float x1[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x1[i] = __ldg(&g1[(size_t)i * 128]);
+    // the slice's sums of dz2 and GELU(z2) dout, under the MMAs
+#pragma unroll
+    for (int u = 0; u < kSliceCols / (kTrainThreads / 32); ++u) {
+        const int n = kSliceCols * slice + warp + u * (kTrainThreads / 32);
+        const float *g2 = a.g2 + ((size_t)tile * kHid + n) * 128, *h2 = a.h2 + ((size_t)tile * kHid + n) * 128;
+        const float s2 = column_sum(lane, [&](int b) { return dout_s[b] * w3s[n] * __ldg(&g2[b]); });
+        const float s3 = column_sum(lane, [&](int b) { return __ldg(&h2[b]) * dout_s[b]; });
+        if (lane == 0) { a.db2[tile * kHid + n] = s2; a.dw3[tile * kHid + n] = s3; }
+    }
+    const bool ok = train_wait(&bar_m, 0u);
+    if (ok) {
+        float *f = reinterpret_cast<float *>(sZ);    // [column of the slice][row]; the MMAs have read dz2
+        float x[16];
+        train_acc(tbase, q4, group, x);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            x[i] *= x1[i];
+            f[(16 * group + i) * 128 + row] = x[i];
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+            *reinterpret_cast<uint4 *>(a.dz1t + (size_t)tile * kTileH + tile_offset<kHid>((uint32_t)row, (uint32_t)(col0 + 8 * p))) =
+                make_uint4(pack_bf16x2(x[8 * p], x[8 * p + 1]), pack_bf16x2(x[8 * p + 2], x[8 * p + 3]),
+                           pack_bf16x2(x[8 * p + 4], x[8 * p + 5]), pack_bf16x2(x[8 * p + 6], x[8 * p + 7]));
+        __syncthreads();
+        for (int c = warp; c < kSliceCols; c += kTrainThreads / 32) {
+            const float s1 = column_sum(lane, [&](int row2) { return f[c * 128 + row2]; });
+            if (lane == 0) a.db1[tile * kHid + kSliceCols * slice + c] = s1;
+        }
+    }
+    train_end(ok, tbase, 64, a.err);
 }
 
-__global__ void step_advance_kernel(int64_t *step) { *step += 1; }
+// CTA (half, split): rows [128 half, ...) of dW2 = dz2^T h1 and dW1 = dz1^T x over the split's tiles. Both
+// operands are read transposed: a tile's rows are the MMA's K.
+constexpr int kWgradSmem = kTileH / 2 + kTileH + kTileH / 2 + kTileX;
+__global__ void __launch_bounds__(kTrainThreads) train_wgrad_kernel(TrainArgs a, int64_t *advance)
+{
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *sZ2 = sm, *sH = sZ2 + kTileH / 2, *sZ1 = sH + kTileH, *sX = sZ1 + kTileH / 2;
+    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = blockIdx.x, split = blockIdx.y;
+    train_begin(&bar_c, &bar_m, &tmem_base, 512);
+    const uint32_t tbase = tmem_base;
+    if (advance && tid == 0 && half == 0 && split == 0) *advance += 1;     // nobody reads it in this kernel
+    const int tiles = a.B / 128, per = (tiles + a.splits - 1) / a.splits;
+    const int t0 = split * per, t1 = min(tiles, t0 + per);
+    bool ok = true;
+    uint32_t phase = 0;
+    constexpr uint32_t kRowBlock = kHid / 8 * 128u, kHalfBlock = kRowBlock / 2;    // 8 rows of a tile, of half its columns
+    for (int t = t0; t < t1 && ok; ++t) {
+        if (tid == 0) {
+            tc::mbar_expect(&bar_c, kWgradSmem);
+            tc::bulk_load(sH, a.ht + (size_t)t * kTileH, kTileH, &bar_c);
+            tc::bulk_load(sX, a.xt + (size_t)t * kTileX, kTileX, &bar_c);
+            for (uint32_t b = 0; b < 16; ++b) {
+                const size_t src = (size_t)t * kTileH + b * kRowBlock + half * kHalfBlock;
+                tc::bulk_load(sZ2 + b * kHalfBlock, a.dz2t + src, kHalfBlock, &bar_c);
+                tc::bulk_load(sZ1 + b * kHalfBlock, a.dz1t + src, kHalfBlock, &bar_c);
+            }
+        }
+        ok = train_wait(&bar_c, phase);
+        if (!ok) break;
+        if (tid == 0) {
+            const uint32_t z2 = tc::smem_addr(sZ2), h = tc::smem_addr(sH), z1 = tc::smem_addr(sZ1), x = tc::smem_addr(sX);
+            const uint32_t id2 = tc::make_idesc_bf16(128, kHid, true, true), id1 = tc::make_idesc_bf16(128, kIn, true, true);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                const uint32_t acc = t > t0 || s > 0 ? 1u : 0u;
+                tc::mma_bf16(tbase, tc::make_desc(z2 + 2u * kHalfBlock * s, kHalfBlock, 128u),
+                             tc::make_desc(h + 2u * kRowBlock * s, kRowBlock, 128u), id2, acc);
+                tc::mma_bf16(tbase + kHid, tc::make_desc(z1 + 2u * kHalfBlock * s, kHalfBlock, 128u),
+                             tc::make_desc(x + 2u * (kIn / 8 * 128u) * s, kIn / 8 * 128u, 128u), id1, acc);
+            }
+            tc::mma_commit(&bar_m);
+        }
+        ok = train_wait(&bar_m, phase);
+        phase ^= 1u;
+    }
+    if (ok) {
+        // 320 accumulator columns in 20 groups of 16, five a warp of a lane quarter
+        const int q4 = warp & 3, n = 128 * half + 32 * q4 + lane;
+        for (int g = warp >> 2; g < (kHid + kIn) / 16; g += 4) {
+            float x[16];
+            train_acc(tbase, q4, g, x);
+            float *dst = g < kHid / 16 ? a.w2part + ((size_t)split * kHid + n) * kHid + 16 * g
+                                       : a.w1part + ((size_t)split * kHid + n) * kIn + 16 * (g - kHid / 16);
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4 *>(dst + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+        }
+    }
+    train_end(ok, tbase, 512, a.err);
+}
+
+// Adam of one training step: the moments and, for steps counted on the device, the bias corrections
+// c12[2 * step], c12[2 * step + 1] (the counter has been advanced).
+struct AdamArgs {
+    float *p, *m, *v;            // p null: gradients only
+    bf16 *W1b, *W2b;             // BF16 copies of the weights
+    float lr, beta1, beta2, eps;
+    const float *c12;
+    const int64_t *step;
+};
+
+// The gradient of every parameter: the splits' or tiles' sums in order; then Adam, if asked for.
+constexpr int kReduceThreads = 128;
+__global__ void __launch_bounds__(kReduceThreads) train_reduce_kernel(TrainArgs a, float *grad, float *loss, AdamArgs ad)
+{
+    const int i = blockIdx.x * kReduceThreads + threadIdx.x, tiles = a.B / 128;
+    if (i > kParams) return;
+    float s = 0.0f;
+    auto add = [&](const float *p, size_t stride, int n) {
+#pragma unroll 8
+        for (int k = 0; k < n; ++k) s += __ldg(p + (size_t)k * stride);
+    };
+    if (i < ob1) add(a.w1part + i, (size_t)kHid * kIn, a.splits);
+    else if (i < oW2) add(a.db1 + (i - ob1), kHid, tiles);
+    else if (i < ob2) add(a.w2part + (i - oW2), (size_t)kHid * kHid, a.splits);
+    else if (i < ow3) add(a.db2 + (i - ob2), kHid, tiles);
+    else if (i < ob3) add(a.dw3 + (i - ow3), kHid, tiles);
+    else add(a.dloss + (i - ob3), 2, 4 * tiles);
+    if (i == kParams) { *loss = s; return; }
+    grad[i] = s;
+    if (!ad.p) return;
+    const int64_t st = *ad.step - 1;
+    const float c1 = ad.c12[2 * st], c2 = ad.c12[2 * st + 1];
+    const float mi = ad.beta1 * ad.m[i] + (1.0f - ad.beta1) * s;
+    const float vi = ad.beta2 * ad.v[i] + (1.0f - ad.beta2) * s * s;
+    ad.m[i] = mi;
+    ad.v[i] = vi;
+    const float p = ad.p[i] - ad.lr * (mi / c1) / (sqrtf(vi / c2) + ad.eps);
+    ad.p[i] = p;
+    if (i < ob1) ad.W1b[i] = __float2bfloat16_rn(p);
+    else if (i >= oW2 && i < ob2) ad.W2b[i - oW2] = __float2bfloat16_rn(p);
+}
 
 __global__ void to_bf16_kernel(const float *__restrict__ src, bf16 *__restrict__ dst, int n)
 {
@@ -315,29 +663,9 @@ __global__ void to_bf16_kernel(const float *__restrict__ src, bf16 *__restrict__
     if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
 }
 
-__global__ void sum_kernel(const float *__restrict__ v, int n, float *__restrict__ dst)
-{
-    __shared__ float red[256];
-    float s = 0.0f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) dst[0] = red[0];
-}
-
 // ------------------------------------------------------------------------------------------
 // fused inference
 // ------------------------------------------------------------------------------------------
-// two floats as BF16 (round to nearest even) in one word, the first in the low half
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
-{
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&v);
-}
 
 // One tile is 128 queries. What bounds the kernel is the epilogues' arithmetic (65,536 GELUs a tile,
 // the FP32 pipe first; the MMAs take about 2,600 clocks), so everything else runs beside it on warps
@@ -719,40 +1047,40 @@ int refresh_bf16(aiwcrf_surrogate *s, cudaStream_t st)
     return e == cudaSuccess ? AIWCRF_OK : cuda_fail(e, "bf16 weight copies");
 }
 
-// scratch of one training batch
+// scratch of one training batch: the arrays of TrainArgs, gradients, Adam's moments
 struct Batch {
-    int B = 0;
-    bf16 *xin = nullptr, *h1 = nullptr, *dz2b = nullptr, *dz1b = nullptr;
-    float *yb = nullptr, *z1 = nullptr, *z2 = nullptr, *h2 = nullptr, *out = nullptr, *dout = nullptr;
-    float *loss_rows = nullptr, *dz2f = nullptr, *dh1 = nullptr, *dz1f = nullptr, *grad = nullptr, *part = nullptr;
-    float *m = nullptr, *v = nullptr, *loss = nullptr;
+    TrainArgs a = {};
+    float *grad = nullptr, *m = nullptr, *v = nullptr, *loss = nullptr;
     uint32_t *err = nullptr;
     void *block = nullptr;
     cudaStream_t s = nullptr;
     ~Batch() { if (block) cudaFreeAsync(block, s); }
-    int alloc(int B_, cudaStream_t st)
+    int alloc(int B, bool adam, cudaStream_t st)
     {
-        B = B_;
         s = st;
+        const size_t tiles = (size_t)B / 128, BH4 = 4 * (size_t)B * kHid;
+        a.B = B;
+        a.splits = (int)std::min<size_t>(tiles, kMaxSplits);
+        const int per = ((int)tiles + a.splits - 1) / a.splits;
+        a.splits = ((int)tiles + per - 1) / per;                     // none is empty
+        struct Part { void **p; size_t bytes; };
+        const size_t mv = adam ? 4 * (size_t)kParams : 0;
+        const Part parts[] = {
+            {(void **)&err, 4}, {(void **)&m, mv}, {(void **)&v, mv},                       // cleared below
+            {(void **)&a.xt, tiles * kTileX}, {(void **)&a.ht, tiles * kTileH}, {(void **)&a.dz2t, tiles * kTileH},
+            {(void **)&a.dz1t, tiles * kTileH}, {(void **)&a.yb, 4 * (size_t)B}, {(void **)&a.g1, BH4}, {(void **)&a.g2, BH4},
+            {(void **)&a.h2, BH4}, {(void **)&a.dots, 4 * (size_t)B * 32}, {(void **)&a.db1, 4 * tiles * kHid},
+            {(void **)&a.db2, 4 * tiles * kHid}, {(void **)&a.dw3, 4 * tiles * kHid}, {(void **)&a.dloss, 4 * tiles * 8},
+            {(void **)&a.w2part, 4 * (size_t)a.splits * kHid * kHid}, {(void **)&a.w1part, 4 * (size_t)a.splits * kHid * kIn},
+            {(void **)&grad, 4 * (size_t)kParams}, {(void **)&loss, 4}};
         auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-        const size_t BH = (size_t)B * kHid;
-        const size_t sizes[] = {up(2 * (size_t)B * kIn), up(2 * BH), up(2 * BH), up(2 * BH),     // xin h1 dz2b dz1b
-                                up(4 * (size_t)B), up(4 * BH), up(4 * BH), up(4 * BH), up(4 * (size_t)B),
-                                up(4 * (size_t)B), up(4 * (size_t)B), up(4 * BH), up(4 * BH), up(4 * BH),
-                                up(4 * (size_t)kParams), up(4 * (size_t)16 * kHid * kHid), up(4 * (size_t)kParams),
-                                up(4 * (size_t)kParams), up(4), up(4)};
         size_t tot = 0;
-        for (size_t b : sizes) tot += b;
+        for (const Part &p : parts) tot += up(p.bytes);
         if (cudaMallocAsync(&block, tot, st) != cudaSuccess) return fail(AIWCRF_E_OOM, "surrogate batch scratch");
         unsigned char *c = static_cast<unsigned char *>(block);
-        void **dst[] = {(void **)&xin, (void **)&h1, (void **)&dz2b, (void **)&dz1b, (void **)&yb, (void **)&z1,
-                        (void **)&z2, (void **)&h2, (void **)&out, (void **)&dout, (void **)&loss_rows,
-                        (void **)&dz2f, (void **)&dh1, (void **)&dz1f, (void **)&grad, (void **)&part, (void **)&m,
-                        (void **)&v, (void **)&loss, (void **)&err};
-        for (int i = 0; i < 20; ++i) { *dst[i] = c; c += sizes[i]; }
-        cudaMemsetAsync(m, 0, 4 * (size_t)kParams, st);
-        cudaMemsetAsync(v, 0, 4 * (size_t)kParams, st);
-        cudaMemsetAsync(err, 0, 4, st);
+        for (const Part &p : parts) { *p.p = c; c += up(p.bytes); }
+        a.err = err;
+        cudaMemsetAsync(block, 0, up(4) + 2 * up(mv), st);
         return AIWCRF_OK;
     }
 };
@@ -763,38 +1091,38 @@ struct Batch {
         if (e_ != cudaSuccess) return cuda_fail(e_, what);               \
     } while (0)
 
-// forward + backward of one batch; gradients land in bt.grad (parameter layout)
-int forward_backward(const aiwcrf_surrogate *sg, Batch &bt, const float *X, int64_t ld, const uint32_t *perm,
-                     int64_t r0, const float *y, cudaStream_t s, const int64_t *step = nullptr, int64_t spe = 1)
+// the training kernels' shared memory, once per device (a function's attributes last as its context)
+cudaError_t train_kernel_attributes(int device)
 {
-    const int B = bt.B, BH = B * kHid, ks = 16;
-    const Encoder e = encoder_of(sg);
-    const float *P = sg->d_param;
-    int rc;
-    encode_batch_kernel<<<(B * kIn + 255) / 256, 256, 0, s>>>(e, X, ld, perm, r0, B, y, bt.xin, bt.yb, step, spe);
-    if ((rc = tc_gemm(bt.xin, kIn, false, sg->d_W1b, kIn, false, bt.z1, B, kHid, kIn, 1, bt.part, bt.err, s))) return rc;
-    act1_kernel<<<(BH + 255) / 256, 256, 0, s>>>(bt.z1, P + ob1, bt.h1, BH);
-    if ((rc = tc_gemm(bt.h1, kHid, false, sg->d_W2b, kHid, false, bt.z2, B, kHid, kHid, 1, bt.part, bt.err, s))) return rc;
-    act2_out_kernel<<<(B + 7) / 8, 256, 0, s>>>(bt.z2, P + ob2, P + ow3, P + ob3, bt.h2, bt.yb, B, bt.out, bt.dout,
-                                                bt.loss_rows);
-    back2_kernel<<<(BH + 255) / 256, 256, 0, s>>>(bt.z2, P + ow3, bt.dout, bt.dz2b, bt.dz2f, BH);
-    colsum_part_kernel<<<dim3(kHid / 32, kColChunks), 256, 0, s>>>(bt.h2, B, bt.dout, bt.part);    // dw3
-    colsum_finish_kernel<<<1, kHid, 0, s>>>(bt.part, bt.grad + ow3);
-    sum_kernel<<<1, 256, 0, s>>>(bt.dout, B, bt.grad + ob3);                            // db3
-    colsum_part_kernel<<<dim3(kHid / 32, kColChunks), 256, 0, s>>>(bt.dz2f, B, nullptr, bt.part);  // db2
-    colsum_finish_kernel<<<1, kHid, 0, s>>>(bt.part, bt.grad + ob2);
-    sum_kernel<<<1, 256, 0, s>>>(bt.loss_rows, B, bt.loss);
-    count_launches(10);
-    SG_LAUNCH_CHECK("surrogate forward");
-    // dW2 = dz2^T h1 ; dh1 = dz2 W2 ; dz1 = dh1 GELU'(z1) ; dW1 = dz1^T xin
-    if ((rc = tc_gemm(bt.dz2b, kHid, true, bt.h1, kHid, true, bt.grad + oW2, kHid, kHid, B, ks, bt.part, bt.err, s))) return rc;
-    if ((rc = tc_gemm(bt.dz2b, kHid, false, sg->d_W2b, kHid, true, bt.dh1, B, kHid, kHid, 1, bt.part, bt.err, s))) return rc;
-    back1_kernel<<<(BH + 255) / 256, 256, 0, s>>>(bt.dh1, bt.z1, bt.dz1b, bt.dz1f, BH);
-    colsum_part_kernel<<<dim3(kHid / 32, kColChunks), 256, 0, s>>>(bt.dz1f, B, nullptr, bt.part);  // db1
-    colsum_finish_kernel<<<1, kHid, 0, s>>>(bt.part, bt.grad + ob1);
-    count_launches(3);
-    if ((rc = tc_gemm(bt.dz1b, kHid, true, bt.xin, kIn, true, bt.grad + oW1, kHid, kIn, B, ks, bt.part, bt.err, s))) return rc;
-    SG_LAUNCH_CHECK("surrogate backward");
+    static std::atomic<bool> done[64];
+    if (device >= 0 && device < 64 && done[device].load(std::memory_order_acquire)) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(train_layer2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLayer2Smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(train_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBackSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(train_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgradSmem);
+    if (e == cudaSuccess && device >= 0 && device < 64) done[device].store(true, std::memory_order_release);
+    return e;
+}
+
+// forward + backward of one batch; gradients land in bt.grad (parameter layout), the loss in bt.loss. With
+// Adam's arguments the parameters and their BF16 copies move too, and the device counter `step` advances.
+int forward_backward(const aiwcrf_surrogate *sg, Batch &bt, const float *X, int64_t ld, const uint32_t *perm,
+                     int64_t r0, const float *y, cudaStream_t s, int64_t *step = nullptr, int64_t spe = 1,
+                     const AdamArgs &adam = AdamArgs{})
+{
+    TrainArgs a = bt.a;
+    a.e = encoder_of(sg);
+    a.X = X; a.ld = ld; a.perm = perm; a.r0 = r0; a.yall = y; a.step = step; a.spe = spe;
+    a.P = sg->d_param; a.W1b = sg->d_W1b; a.W2b = sg->d_W2b;
+    const cudaError_t e = train_kernel_attributes(sg->device);
+    if (e != cudaSuccess) return cuda_fail(e, "surrogate training attributes");
+    const dim3 grid(kSlices, (unsigned)(a.B / 128));
+    train_layer1_kernel<<<grid, kTrainThreads, 0, s>>>(a);
+    train_layer2_kernel<<<grid, kTrainThreads, kLayer2Smem, s>>>(a);
+    train_back_kernel<<<grid, kTrainThreads, kBackSmem, s>>>(a);
+    train_wgrad_kernel<<<dim3(2, (unsigned)a.splits), kTrainThreads, kWgradSmem, s>>>(a, step);
+    train_reduce_kernel<<<(kParams + kReduceThreads) / kReduceThreads, kReduceThreads, 0, s>>>(a, bt.grad, bt.loss, adam);
+    count_launches(5);
+    SG_LAUNCH_CHECK("surrogate training step");
     return AIWCRF_OK;
 }
 
@@ -836,11 +1164,12 @@ struct TrainGraph {
 
 int check_err(const Batch &bt, cudaStream_t s)
 {
-    uint32_t h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, bt.err, 4, cudaMemcpyDeviceToHost, s);
+    uint32_t pageable = 0, *h = static_cast<uint32_t *>(pinned_scratch());      // an asynchronous read, if it can be had
+    if (!h) h = &pageable;
+    cudaError_t e = cudaMemcpyAsync(h, bt.err, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "surrogate");
-    if (h & kErrTimeout) return fail(AIWCRF_E_TIMEOUT, "a tensor-core wait gave up");
+    if (*h & kErrTimeout) return fail(AIWCRF_E_TIMEOUT, "a tensor-core wait gave up");
     return AIWCRF_OK;
 }
 
@@ -1050,7 +1379,7 @@ int aiwcrf_surrogate_fit(const aiwcrf_surrogate_params *p, const aiwcrf_forest *
     if ((rc = refresh_bf16(sg, s))) return rc;
 
     Batch bt;
-    if ((rc = bt.alloc(p->batch, s))) return rc;
+    if ((rc = bt.alloc(p->batch, true, s))) return rc;
     const int64_t steps_per_epoch = n / p->batch;
     uint32_t *d_perm = nullptr;
     if (cudaMallocAsync(&d_perm, 4 * (size_t)n, s) != cudaSuccess) return fail(AIWCRF_E_OOM, "surrogate permutation");
@@ -1081,14 +1410,9 @@ int aiwcrf_surrogate_fit(const aiwcrf_surrogate_params *p, const aiwcrf_forest *
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "surrogate step tables");
     if ((rc = tg.capture([&](cudaStream_t ts) {
-             int r = forward_backward(sg, bt, X, n, d_perm, 0, d_y, ts, d_step, steps_per_epoch);
-             if (r) return r;
-             adam_kernel<<<(kParams + 255) / 256, 256, 0, ts>>>(sg->d_param, bt.grad, bt.m, bt.v, kParams, p->lr,
-                                                                p->beta1, p->beta2, p->eps, 1.0f, 1.0f, d_c12, d_step);
-             if ((r = refresh_bf16(sg, ts))) return r;
-             step_advance_kernel<<<1, 1, 0, ts>>>(d_step);
-             const cudaError_t e2 = cudaGetLastError();
-             return e2 == cudaSuccess ? AIWCRF_OK : cuda_fail(e2, "surrogate step launches");
+             return forward_backward(sg, bt, X, n, d_perm, 0, d_y, ts, d_step, steps_per_epoch,
+                                     AdamArgs{sg->d_param, bt.m, bt.v, sg->d_W1b, sg->d_W2b, p->lr, p->beta1, p->beta2,
+                                              p->eps, d_c12, d_step});
          })))
         return rc;
     int64_t t = 0;
@@ -1144,7 +1468,18 @@ int aiwcrf_surrogate_grad(const aiwcrf_surrogate *sg, const float *X, const floa
     cudaStream_t s = (cudaStream_t)cuda_stream;
     Batch bt;
     int rc;
-    if ((rc = bt.alloc(n, s))) return rc;
+    if ((rc = bt.alloc(n, false, s))) return rc;
+    // the last kernel writes to the caller's arrays where they are this device's
+    cudaPointerAttributes ag, al;
+    if (cudaPointerGetAttributes(&ag, grad) == cudaSuccess && cudaPointerGetAttributes(&al, loss) == cudaSuccess &&
+        ag.type == cudaMemoryTypeDevice && al.type == cudaMemoryTypeDevice && ag.device == sg->device &&
+        al.device == sg->device) {
+        bt.grad = grad;
+        bt.loss = loss;
+        if ((rc = forward_backward(sg, bt, X, n, nullptr, 0, y, s))) return rc;
+        return check_err(bt, s);
+    }
+    cudaGetLastError();
     if ((rc = forward_backward(sg, bt, X, n, nullptr, 0, y, s))) return rc;
     cudaError_t e = cudaMemcpyAsync(grad, bt.grad, 4 * (size_t)kParams, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(loss, bt.loss, 4, cudaMemcpyDeviceToDevice, s);
