@@ -714,10 +714,10 @@ struct LevelArgs {
     uint32_t *tile_splits;      // per tile of kScanTile nodes: nodes that split (zero on entry)
     const uint32_t *depth_ptr;  // when set, the depth is read here (a graph replays one level body)
     uint32_t node_cap;          // entries of the node table (bounds checks of debug builds)
-    // presorted lists (the list kernel): per feature f, per tree t, a node's segment of
+    // presorted lists (the list kernels): per feature f, per tree t, a node's segment of
     // lists_in[f * list_stride + t * row_cap + ...] holds the positions of its entries within its
-    // segment of rows_in, in increasing rank of f; newpos[t * row_cap + start + p] receives the
-    // position in rows_out of the entry at position p when the node splits
+    // segment of rows_in, in increasing rank of f (list words, see kListBreak); newpos[t * row_cap +
+    // start + p]: scratch of nodes too long for the split's shared memory
     const uint32_t *lists_in = nullptr;
     uint32_t *lists_out = nullptr;
     int64_t list_stride = 0;
@@ -1008,6 +1008,24 @@ __global__ void __launch_bounds__(1024) rep_order_kernel(const uint32_t *__restr
     }
 }
 
+// A list word: the entry's position within its node's segment, and in the top bit whether its rank
+// differs from that of the word before it in the node's segment (a break; always set on the first).
+// A candidate is the last word of a run of equal ranks, that is one before a break: the search needs
+// no rank but the winner's.
+constexpr uint32_t kListBreak = 0x80000000u, kListPos = 0x7FFFFFFFu;
+
+// marks the representatives whose rank differs from the one before them in the column's order
+template <typename RT>
+__global__ void rep_break_kernel(uint32_t *__restrict__ ordG, uint32_t G, const RT *__restrict__ Rr, int F)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int f = blockIdx.y;
+    if (i >= G) return;
+    uint32_t *o = ordG + (size_t)f * (size_t)G;
+    const uint32_t row = o[i] & kListPos;
+    if (i == 0 || Rr[(size_t)row * F + f] != Rr[(size_t)(o[i - 1] & kListPos) * F + f]) o[i] = row | kListBreak;
+}
+
 // every tree's entry position (plus one) by representative row ([T][N], zero elsewhere)
 __global__ void list_pos_kernel(const Entry *__restrict__ rows, int64_t row_cap, const NodeRec *__restrict__ root,
                                 int64_t N, uint32_t *__restrict__ P)
@@ -1019,24 +1037,57 @@ __global__ void list_pos_kernel(const Entry *__restrict__ rows, int64_t row_cap,
     P[(size_t)t * (size_t)N + AIWCRF_IDX(e.row, (uint32_t)N, kBoundRow)] = (uint32_t)i + 1u;
 }
 
-// CTA (tree, feature): the positions of the tree's entries in increasing rank of the feature
+// CTA (tree, feature): the tree's list of a feature, 4,096 representatives a step (each thread four
+// gathers in flight; 1,024 a step with one was 11.6 ms for 500 trees of 111,000 rows)
+constexpr int kBuildPer = 4;
 __global__ void __launch_bounds__(1024) list_build_kernel(const uint32_t *__restrict__ ordG, uint32_t G,
                                                           const uint32_t *__restrict__ P, int64_t N, int64_t row_cap,
                                                           int64_t stride, uint32_t *__restrict__ lists)
 {
     __shared__ uint32_t warp_tmp[32];
-    const int64_t t = blockIdx.x;
-    const uint32_t *src = ordG + (size_t)blockIdx.y * (size_t)G;
+    __shared__ uint32_t s_pos[1024 * kBuildPer], s_run[1024 * kBuildPer];
+    __shared__ uint32_t s_last;                     // the run of the last kept word
+    const int64_t t = blockIdx.y;                   // a tree's features side by side: its P stays in L2
+    const int tid = threadIdx.x;
+    const uint32_t *src = ordG + (size_t)blockIdx.x * (size_t)G;
     const uint32_t *Pt = P + (size_t)t * (size_t)N;
-    uint32_t *dst = lists + (size_t)blockIdx.y * (size_t)stride + (size_t)t * (size_t)row_cap;
-    uint32_t running = 0;
-    for (uint32_t b0 = 0; b0 < G; b0 += 1024) {
-        const uint32_t i = b0 + threadIdx.x;
-        const uint32_t pos = i < G ? Pt[src[i]] : 0u;
+    uint32_t *dst = lists + (size_t)blockIdx.x * (size_t)stride + (size_t)t * (size_t)row_cap;
+    uint32_t running = 0, runs = 0;                 // words kept, breaks seen
+    if (tid == 0) s_last = 0xFFFFFFFFu;
+    for (uint32_t b0 = 0; b0 < G; b0 += 1024 * kBuildPer) {
+        uint32_t o[kBuildPer], pos[kBuildPer];
+#pragma unroll
+        for (int u = 0; u < kBuildPer; ++u) {
+            const uint32_t i = b0 + (uint32_t)(kBuildPer * tid + u);
+            o[u] = i < G ? __ldg(&src[i]) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kBuildPer; ++u) {
+            const uint32_t i = b0 + (uint32_t)(kBuildPer * tid + u);
+            pos[u] = i < G ? __ldg(&Pt[o[u] & kListPos]) : 0u;
+        }
+        uint32_t mine = 0u;                         // kept words, breaks in the upper half
+#pragma unroll
+        for (int u = 0; u < kBuildPer; ++u) mine += (pos[u] ? 1u : 0u) + (o[u] >> 31 << 16);
         uint32_t tot;
-        const uint32_t incl = block_incl_scan(pos > 0u ? 1u : 0u, warp_tmp, tot);
-        if (pos > 0u && (int64_t)(running + incl - 1u) < row_cap) dst[running + incl - 1u] = pos - 1u;
-        running += tot;
+        const uint32_t excl = block_incl_scan(mine, warp_tmp, tot) - mine;
+        uint32_t at = excl & 0xFFFFu, run = runs + (excl >> 16);
+#pragma unroll
+        for (int u = 0; u < kBuildPer; ++u) {
+            run += o[u] >> 31;
+            if (pos[u]) { s_pos[at] = pos[u] - 1u; s_run[at] = run; ++at; }
+        }
+        const uint32_t kept = tot & 0xFFFFu, before = s_last;
+        __syncthreads();
+        for (uint32_t i = (uint32_t)tid; i < kept; i += 1024u) {
+            const uint32_t prev = i ? s_run[i - 1] : before;
+            if ((int64_t)(running + i) < row_cap) dst[running + i] = s_pos[i] | (s_run[i] != prev ? kListBreak : 0u);
+        }
+        __syncthreads();
+        if (tid == 0 && kept) s_last = s_run[kept - 1];
+        running += kept;
+        runs += tot >> 16;
+        __syncthreads();
     }
 }
 
@@ -1053,204 +1104,533 @@ inline int big_bin_cap(int mtry, int F, uint32_t max_card)
     return (int)std::min<int64_t>(4096, (need + 31) & ~(int64_t)31);
 }
 
-// A big node's split search from the presorted lists. The warps take the tried features in
-// turn; a warp scans (w, w*y) along the node's segment of its feature's list (entry positions,
-// read from the node's own entry segment), 32 entries a step and kListIlp steps' loads in
-// flight, so the left sums of every threshold come without block barriers. A candidate sits at
-// the last entry of each run of equal ranks but the last run.
-// With AIWCRF_LIST_STAGE > 0, a node of at most that many entries is staged in shared memory
-// first (its entries, then per warp the ranks of the feature it scans, gathered in entry order
-// with no dependence on the list), so that each scan step reads one list position from HBM and
-// the rest from shared memory. Off by default: on the per-row fit the staging passes and the
-// smaller L1 cost more than the dependent loads they remove.
-constexpr int kListIlp = 4;
-#ifndef AIWCRF_LIST_STAGE
-#define AIWCRF_LIST_STAGE 0            // entries staged per node (0: none; 768 and 1536 were slower)
-#endif
-constexpr int kListStage = AIWCRF_LIST_STAGE;
+// A depth's big nodes with presorted lists, in three steps. What bounds them is dependent loads (word ->
+// entry) and issue slots, so a node is a warp's work, without block barriers, unless it is large:
+//  - list_draw_kernel, a warp per node: its tried features; nodes of more than kWarpNode entries are
+//    listed for the CTA forms of the other two.
+//  - list_search_kernel, a warp per (node, tried feature), or a CTA above kCtaSearch entries: consecutive
+//    items share a node, so its entries (1.1 MB at a root of 70,000) are in L2 while its features are
+//    searched. With a warp per item at the root, 500 trees' entries were in use at once, 7.7 ms of that
+//    depth; a CTA per item takes 2.2.
+//  - list_split_kernel, a warp per node, or CTAs: the best of its features' candidates, the entries' stable
+//    partition and that of every feature's list. Which entries go left is a bit set, filled from the
+//    winning feature's list, whose first lenL words are the left side; a bit and a prefix count give an
+//    entry's side and place, for the entries and in every list.
+// 500 trees of 111,000 rows with 32 features of as many values, 10 tried (666 million entries searched):
+// draw 1.7 ms, search 44, split 66, beside 50 of level_small_kernel. One CTA per node, four warps over its
+// features with a rank gathered beside each entry, and a second kernel over all lists took 128 and 125 ms;
+// the lists are 134 GB of reads and writes, 20 ms of memory time.
+constexpr int kListWarps = 8;            // of a CTA of the warp-per-item kernels
+constexpr int kListThreads = 32 * kListWarps;
+constexpr int kListCtasPerSm = 4;
+constexpr uint32_t kWarpNode = 1024;     // entries of a node that one warp splits: 32 bits a lane
+constexpr uint32_t kCtaSearch = 4096;    // entries of a node above which a CTA searches a feature
+constexpr uint32_t kCtaNodeWords = 4096; // bit-set words of the CTA form in shared memory (131,072 entries)
 
-template <int NW>
-constexpr int list_stage_bytes() { return kListStage > 0 ? kListStage * 16 + NW * kListStage * 4 : 0; }
+struct alignas(16) ListNode {     // what a search needs of a node
+    int64_t S;
+    int64_t mean;                 // S / n, towards zero
+    size_t at;                    // of its entries and list words
+    uint32_t len, n;              // len 0: the node stops
+    float rest;                   // (S - n * mean) / n
+    uint32_t pad;
+};
+static_assert(sizeof(ListNode) == 48, "ListNode");
 
-template <typename RT, int NW>
-__device__ __forceinline__ Cand list_search(const LevelArgs &a, const NodeRec &nd, const int *feats, int m,
-                                            unsigned char *stage)
+struct ListArgs {
+    ListNode *node;               // per slot of the depth's list
+    uint8_t *feat;                // [slot][tried feature]
+    Cand *cand;                   // [slot][tried feature]: r is the position in the list
+    int m;                        // tried features of a node
+    int32_t *huge;                // nodes for the CTA form
+    uint32_t *n_huge;             // their number, by depth parity
+};
+
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_draw_kernel(LevelArgs a, ListArgs l)
 {
-    const RT *__restrict__ Rr = static_cast<const RT *>(a.Rr);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t tb = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
-    const Entry *__restrict__ rin = a.rows_in + tb;
-    const bool staged = kListStage > 0 && nd.len <= (uint32_t)kListStage;   // block-uniform
-    long long *s_wy = reinterpret_cast<long long *>(stage);
-    uint32_t *s_w = reinterpret_cast<uint32_t *>(stage + 8 * kListStage);
-    uint32_t *s_row = s_w + kListStage;
-    uint32_t *s_rk = s_row + kListStage + warp * kListStage;     // this warp's ranks
-    if (staged) {
-        for (uint32_t q = threadIdx.x; q < nd.len; q += 32u * NW) {
-            const Entry e = load_entry(rin + q);
-            s_wy[q] = (long long)e.wy;
-            s_w[q] = e.w;
-            s_row[q] = AIWCRF_IDX(e.row, (uint32_t)a.N, kBoundRow);
+    const int lane = threadIdx.x & 31, parity = level_depth(a) & 1;
+    const uint32_t list_n = *a.list_n, step = gridDim.x * kListWarps;
+    if (blockIdx.x == 0 && threadIdx.x == 0) l.n_huge[parity ^ 1] = 0u;      // the depth before is done with it
+    for (uint32_t k = blockIdx.x * kListWarps + (threadIdx.x >> 5); k < list_n; k += step) {
+        const int j = AIWCRF_IDX(a.list[k], a.node_cap, kBoundNode);
+        const NodeRec nd = a.nodes[j];
+        uint32_t mask[4] = {0u, 0u, 0u, 0u};
+        if (node_stops(a, nd)) {
+            if (lane == 0) write_leaf(a.res, j, -2, 0);
+        } else {
+            warp_mtry(a, a.tree_rng[nd.tree], nd.idx, mask);
+            if (lane == 0 && nd.len > kWarpNode) l.huge[atomicAdd(&l.n_huge[parity], 1u)] = (int32_t)k;
         }
-        __syncthreads();
+        for (int q = lane; q < l.m; q += 32) l.feat[(size_t)k * (size_t)l.m + q] = (uint8_t)nth_feature(mask, q);
+        if (lane == 0) {
+            ListNode o;
+            o.S = nd.S;
+            o.mean = nd.S / (int64_t)nd.n;
+            o.at = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
+            o.len = node_stops(a, nd) ? 0u : nd.len;
+            o.n = nd.n;
+            o.pad = 0u;
+            o.rest = (float)(int32_t)(nd.S - o.mean * (int64_t)nd.n) / (float)nd.n;
+            l.node[k] = o;
+        }
     }
+}
+
+// A step takes 32 * per words, per = 4, 2 or 1 by what is left of the node (a node of 150 entries is 128 +
+// 32 words, not 256); lane l holds words per * l .. per * l + per - 1, so one warp scan of (w, w*y) serves
+// them all. Exact candidates (a 128-bit delta each) are formed only where an estimate can still win: with
+// c = SL - nL * mean (64 bits, exact), |delta| / n = |c - nL * rest|, so |c - nL * rest| / sqrt(nL * nR)
+// orders the candidates. Its error is below 2^-20 (|c| + nL) / sqrt(nL * nR): the conversions of c and
+// rest and the subtraction give 2^-22, rsqrtf and its argument 2^-21 (n < 2^24: nL and nR are exact). A
+// candidate whose estimate plus that (twice it, 2^-19) is below another's estimate less that loses; the
+// warp keeps the largest such bound. Every other one, so every one of the largest gain, is compared as
+// exactly as before.
+constexpr int kListIlp = 4;
+struct ListTotals {               // of a step's warps, by step parity
+    uint32_t w[2][kListWarps];
+    long long s[2][kListWarps];
+};
+
+// NW warps search feature f of a node: their best candidate, warp by warp
+template <int NW>
+__device__ __forceinline__ Cand list_search(const LevelArgs &a, const ListNode &nd, int f, int warp, ListTotals *tot)
+{
+    const int lane = threadIdx.x & 31;
+    const Entry *__restrict__ rin = a.rows_in + nd.at;
+    const uint32_t *__restrict__ L = a.lists_in + (size_t)f * (size_t)a.list_stride + nd.at;
+    const float nf = (float)nd.n;
     Cand best = cand_none();
-    for (int k = warp; k < m; k += NW) {
-        const int f = feats[k];
-        const uint32_t *__restrict__ L = a.lists_in + (size_t)f * (size_t)a.list_stride + tb;
-        uint32_t cw = 0u;                       // sums of the earlier steps (warp-uniform)
-        long long cs = 0ll;
-        if (staged) {
-            __syncwarp();                       // the previous feature's ranks are no longer read
-#pragma unroll 8
-            for (uint32_t q = (uint32_t)lane; q < nd.len; q += 32u) s_rk[q] = (uint32_t)__ldg(&Rr[(size_t)s_row[q] * (size_t)a.F + f]);
-            __syncwarp();
+    float floor_h = 0.0f;                                      // no candidate below it wins (warp-uniform)
+    uint32_t cw = 0u;                                          // sums of the earlier steps (uniform)
+    long long cs = 0ll;
+    uint32_t v[kListIlp], nv[kListIlp];
+    auto words = [&](uint32_t b0) { return NW > 1 || b0 + 64u < nd.len ? 4 : b0 + 32u < nd.len ? 2 : 1; };
+    auto load = [&](uint32_t b0, int per, uint32_t (&x)[kListIlp]) {
+#pragma unroll
+        for (int u = 0; u < kListIlp; ++u) {
+            const uint32_t i = b0 + (uint32_t)(per * (32 * warp + lane) + u);
+            x[u] = u < per && i < nd.len ? __ldg(&L[i]) : 0u;
         }
-        for (uint32_t b0 = 0; b0 < nd.len; b0 += 32u * kListIlp) {
-            uint32_t w[kListIlp], rank[kListIlp], nrank[kListIlp];
-            long long wy[kListIlp];
+    };
+    int per = words(0u), parity = 0;
+    load(0u, per, v);
+    for (uint32_t b0 = 0; b0 < nd.len; parity ^= 1) {
+        const uint32_t i0 = b0 + (uint32_t)(per * (32 * warp + lane)), b1 = b0 + (uint32_t)(32 * NW * per);
+        uint32_t w[kListIlp];
+        long long wy[kListIlp];
+#pragma unroll
+        for (int u = 0; u < kListIlp; ++u) {
+            w[u] = 0u;
+            wy[u] = 0ll;
+            if (u < per && i0 + (uint32_t)u < nd.len) {
+                const Entry e = load_entry(rin + AIWCRF_IDX(v[u] & kListPos, nd.len, kBoundOut));
+                w[u] = e.w;
+                wy[u] = (long long)e.wy;
+            }
+        }
+        const int nper = words(b1);
+        uint32_t after;                                        // the word behind the warp's
+        if constexpr (NW > 1) {
+            after = lane == 31 && i0 + kListIlp < nd.len ? __ldg(&L[i0 + kListIlp]) : 0u;
+            load(b1, nper, nv);                                // the next step's words, beside these entries
+        } else {
+            load(b1, nper, nv);
+            after = __shfl_sync(kFull, nv[0], 0);
+        }
+        uint32_t next = __shfl_down_sync(kFull, v[0], 1);
+        if (lane == 31) next = after;
+        uint32_t ends = 0u;                                    // bit u: a break follows word u
+#pragma unroll
+        for (int u = 0; u < kListIlp; ++u) {
+            const uint32_t x = u + 1 < per ? v[u + 1 < kListIlp ? u + 1 : 0] : next;
+            if (u < per && i0 + (uint32_t)u + 1u < nd.len && (x & kListBreak)) ends |= 1u << u;
+        }
+        uint32_t lw = 0u;
+        long long ls = 0ll;
+#pragma unroll
+        for (int u = 0; u < kListIlp; ++u) { lw += w[u]; ls += wy[u]; }
+        uint32_t pw = lw;
+        long long ps = ls;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t tw = __shfl_up_sync(kFull, pw, o);
+            const long long ts = __shfl_up_sync(kFull, ps, o);
+            if (lane >= o) { pw += tw; ps += ts; }
+        }
+        uint32_t w0 = cw + pw - lw;                            // before this lane's words
+        long long s0 = cs + ps - ls;
+        if constexpr (NW > 1) {
+            if (lane == 31) { tot->w[parity][warp] = pw; tot->s[parity][warp] = ps; }
+            __syncthreads();                                   // a parity is written again two barriers on
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const uint32_t tw = tot->w[parity][i];
+                const long long ts = tot->s[parity][i];
+                if (i < warp) { w0 += tw; s0 += ts; }
+                cw += tw;
+                cs += ts;
+            }
+        } else {
+            cw += __shfl_sync(kFull, pw, 31);
+            cs += __shfl_sync(kFull, ps, 31);
+        }
+        float hi[kListIlp], lo = 0.0f;
+        {
+            uint32_t nL = w0;
+            long long SL = s0;
 #pragma unroll
             for (int u = 0; u < kListIlp; ++u) {
-                const uint32_t i = b0 + 32u * u + (uint32_t)lane;
-                w[u] = 0u; wy[u] = 0ll; rank[u] = 0u; nrank[u] = 0u;
-                if (staged) {
-                    if (i < nd.len) {
-                        const uint32_t q = AIWCRF_IDX(__ldg(&L[i]), nd.len, kBoundOut);
-                        w[u] = s_w[q];
-                        wy[u] = s_wy[q];
-                        rank[u] = s_rk[q];
-                    }
-                    if (lane == 31 && i + 1u < nd.len) nrank[u] = s_rk[AIWCRF_IDX(__ldg(&L[i + 1u]), nd.len, kBoundOut)];
-                } else if (i < nd.len) {
-                    const Entry e = load_entry(rin + AIWCRF_IDX(__ldg(&L[i]), nd.len, kBoundOut));
-                    w[u] = e.w;
-                    wy[u] = (long long)e.wy;
-                    rank[u] = (uint32_t)__ldg(&Rr[(size_t)AIWCRF_IDX(e.row, (uint32_t)a.N, kBoundRow) * (size_t)a.F + f]);
-                }
-                // the rank after the warp's last entry of this step
-                if (!staged && lane == 31 && i + 1u < nd.len) {
-                    const uint32_t row2 = __ldg(&rin[AIWCRF_IDX(__ldg(&L[i + 1u]), nd.len, kBoundOut)].row);
-                    nrank[u] = (uint32_t)__ldg(&Rr[(size_t)AIWCRF_IDX(row2, (uint32_t)a.N, kBoundRow) * (size_t)a.F + f]);
+                hi[u] = -1.0f;
+                if (u >= per) continue;
+                nL += w[u];
+                SL += wy[u];
+                const float c = __ll2float_rn(SL - (long long)nL * nd.mean), fl = (float)nL;
+                const float rs = rsqrtf(fl * (nf - fl));
+                const float h = fabsf(fmaf(-fl, nd.rest, c)) * rs, e = (fabsf(c) + fl) * rs * 0x1p-19f;
+                if (ends & (1u << u)) {
+                    hi[u] = h + e;
+                    lo = fmaxf(lo, h - e);
                 }
             }
+        }
+        floor_h = fmaxf(floor_h, __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(lo))));
+        {
+            uint32_t nL = w0;
+            long long SL = s0;
 #pragma unroll
             for (int u = 0; u < kListIlp; ++u) {
-                const uint32_t i = b0 + 32u * u + (uint32_t)lane;
-                const uint32_t nr_lane = __shfl_down_sync(kFull, rank[u], 1);
-                const uint32_t nr = lane == 31 ? nrank[u] : nr_lane;
-                uint32_t pw = w[u];
-                long long ps = wy[u];
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t tw = __shfl_up_sync(kFull, pw, o);
-                    const long long tsum = __shfl_up_sync(kFull, ps, o);
-                    if (lane >= o) { pw += tw; ps += tsum; }
-                }
-                if (i + 1u < nd.len && nr != rank[u]) {        // the last entry of a rank's run
-                    const uint32_t nL = cw + pw;
-                    const long long SL = cs + ps;
+                nL += w[u];
+                SL += wy[u];
+                if (hi[u] >= floor_h) {
                     const i128_t delta = cand_delta(nd.n, nd.S, nL, SL);
                     if (delta != 0) {
                         Cand cd;
                         cd.h = cand_h(delta, nd.n, nL);
-                        cd.f = f; cd.r = rank[u]; cd.nL = nL; cd.SL = SL;
+                        cd.f = f; cd.r = i0 + (uint32_t)u; cd.nL = nL; cd.SL = SL;
                         if (cand_better(cd, best, nd.n, nd.S)) best = cd;
                     }
                 }
-                cw += __shfl_sync(kFull, pw, 31);
-                cs += __shfl_sync(kFull, ps, 31);
             }
         }
+        b0 = b1;
+        per = nper;
+#pragma unroll
+        for (int u = 0; u < kListIlp; ++u) v[u] = nv[u];
     }
-    return best;
+    return warp_best(best, nd.n, nd.S);
 }
 
-// Stable partition of a split big node's segment of one feature's list, by one warp: ballots
-// give each entry its place, so the children's segments stay in rank order. An entry's new
-// position, written by the entry partition, also says its side; the list receives the positions
-// within the child's own segment.
-constexpr int kPartIlp = 8;
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_kernel(LevelArgs a, ListArgs l)
+{
+    const uint32_t list_n = *a.list_n, m = (uint32_t)l.m, step = gridDim.x * kListWarps;
+    const uint32_t first = blockIdx.x * kListWarps + (threadIdx.x >> 5), dk = step / m, dq = step - dk * m;
+    uint32_t k = first / m, q = first - k * m;
+    while (k < list_n) {
+        const ListNode nd = l.node[k];
+        if (nd.len != 0u && nd.len <= kCtaSearch) {
+            const size_t at = (size_t)k * m + q;
+            const Cand c = list_search<1>(a, nd, l.feat[at], 0, nullptr);
+            if ((threadIdx.x & 31) == 0) l.cand[at] = c;
+        }
+        k += dk;
+        q += dq;
+        if (q >= m) { q -= m; ++k; }
+    }
+}
 
-// needL / needR: whether the left / right child will search its lists (the other side's entries
-// are not written: a child of at most 32 entries is searched from the entries, a stopping one not
-// at all).
-__device__ __forceinline__ void list_partition_feature(const LevelArgs &a, const NodeRec &nd, int f, uint32_t lenL,
-                                                       const uint32_t *np, bool needL, bool needR)
+// The same by a CTA per (node, tried feature), for nodes of more than kCtaSearch entries: 1,024 words a step.
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_huge_kernel(LevelArgs a, ListArgs l)
+{
+    __shared__ ListTotals tot;
+    __shared__ Cand cands[kListWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t n = l.n_huge[level_depth(a) & 1], m = (uint32_t)l.m;
+    for (uint32_t it = blockIdx.x; it < n * m; it += gridDim.x) {
+        const uint32_t k = (uint32_t)l.huge[it / m];
+        const ListNode nd = l.node[k];
+        if (nd.len <= kCtaSearch) continue;                        // block-uniform
+        const size_t at = (size_t)k * m + it % m;
+        const Cand c = list_search<kListWarps>(a, nd, l.feat[at], warp, &tot);
+        if (lane == 0) cands[warp] = c;
+        __syncthreads();
+        if (warp == 0) {
+            const Cand b = warp_best(lane < kListWarps ? cands[lane] : cand_none(), nd.n, nd.S);
+            if (lane == 0) l.cand[at] = b;
+        }
+        __syncthreads();
+    }
+}
+
+// The partition of the lists of features f0, f0 + df, ... < F of a node by one warp. place(p) says for the
+// entry at position p whether it goes left (top bit) and its position within its child. Ballots give each
+// word its place, so the children's segments stay in rank order. A side's word is a break if there was one
+// since the side's word before it: with the other side's lanes as ones, adding the breaks among them
+// carries each into the side's next word (and out of the top into the next step). needL / needR: whether
+// the child will search its lists (otherwise its words are not written: a child of at most 32 entries is
+// searched from the entries, a stopping one not at all). The next words, of this feature or the next, are
+// on their way while these are placed.
+constexpr int kPartIlp = 4;
+template <typename Place>
+__device__ __forceinline__ void list_partition(const LevelArgs &a, const NodeRec &nd, int f0, int df, uint32_t lenL,
+                                               bool needL, bool needR, const Place &place)
 {
     const int lane = threadIdx.x & 31;
     const uint32_t lt = lanemask_lt();
     const size_t tb = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
-    const uint32_t *__restrict__ Li = a.lists_in + (size_t)f * (size_t)a.list_stride + tb;
-    uint32_t *__restrict__ Lo = a.lists_out + (size_t)f * (size_t)a.list_stride + tb;
-    uint32_t rl = 0u, rr = 0u;
-    for (uint32_t b0 = 0; b0 < nd.len; b0 += 32u * kPartIlp) {
-        uint32_t p[kPartIlp], d[kPartIlp];
+    uint32_t p[kPartIlp], pn[kPartIlp];
+    auto load = [&](const uint32_t *__restrict__ L, uint32_t b0, uint32_t (&x)[kPartIlp]) {
 #pragma unroll
         for (int u = 0; u < kPartIlp; ++u) {
             const uint32_t i = b0 + 32u * u + (uint32_t)lane;
-            p[u] = i < nd.len ? AIWCRF_IDX(__ldg(&Li[i]), nd.len, kBoundOut) : 0u;
+            x[u] = i < nd.len ? __ldg(&L[i]) : 0u;
         }
+    };
+    if (f0 >= a.F) return;
+    const uint32_t *__restrict__ Li = a.lists_in + (size_t)f0 * (size_t)a.list_stride + tb;
+    uint32_t *__restrict__ Lo = a.lists_out + (size_t)f0 * (size_t)a.list_stride + tb;
+    const size_t stride = (size_t)df * (size_t)a.list_stride;
+    load(Li, 0u, p);
+    for (int f = f0; f < a.F; f += df, Lo += stride) {
+        uint32_t rl = 0u, cl = 1u, cr = 1u;        // words left so far; a break pending for either side (or no word yet)
+        for (uint32_t b0 = 0; b0 < nd.len; b0 += 32u * kPartIlp) {
+            if (b0 + 32u * kPartIlp < nd.len) load(Li, b0 + 32u * kPartIlp, pn);
+            else if (f + df < a.F) { Li += stride; load(Li, 0u, pn); }
+            uint32_t d[kPartIlp];
 #pragma unroll
-        for (int u = 0; u < kPartIlp; ++u) {
-            const uint32_t i = b0 + 32u * u + (uint32_t)lane;
-            d[u] = i < nd.len ? AIWCRF_IDX(np[p[u]], nd.len, kBoundOut) : 0u;
-        }
+            for (int u = 0; u < kPartIlp; ++u) d[u] = place(AIWCRF_IDX(p[u] & kListPos, nd.len, kBoundOut));
 #pragma unroll
-        for (int u = 0; u < kPartIlp; ++u) {
-            const uint32_t s0 = b0 + 32u * u;
-            if (s0 >= nd.len) break;                                // warp-uniform
-            const uint32_t i = s0 + (uint32_t)lane;
-            const bool left = i < nd.len && d[u] < lenL;
-            const uint32_t bal = __ballot_sync(kFull, left);
-            const uint32_t before = (uint32_t)__popc(bal & lt);
-            if (i < nd.len && (left ? needL : needR))
-                Lo[AIWCRF_IDX(left ? rl + before : lenL + rr + ((uint32_t)lane - before), nd.len, kBoundOut)] =
-                    left ? d[u] : d[u] - lenL;
-            const uint32_t nl = (uint32_t)__popc(bal);
-            rl += nl;
-            rr += min(32u, nd.len - s0) - nl;
+            for (int u = 0; u < kPartIlp; ++u) {
+                const uint32_t s0 = b0 + 32u * u, i = s0 + (uint32_t)lane;
+                if (s0 >= nd.len) break;                            // warp-uniform
+                const bool valid = i < nd.len, left = valid && (d[u] & kListBreak);
+                const uint32_t bl = __ballot_sync(kFull, left), br = __ballot_sync(kFull, valid) & ~bl;
+                const uint32_t bk = __ballot_sync(kFull, valid && (p[u] & kListBreak));
+                const uint64_t sl = (uint64_t)(~bl) + (bk & ~bl) + cl, sr = (uint64_t)(~br) + (bk & ~br) + cr;
+                cl = (uint32_t)(sl >> 32);
+                cr = (uint32_t)(sr >> 32);
+                const uint32_t brk = ((left ? (uint32_t)sl : (uint32_t)sr) | bk) >> lane << 31;
+                const uint32_t nl = rl + (uint32_t)__popc(bl & lt);
+                if (valid && (left ? needL : needR))
+                    Lo[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)] = (d[u] & kListPos) | brk;
+                rl += (uint32_t)__popc(bl);
+            }
+#pragma unroll
+            for (int u = 0; u < kPartIlp; ++u) p[u] = pn[u];
         }
     }
 }
 
-// After the list kernel of a depth: one CTA per split big node, its warps taking the features
-// in turn. A node of at most kPartStage entries first copies its new positions into shared
-// memory, so each step's second load is a shared-memory read.
-constexpr int kPartThreads = 256;
-constexpr int kPartCtasPerSm = 4;
-constexpr int kPartStage = 8192;
-__global__ void __launch_bounds__(kPartThreads, kPartCtasPerSm) list_partition_kernel(LevelArgs a)
+// a child searches its lists next depth
+__device__ __forceinline__ bool needs_lists(const LevelArgs &a, uint32_t len, uint32_t n)
 {
-    __shared__ uint32_t s_np[kPartStage];
-    const uint32_t list_n = *a.list_n;
-    const int warp = threadIdx.x >> 5;
-    for (uint32_t k = blockIdx.x; k < list_n; k += gridDim.x) {
+    const int d1 = level_depth(a) + 1;
+    return !(a.max_depth > 0 && d1 >= a.max_depth) && len > (uint32_t)kSmallNodeRows && n > (uint32_t)a.min_node;
+}
+
+// the best of a node's candidates, in every lane of a warp
+__device__ __forceinline__ Cand list_winner(const LevelArgs &a, const ListArgs &l, uint32_t k, const NodeRec &nd)
+{
+    const int lane = threadIdx.x & 31;
+    Cand c = cand_none();
+    for (int q = lane; q < l.m; q += 32) {
+        const Cand o = l.cand[(size_t)k * (size_t)l.m + q];
+        if (cand_better(o, c, nd.n, nd.S)) c = o;
+    }
+    return warp_best(c, nd.n, nd.S);
+}
+
+// one lane: the split of node j by candidate c, whose left side ends at word c.r of its feature's list L
+template <typename RT>
+__device__ __forceinline__ void write_list_split(const LevelArgs &a, int j, const Cand &c, const uint32_t *L, const Entry *rin)
+{
+    SplitRes sr;
+    const uint32_t row = AIWCRF_IDX(rin[L[c.r] & kListPos].row, (uint32_t)a.N, kBoundRow);
+    sr.feature = c.f;
+    sr.rank = (uint32_t)static_cast<const RT *>(a.Rr)[(size_t)row * (size_t)a.F + c.f];
+    sr.thr_bits = 0u;                                   // looked up where the node is encoded
+    sr.nL = c.nL; sr.lenL = c.r + 1u; sr.pad = 0u; sr.v = c.SL;
+    a.res[j] = sr;
+    atomicAdd(&a.tile_splits[(uint32_t)j / (uint32_t)kScanTile], 1u);
+}
+
+template <typename RT>
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kernel(LevelArgs a, ListArgs l)
+{
+    __shared__ uint32_t bits_s[kListWarps][32];
+    __shared__ uint16_t dest_s[kListWarps][kWarpNode];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t list_n = *a.list_n, step = gridDim.x * kListWarps, lt = lanemask_lt();
+    for (uint32_t k = blockIdx.x * kListWarps + warp; k < list_n; k += step) {
         const int j = AIWCRF_IDX(a.list[k], a.node_cap, kBoundNode);
-        const SplitRes sr = a.res[j];
-        if (sr.feature < 0) continue;                                // block-uniform: a leaf
         const NodeRec nd = a.nodes[j];
-        // a child needs its lists only if it is searched by the list kernel next depth
-        const int d1 = level_depth(a) + 1;
-        const bool deep = a.max_depth > 0 && d1 >= a.max_depth;
-        const bool needL = !deep && sr.lenL > (uint32_t)kSmallNodeRows && sr.nL > (uint32_t)a.min_node;
-        const bool needR = !deep && nd.len - sr.lenL > (uint32_t)kSmallNodeRows && nd.n - sr.nL > (uint32_t)a.min_node;
-        if (!needL && !needR) continue;                              // block-uniform
-        const uint32_t *np = a.newpos + (size_t)nd.tree * (size_t)a.row_cap + nd.start;
-        const bool staged = nd.len <= (uint32_t)kPartStage;
-        __syncthreads();                                             // the previous node's copy is read
-        if (staged) {
-            for (uint32_t q = threadIdx.x; q < nd.len; q += kPartThreads) s_np[q] = __ldg(&np[q]);
-            __syncthreads();
+        if (nd.len > kWarpNode || node_stops(a, nd)) continue;
+        const Cand c = list_winner(a, l, k, nd);
+        if (c.h < 0.0f) {
+            if (lane == 0) write_leaf(a.res, j, -1, 0);
+            continue;
         }
-        for (int f = warp; f < a.F; f += kPartThreads / 32)
-            list_partition_feature(a, nd, f, sr.lenL, staged ? s_np : np, needL, needR);
+        const size_t tb = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
+        const Entry *__restrict__ rin = a.rows_in + tb;
+        Entry *__restrict__ rout = a.rows_out + tb;
+        const uint32_t *__restrict__ L = a.lists_in + (size_t)c.f * (size_t)a.list_stride + tb;
+        const uint32_t lenL = c.r + 1u;
+        bits_s[warp][lane] = 0u;
+        __syncwarp();
+        for (uint32_t i = (uint32_t)lane; i < lenL; i += 32u) {
+            const uint32_t p = AIWCRF_IDX(__ldg(&L[i]) & kListPos, nd.len, kBoundOut);
+            atomicOr(&bits_s[warp][p >> 5], 1u << (p & 31u));
+        }
+        __syncwarp();
+        const uint32_t bits = bits_s[warp][lane];
+        uint32_t before = __popc(bits);                             // entries of the earlier words that go left
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, before, o);
+            if (lane >= o) before += t;
+        }
+        before -= __popc(bits);
+        uint16_t *dest = dest_s[warp];                              // place within the child; top bit: left
+        for (uint32_t w0 = 0; 32u * w0 < nd.len; w0 += 4u) {        // four words of entries in flight
+            Entry e[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4u; ++u) {
+                const uint32_t i = 32u * (w0 + u) + (uint32_t)lane;
+                if (i < nd.len) e[u] = load_entry(rin + i);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < 4u; ++u) {
+                const uint32_t i = 32u * (w0 + u) + (uint32_t)lane;
+                const uint32_t bw = __shfl_sync(kFull, bits, (int)(w0 + u) & 31);
+                const uint32_t nl = __shfl_sync(kFull, before, (int)(w0 + u) & 31) + __popc(bw & lt);
+                if (i < nd.len) {
+                    const bool left = (bw >> lane) & 1u;
+                    store_entry(&rout[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)], e[u]);
+                    dest[i] = (uint16_t)(left ? nl | 0x8000u : i - nl);
+                }
+            }
+        }
+        const bool needL = needs_lists(a, lenL, c.nL), needR = needs_lists(a, nd.len - lenL, nd.n - c.nL);
+        if (needL || needR) {
+            __syncwarp();
+            list_partition(a, nd, 0, 1, lenL, needL, needR, [&](uint32_t p) {
+                const uint32_t d = dest[p];
+                return (d & 0x8000u) << 16 | (d & 0x7FFFu);
+            });
+        }
+        if (lane == 0) write_list_split<RT>(a, j, c, L, rin);
+        __syncwarp();
+    }
+}
+
+// The CTA form, for nodes of more than kWarpNode entries: the bit set and its prefix counts in shared
+// memory, the entries over all threads, the features over the warps. A node of more than 32 *
+// kCtaNodeWords entries has no room there: its entries' new positions go to a.newpos instead.
+// kHugeParts CTAs take one node, each a share of its features (the first also the entries): 500 roots of
+// 70,000 entries are then 2,000 items for 608 resident CTAs.
+constexpr int kHugeThreads = 256, kHugeParts = 4, kHugeCtasPerSm = 4;
+template <typename RT>
+__global__ void __launch_bounds__(kHugeThreads, kHugeCtasPerSm) list_split_huge_kernel(LevelArgs a, ListArgs l)
+{
+    __shared__ uint2 bits[kCtaNodeWords];                           // a word, entries of the earlier words that go left
+    __shared__ uint32_t warp_tmp[32];
+    __shared__ Cand winner;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t n = l.n_huge[level_depth(a) & 1];
+    for (uint32_t h = blockIdx.x; h < n * kHugeParts; h += gridDim.x) {
+        const uint32_t k = (uint32_t)l.huge[h / kHugeParts];
+        const int part = (int)(h % kHugeParts);
+        const bool first = part == 0;
+        const int j = AIWCRF_IDX(a.list[k], a.node_cap, kBoundNode);
+        const NodeRec nd = a.nodes[j];
+        __syncthreads();                                            // the node before is done with shared memory
+        if (warp == 0) {
+            const Cand c = list_winner(a, l, k, nd);
+            if (lane == 0) winner = c;
+        }
+        __syncthreads();
+        const Cand c = winner;
+        if (c.h < 0.0f) {
+            if (first && tid == 0) write_leaf(a.res, j, -1, 0);
+            continue;                                               // block-uniform
+        }
+        const size_t tb = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
+        const Entry *__restrict__ rin = a.rows_in + tb;
+        Entry *__restrict__ rout = a.rows_out + tb;
+        const uint32_t *__restrict__ L = a.lists_in + (size_t)c.f * (size_t)a.list_stride + tb;
+        const uint32_t lenL = c.r + 1u, words = (nd.len + 31u) >> 5;
+        const bool whole = words > kCtaNodeWords;                   // the first CTA alone writes a.newpos
+        if (!first && (whole || part * (kHugeThreads / 32) >= a.F)) continue;
+        const int f0 = part * (kHugeThreads / 32) + warp, df = (whole ? 1 : kHugeParts) * (kHugeThreads / 32);
+        const bool needL = needs_lists(a, lenL, c.nL), needR = needs_lists(a, nd.len - lenL, nd.n - c.nL);
+        if (!whole) {
+            for (uint32_t w = (uint32_t)tid; w < words; w += kHugeThreads) bits[w] = make_uint2(0u, 0u);
+            __syncthreads();
+#pragma unroll 4
+            for (uint32_t i = (uint32_t)tid; i < lenL; i += kHugeThreads) {
+                const uint32_t p = AIWCRF_IDX(__ldg(&L[i]) & kListPos, nd.len, kBoundOut);
+                atomicOr(&bits[p >> 5].x, 1u << (p & 31u));
+            }
+            __syncthreads();
+            constexpr uint32_t kPer = kCtaNodeWords / kHugeThreads;  // consecutive words a thread
+            uint32_t sum = 0u;
+            for (uint32_t u = 0; u < kPer; ++u) {
+                const uint32_t w = kPer * (uint32_t)tid + u;
+                if (w < words) sum += __popc(bits[w].x);
+            }
+            uint32_t tot;
+            uint32_t run = block_incl_scan(sum, warp_tmp, tot) - sum;
+            for (uint32_t u = 0; u < kPer; ++u) {
+                const uint32_t w = kPer * (uint32_t)tid + u;
+                if (w < words) { bits[w].y = run; run += __popc(bits[w].x); }
+            }
+            __syncthreads();
+            auto place = [&](uint32_t p) {
+                const uint2 bw = bits[p >> 5];
+                const uint32_t nl = bw.y + __popc(bw.x & ((1u << (p & 31u)) - 1u));
+                return (bw.x >> (p & 31u)) & 1u ? nl | kListBreak : p - nl;
+            };
+#pragma unroll 4
+            for (uint32_t i = (uint32_t)tid; first && i < nd.len; i += kHugeThreads) {
+                const uint32_t d = place(i);
+                store_entry(&rout[AIWCRF_IDX(d & kListBreak ? d & kListPos : lenL + d, nd.len, kBoundOut)], load_entry(rin + i));
+            }
+            if (needL || needR) list_partition(a, nd, f0, df, lenL, needL, needR, place);
+        } else {
+            // stable partition by rank, a CTA's width of entries a step
+            const RT *__restrict__ Rr = static_cast<const RT *>(a.Rr);
+            const uint32_t rank = (uint32_t)Rr[(size_t)AIWCRF_IDX(rin[L[c.r] & kListPos].row, (uint32_t)a.N, kBoundRow) * a.F + c.f];
+            uint32_t *np = a.newpos + tb;
+            uint32_t run_l = 0u, run_r = 0u;
+            for (uint32_t b0 = 0; b0 < nd.len; b0 += kHugeThreads) {
+                const uint32_t i = b0 + (uint32_t)tid;
+                const bool valid = i < nd.len;
+                Entry e;
+                e.row = 0u; e.w = 0u; e.wy = 0;
+                if (valid) e = load_entry(rin + i);
+                const bool left =
+                    valid && (uint32_t)__ldg(&Rr[(size_t)AIWCRF_IDX(e.row, (uint32_t)a.N, kBoundRow) * (size_t)a.F + c.f]) <= rank;
+                uint32_t tot;
+                const uint32_t nl = block_incl_scan(left ? 1u : 0u, warp_tmp, tot) - (left ? 1u : 0u);
+                if (valid) {
+                    const uint32_t d = left ? run_l + nl : run_r + (uint32_t)tid - nl;
+                    store_entry(&rout[AIWCRF_IDX(left ? d : lenL + d, nd.len, kBoundOut)], e);
+                    np[i] = left ? d | kListBreak : d;
+                }
+                run_l += tot;
+                run_r += min((uint32_t)kHugeThreads, nd.len - b0) - tot;
+            }
+            __syncthreads();                                        // the CTA's writes of np are seen by its reads
+            auto place = [&](uint32_t p) { return np[p]; };
+            if (needL || needR) list_partition(a, nd, f0, df, lenL, needL, needR, place);
+        }
+        if (first && tid == 0) write_list_split<RT>(a, j, c, L, rin);
     }
 }
 
 // One CTA per node with more than 32 entries. Shared bins, bin_cap of them, hold per rank
 // of every tried feature: sum w (u32) and sum w*y as an exact (low u32, high i32) pair. All
 // updates are native 32-bit shared atomics; a wrap of the low word carries into the high word.
-template <typename RT, bool LISTS, int NT = kBigThreads>
+template <typename RT, int NT = kBigThreads>
 __device__ __forceinline__ void big_node(const LevelArgs &a, int bin_cap, int j)
 {
     const RT *__restrict__ Rr = static_cast<const RT *>(a.Rr);
@@ -1315,8 +1695,7 @@ __device__ __forceinline__ void big_node(const LevelArgs &a, int bin_cap, int j)
     const uint32_t total_bins = fbase[m];
     Cand best = cand_none();
 
-    if constexpr (LISTS) best = list_search<RT, NT / 32>(a, nd, feats, m, reinterpret_cast<unsigned char *>(sm_bins));
-    else for (uint32_t g0 = 0; g0 < total_bins; g0 += (uint32_t)bin_cap) {
+    for (uint32_t g0 = 0; g0 < total_bins; g0 += (uint32_t)bin_cap) {
         const uint32_t g1 = min(total_bins, g0 + (uint32_t)bin_cap);
         const int nb = (int)(g1 - g0);
         for (int b = tid; b < nb; b += NT) { bw[b] = 0u; blo[b] = 0u; bhi[b] = 0; }
@@ -1507,7 +1886,6 @@ __device__ __forceinline__ void big_node(const LevelArgs &a, int bin_cap, int j)
             const uint32_t before_l = incl - (left ? 1u : 0u);
             const uint32_t dst = AIWCRF_IDX(left ? run_l + before_l : lenL + run_r + ((uint32_t)tid - before_l), nd.len, kBoundOut);
             store_entry(&rout[dst], e);
-            if constexpr (LISTS) a.newpos[tb + i] = dst;
         }
         run_l += tot;
         run_r += min((uint32_t)NT, nd.len - b0) - tot;
@@ -1530,25 +1908,7 @@ __global__ void __launch_bounds__(kBigThreads, kBigCtasPerSm) level_big_kernel(L
     const uint32_t list_n = *a.list_n;
     for (uint32_t k = blockIdx.x; k < list_n; k += gridDim.x) {
         __syncthreads();                 // the previous node's shared state is no longer read
-        big_node<RT, false>(a, bin_cap, a.list[k]);
-    }
-}
-
-// the same with the presorted-list search (a.lists_in set): wider CTAs (a node's lists are
-// shared among more warps: the top depths hold few, long nodes) with 128 registers per thread
-// for the loads the warps keep in flight
-#ifndef AIWCRF_LIST_THREADS
-#define AIWCRF_LIST_THREADS 128
-#endif
-constexpr int kListThreads = AIWCRF_LIST_THREADS;
-constexpr int kListCtasPerSm = 65536 / (kListThreads * 128);
-template <typename RT>
-__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) level_list_kernel(LevelArgs a)
-{
-    const uint32_t list_n = *a.list_n;
-    for (uint32_t k = blockIdx.x; k < list_n; k += gridDim.x) {
-        __syncthreads();
-        big_node<RT, true, kListThreads>(a, 0, a.list[k]);
+        big_node<RT>(a, bin_cap, a.list[k]);
     }
 }
 
@@ -3054,8 +3414,10 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
         AIWCRF_CUDA(cudaMemsetAsync(is_rep, 0, (size_t)N, s));
         rep_mark_kernel<<<(unsigned)((n_groups + 255) / 256), 256, 0, s>>>(grp_rows, grp_off, n_groups, is_rep);
         rep_order_kernel<<<(unsigned)F, 1024, 0, s>>>(d_ordF, N, is_rep, n_groups, d_ordG);
-        count_launches(1);
-        AIWCRF_LAUNCH_CHECK("rep_mark / rep_order");
+        AIWCRF_BY_RANK(rank_bytes, rep_break_kernel<RT><<<dim3((unsigned)((n_groups + 255) / 256), (unsigned)F), 256, 0, s>>>(
+                                       d_ordG, n_groups, (const RT *)d_Rr, F))
+        count_launches(2);
+        AIWCRF_LAUNCH_CHECK("rep_mark / rep_order / rep_break");
         sc.drop(is_rep);
         sc.drop(d_ordF);
     }
@@ -3222,16 +3584,28 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
     // presorted lists of every tree: its entries by representative row, then per feature in rank order
     const int64_t list_stride = T * row_cap;
     uint32_t *lists_a = nullptr, *lists_b = nullptr, *newpos = nullptr;
+    ListArgs ll = {};
     if (use_lists) {
         uint32_t *P = sc.get<uint32_t>((size_t)T * (size_t)N, &rc); if (rc) return rc;
         lists_a = sc.get<uint32_t>((size_t)F * (size_t)list_stride, &rc); if (rc) return rc;
         lists_b = sc.get<uint32_t>((size_t)F * (size_t)list_stride, &rc); if (rc) return rc;
-        newpos = sc.get<uint32_t>((size_t)list_stride, &rc); if (rc) return rc;
+        if (row_cap > 32 * (int64_t)kCtaNodeWords) {
+            newpos = sc.get<uint32_t>((size_t)list_stride, &rc); if (rc) return rc;
+        }
+        // a depth's list holds nodes of more than kSmallNodeRows entries, and a root of any size per tree
+        const size_t slots = (size_t)(list_stride / (kSmallNodeRows + 1) + T + 1);
+        ll.m = std::min(p.mtry, F);
+        ll.node = sc.get<ListNode>(slots, &rc); if (rc) return rc;
+        ll.feat = sc.get<uint8_t>(slots * (size_t)ll.m, &rc); if (rc) return rc;
+        ll.cand = sc.get<Cand>(slots * (size_t)ll.m, &rc); if (rc) return rc;
+        ll.huge = sc.get<int32_t>((size_t)(list_stride / (kWarpNode + 1) + T + 1), &rc); if (rc) return rc;
+        ll.n_huge = sc.get<uint32_t>(2, &rc); if (rc) return rc;
+        AIWCRF_CUDA(cudaMemsetAsync(ll.n_huge, 0, 2 * sizeof(uint32_t), s));
         prof_begin(s, kProfBoot);
         AIWCRF_CUDA(cudaMemsetAsync(P, 0, sizeof(uint32_t) * (size_t)T * (size_t)N, s));
         list_pos_kernel<<<dim3((unsigned)((row_cap + 255) / 256), (unsigned)T), 256, 0, s>>>(rows_a, row_cap, nodes_cur, N, P);
         AIWCRF_LAUNCH_CHECK("list_pos_kernel");
-        list_build_kernel<<<dim3((unsigned)T, (unsigned)F), 1024, 0, s>>>(d_ordG, n_groups, P, N, row_cap, list_stride,
+        list_build_kernel<<<dim3((unsigned)F, (unsigned)T), 1024, 0, s>>>(d_ordG, n_groups, P, N, row_cap, list_stride,
                                                                          lists_a);
         AIWCRF_LAUNCH_CHECK("list_build_kernel");
         prof_end(s, kProfBoot);
@@ -3310,11 +3684,6 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
         AIWCRF_BY_RANK(rank_bytes, e_ = cudaFuncSetAttribute(level_big_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                              big_smem))
         if (e_ != cudaSuccess) return cuda_fail(e_, "level_big_kernel attribute");
-        if (use_lists) {
-            AIWCRF_BY_RANK(rank_bytes, e_ = cudaFuncSetAttribute(level_list_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                                 list_stage_bytes<kListThreads / 32>()))
-            if (e_ != cudaSuccess) return cuda_fail(e_, "level_list_kernel attribute");
-        }
     }
 
     LevelArgs la;
@@ -3382,16 +3751,25 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
                 const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb, cps_big * dev_sms));
                 prof_begin(s, kProfLevelBig);
                 if (use_lists) {
-                    const int64_t cps_list = p.ctas_per_sm > 0 ? p.ctas_per_sm : kListCtasPerSm;
-                    const unsigned lgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb, cps_list * dev_sms));
-                    AIWCRF_BY_RANK(rank_bytes, level_list_kernel<RT><<<lgrid, kListThreads, list_stage_bytes<kListThreads / 32>(), s>>>(la))
-                    AIWCRF_LAUNCH_CHECK("level_list_kernel");
+                    // warps per node and per (node, feature); a depth has at most Cb nodes in its list
+                    const int64_t cps = p.ctas_per_sm > 0 ? p.ctas_per_sm : kListCtasPerSm;
+                    auto warps = [&](int64_t items) {
+                        return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + kListWarps - 1) / kListWarps, cps * dev_sms));
+                    };
+                    list_draw_kernel<<<warps(Cb), kListThreads, 0, s>>>(la, ll);
+                    AIWCRF_LAUNCH_CHECK("list_draw_kernel");
+                    list_search_kernel<<<warps(Cb * ll.m), kListThreads, 0, s>>>(la, ll);
+                    AIWCRF_LAUNCH_CHECK("list_search_kernel");
+                    list_search_huge_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb * ll.m, cps * dev_sms)),
+                                              kListThreads, 0, s>>>(la, ll);
+                    AIWCRF_LAUNCH_CHECK("list_search_huge_kernel");
                     prof_end(s, kProfLevelBig);
                     prof_begin(s, kProfListPart);
-                    const int64_t cps_part = p.ctas_per_sm > 0 ? p.ctas_per_sm : kPartCtasPerSm;
-                    const unsigned pgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb, cps_part * dev_sms));
-                    list_partition_kernel<<<pgrid, kPartThreads, 0, s>>>(la);
-                    AIWCRF_LAUNCH_CHECK("list_partition_kernel");
+                    const unsigned hgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb * kHugeParts, std::min<int64_t>(cps, kHugeCtasPerSm) * dev_sms));
+                    AIWCRF_BY_RANK(rank_bytes, list_split_huge_kernel<RT><<<hgrid, kHugeThreads, 0, s>>>(la, ll))
+                    AIWCRF_LAUNCH_CHECK("list_split_huge_kernel");
+                    AIWCRF_BY_RANK(rank_bytes, list_split_kernel<RT><<<warps(Cb), kListThreads, 0, s>>>(la, ll))
+                    AIWCRF_LAUNCH_CHECK("list_split_kernel");
                     prof_end(s, kProfListPart);
                 } else {
                     AIWCRF_BY_RANK(rank_bytes, level_big_kernel<RT><<<grid, kBigThreads, big_smem, s>>>(la, bin_cap))

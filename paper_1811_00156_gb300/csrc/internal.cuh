@@ -287,10 +287,9 @@ __device__ __forceinline__ Cand shfl_cand(const Cand &c, int src)
 // contenders are then compared exactly, in lane order.
 __device__ __forceinline__ Cand warp_best(const Cand &mine, uint32_t n, int64_t S)
 {
-    float hm = mine.h;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) hm = fmaxf(hm, __shfl_xor_sync(kFull, hm, off));
-    if (hm < 0.0f) return cand_none();
+    // a candidate's h is positive (delta != 0), and positive floats order as their bits
+    const float hm = __uint_as_float(__reduce_max_sync(kFull, mine.h > 0.0f ? __float_as_uint(mine.h) : 0u));
+    if (hm == 0.0f) return cand_none();
     const uint32_t cont = __ballot_sync(kFull, mine.h >= 0.0f && mine.h >= hm * kFilterLo);
     int src = __ffs(cont) - 1;
     Cand best = shfl_cand(mine, src);
