@@ -812,6 +812,66 @@ __device__ __forceinline__ void warp_mtry(const LevelArgs &a, uint32_t tg, uint3
     warp_mtry_s(a.F, a.mtry, (uint32_t)level_depth(a), a.seed_lo, a.seed_hi, tg, idx, mask);
 }
 
+// The same draw for F <= 32 by four lanes, so eight nodes a warp (tg, idx: of the lane's node; every lane
+// calls). Lane s of the four holds the keys of features 4 s .. 4 s + 3 and 16 + 4 s .. in a sorted list; mtry
+// rounds pop the smallest head of the four lists, the last is the largest key drawn, and equal keys there
+// go to the lower features. About 50 instructions a node; the warp-wide draw is 250, most of them
+// computed four times over (a key block serves four features) or waiting for its mtry reductions.
+__device__ __forceinline__ uint32_t quad_mtry(int F, int mtry, uint32_t depth, uint32_t seed_lo, uint32_t seed_hi, uint32_t tg,
+                                              uint32_t idx)
+{
+    if (mtry >= F) return F == 32 ? 0xFFFFFFFFu : (1u << F) - 1u;
+    const uint32_t s = threadIdx.x & 3u;
+    uint32_t key[8], v[8];
+#pragma unroll
+    for (uint32_t h = 0; h < 2u; ++h) {
+        const uint4 u = philox10(make_uint4(tg, depth, idx, (kDomMtry << 16) | (s + 4u * h)), seed_lo, seed_hi);
+#pragma unroll
+        for (uint32_t w = 0; w < 4u; ++w) key[4u * h + w] = (int)(16u * h + 4u * s + w) < F ? uint4_word(u, (int)w) : 0xFFFFFFFFu;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = key[i];
+    auto order = [&](int i, int j) {
+        const uint32_t lo = min(v[i], v[j]), hi = max(v[i], v[j]);
+        v[i] = lo;
+        v[j] = hi;
+    };
+    // odd-even merge sort of eight
+    order(0, 1); order(2, 3); order(4, 5); order(6, 7);
+    order(0, 2); order(1, 3); order(4, 6); order(5, 7);
+    order(1, 2); order(5, 6);
+    order(0, 4); order(1, 5); order(2, 6); order(3, 7);
+    order(2, 4); order(3, 5);
+    order(1, 2); order(3, 4); order(5, 6);
+    uint32_t last = 0u;
+    for (int r = 0; r < mtry; ++r) {
+        uint32_t mn = min(v[0], __shfl_xor_sync(kFull, v[0], 1));
+        mn = min(mn, __shfl_xor_sync(kFull, mn, 2));
+        last = mn;
+        // the lowest lane of the four that holds it pops its list
+        const uint32_t has = __ballot_sync(kFull, v[0] == mn) >> (threadIdx.x & 28u) & 15u;
+        if ((has & ((2u << s) - 1u)) == 1u << s) {
+#pragma unroll
+            for (int i = 0; i < 7; ++i) v[i] = v[i + 1];
+            v[7] = 0xFFFFFFFFu;
+        }
+    }
+    uint32_t below = 0u, equal = 0u;
+#pragma unroll
+    for (uint32_t i = 0; i < 8u; ++i) {
+        const uint32_t bit = 1u << ((i >> 2) * 16u + 4u * s + (i & 3u));
+        below |= key[i] < last ? bit : 0u;
+        equal |= key[i] == last ? bit : 0u;
+    }
+#pragma unroll
+    for (int o = 1; o <= 2; o <<= 1) {
+        below |= __shfl_xor_sync(kFull, below, o);
+        equal |= __shfl_xor_sync(kFull, equal, o);
+    }
+    for (int extra = __popc(below) + __popc(equal) - mtry; extra > 0; --extra) equal &= ~(0x80000000u >> __clz(equal));
+    return below | equal;
+}
+
 __device__ __forceinline__ long long shfl_xor_ll(long long v, int m)
 {
     return __shfl_xor_sync(kFull, v, m);
@@ -1918,15 +1978,18 @@ __global__ void __launch_bounds__(kBigThreads, kBigCtasPerSm) level_big_kernel(L
 // partitions into the children's segments. Node tables of the current and the next depth,
 // split results and the big nodes' per-feature candidates live in a global scratch slot of the
 // CTA. Per depth:
+//   0  the tried features of every node to search, four lanes a node (nodes that stop or have one entry
+//      are in no list: the drawing and skipping warp by warp took 230 of 2,750 us, 500 trees of 2,220
+//      groups, and 30 of 740, 128 trees);
 //   A  work items, taken by the warps in turn: (big node, k-th tried feature) -- a warp-private
 //      shared-memory histogram of (sum w, sum w*y) per rank of that feature, a scan and the
-//      best candidate of that feature; then every small node (<= 32 entries), searched whole
-//      by one warp with the bitonic method of level_small_kernel;
+//      best candidate of that feature; then every small node (<= 32 entries) on its list,
+//      searched whole by one warp with the bitonic method of level_small_kernel;
 //   B  per big node, one warp: the best of its features' candidates, and the stable partition
 //      of its entries;
 //   C  all threads: an exclusive scan of the split flags numbers the children breadth first;
-//      every node is encoded into the tree's output and the next depth's nodes and big-node
-//      list are written.
+//      every node is encoded into the tree's output and the next depth's nodes and lists are
+//      written.
 // It is used when every tree's entries fit in shared memory (grouped rows, one-byte ranks,
 // F <= 32) and replaces the level-synchronous path's three launches per depth. Trees are the
 // same node for node: the same BFS numbering, mtry draws, exact candidate comparison,
@@ -1952,7 +2015,7 @@ struct TNode {            // an active node of a CTA's tree at the current depth
     uint32_t n;           // sum of multiplicities
     int64_t S;            // sum of w*y
     uint32_t idx;         // BFS index within the depth
-    uint32_t pad;
+    uint32_t tried;       // tried features (of the list of small nodes to search)
 };
 static_assert(sizeof(TNode) == 24, "TNode layout");
 
@@ -1977,7 +2040,7 @@ struct TreeArgs {
     int ecap;                     // entry capacity of the shared-memory arrays (>= row_cap)
     int bins;                     // histogram bins per warp (>= every card)
     int big_cap;                  // big nodes per depth at most (ecap / 33 + 1)
-    TNode *nodes;                 // per CTA: 2 * ecap
+    TNode *nodes;                 // per CTA: 2 * ecap, then ecap for the small nodes to search
     SplitRes *res;                // per CTA: ecap
     Cand *cands;                  // per CTA: big_cap * 32
     uint64_t *out_nodes, *out_cnodes;   // per tree t at t * node_cap, BFS order
@@ -2033,6 +2096,12 @@ __device__ __forceinline__ bool tnode_stops(const TreeArgs &a, uint32_t n, uint3
 __device__ __forceinline__ bool tnode_big(const TreeArgs &a, const TNode &nd, uint32_t depth)
 {
     return nd.len > (uint32_t)kSmallNodeRows && !tnode_stops(a, nd.n, depth);
+}
+
+// a node that one warp searches whole
+__device__ __forceinline__ bool tnode_small(const TreeArgs &a, const TNode &nd, uint32_t depth)
+{
+    return nd.len > 1 && nd.len <= (uint32_t)kSmallNodeRows && !tnode_stops(a, nd.n, depth);
 }
 
 // One pass of a small node's search with K-entry segments (K a power of two): the keys
@@ -2096,20 +2165,12 @@ __device__ __forceinline__ void small_sort_scan_rt(int K, uint32_t rank, int pos
     if (pos == K - 1) nr = kRankSentinel;
 }
 
-// A small node (or a node that stops) searched whole by one warp: as small_node, on the tree's
+// A small node of at least two entries that does not stop, searched whole by one warp: as small_node, on the tree's
 // shared-memory entries and the group records, with the passes' rank loads issued together and
 // the sort and scan unrolled for the node's segment width.
 __device__ __forceinline__ void tree_small_node(const TreeArgs &a, const TreeSmem &sm, const uint16_t *ix, uint16_t *ox,
-                                                const TNode &nd, uint32_t tg, uint32_t depth, SplitRes *res_j, int lane)
+                                                const TNode &nd, SplitRes *res_j, int lane)
 {
-    if (tnode_stops(a, nd.n, depth)) {
-        if (lane == 0) write_leaf(res_j, 0, -2, 0);
-        return;
-    }
-    if (nd.len == 1) {                  // one entry: every candidate is its last rank, a leaf
-        if (lane == 0) write_leaf(res_j, 0, -1, 0);
-        return;
-    }
     const int len = nd.len;
     const int K = len <= 2 ? 2 : (int)(1u << (32 - __clz(len - 1)));
     const int P = 32 / K;
@@ -2123,8 +2184,7 @@ __device__ __forceinline__ void tree_small_node(const TreeArgs &a, const TreeSme
     }
     const uint8_t *rec = a.Rg + (size_t)AIWCRF_IDX(eg, a.n_groups, kBoundRow) * kRecBytes;
 
-    uint32_t mask[4];
-    warp_mtry_s(a.F, a.mtry, depth, a.seed_lo, a.seed_hi, tg, nd.idx, mask);
+    const uint32_t mask[4] = {nd.tried, 0u, 0u, 0u};
     const int n_tried = __popc(mask[0]);
     const int f_lane = lane < n_tried ? nth_feature(mask, lane) : -1;
 
@@ -2428,12 +2488,13 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
     extern __shared__ __align__(16) unsigned char tree_sm[];
     __shared__ uint32_t warp_tmp[32];
     __shared__ unsigned long long red[6][kTreeWarps];
-    __shared__ uint32_t s_nb[2];
+    __shared__ uint32_t s_nb[2], s_nw;                          // big nodes, by depth parity; small nodes to search
     __shared__ uint32_t s_next;                                 // the next phase-A item to hand out
     const TreeSmem sm = tree_smem(tree_sm, a, kTreeWarps);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    TNode *const nodes0 = a.nodes + (size_t)blockIdx.x * 2 * (size_t)a.ecap;
+    TNode *const nodes0 = a.nodes + (size_t)blockIdx.x * 3 * (size_t)a.ecap;
     TNode *const nodes1 = nodes0 + a.ecap;
+    TNode *const work = nodes1 + a.ecap;                        // the depth's small nodes to search
     SplitRes *const res = a.res + (size_t)blockIdx.x * (size_t)a.ecap;
     Cand *const cands = a.cands + (size_t)blockIdx.x * (size_t)a.big_cap * 32;
     uint32_t *const wbins = sm.bins + (size_t)warp * (size_t)a.bins * 3;
@@ -2456,10 +2517,12 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
         }
         if (tid == 0) {
             TNode r;
-            r.start = 0; r.len = (uint16_t)len0; r.n = root.n; r.S = root.S; r.idx = 0u; r.pad = 0u;
+            r.start = 0; r.len = (uint16_t)len0; r.n = root.n; r.S = root.S; r.idx = 0u; r.tried = 0u;
             nodes0[0] = r;
+            work[0] = r;
             const bool big = tnode_big(a, r, 0u);
             s_nb[0] = big ? 1u : 0u;
+            s_nw = tnode_small(a, r, 0u) ? 1u : 0u;
             sm.big[0][0] = 0;
             s_next = kTreeWarps;
         }
@@ -2476,19 +2539,21 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             uint16_t *ox = sm.ix[p ^ 1];
             const uint16_t *big = sm.big[p];
             const uint32_t nb = s_nb[p];
-            // the big nodes' tried features, once per node (their items share them)
-            if (nb) {
-                for (uint32_t bi = (uint32_t)warp; bi < nb; bi += kTreeWarps) {
-                    const TNode nd = cn[AIWCRF_IDX(big[bi], a.ecap, kBoundNode)];
-                    uint32_t mask[4];
-                    warp_mtry_s(a.F, a.mtry, depth, a.seed_lo, a.seed_hi, tg, nd.idx, mask);
-                    if (lane == 0) sm.big_mask[bi] = mask[0];
+            // the tried features of every node to search, four lanes a node (a big node's items share them)
+            const uint32_t nw = s_nw;
+            for (uint32_t i0 = 8u * (uint32_t)warp; i0 < nb + nw; i0 += 8u * kTreeWarps) {
+                const uint32_t i = i0 + (uint32_t)(lane >> 2);
+                const uint32_t idx = i < nb ? (uint32_t)big[i] : i < nb + nw ? work[i - nb].idx : 0u;
+                const uint32_t tried = quad_mtry(a.F, a.mtry, depth, a.seed_lo, a.seed_hi, tg, idx);
+                if ((lane & 3) == 0) {
+                    if (i < nb) sm.big_mask[i] = tried;
+                    else if (i < nb + nw) work[i - nb].tried = tried;
                 }
-                __syncthreads();
             }
+            __syncthreads();
             // A: big-node feature items first (they are the long ones), then the small nodes; a
             // warp that finishes an item takes the next one not yet handed out
-            const uint32_t items = nb * (uint32_t)m + C;
+            const uint32_t items = nb * (uint32_t)m + nw;
             for (uint32_t j = (uint32_t)warp; j < items;) {
                 if (j < nb * (uint32_t)m) {
                     const uint32_t bi = j / (uint32_t)m, k = j - bi * (uint32_t)m;
@@ -2496,9 +2561,8 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     tree_big_item(a, sm, ix, nd, sm.big_mask[bi], (int)k, wbins, &cands[(size_t)bi * 32 + k], lane,
                                   card_lane);
                 } else {
-                    const uint32_t i = j - nb * (uint32_t)m;
-                    const TNode nd = cn[i];
-                    if (!tnode_big(a, nd, depth)) tree_small_node(a, sm, ix, ox, nd, tg, depth, &res[i], lane);
+                    const TNode nd = work[AIWCRF_IDX(j - nb * (uint32_t)m, a.ecap, kBoundNode)];
+                    tree_small_node(a, sm, ix, ox, nd, &res[AIWCRF_IDX(nd.idx, a.ecap, kBoundNode)], lane);
                 }
 #if AIWCRF_TREE_DYN
                 uint32_t jn = 0u;
@@ -2521,7 +2585,7 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             }
             __syncthreads();
             // C: number the children, encode every node, list the next depth
-            uint32_t run_split = 0u, run_big = 0u;
+            uint32_t run_split = 0u, run_big = 0u, run_work = 0u;
             uint16_t *nbig = sm.big[p ^ 1];
             for (uint32_t i0 = 0; i0 < C; i0 += kTreeThreads) {
                 const uint32_t i = i0 + (uint32_t)tid;
@@ -2529,12 +2593,17 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                 SplitRes r;
                 TNode nd;
                 r.feature = -2;
-                if (valid) { r = res[i]; nd = cn[i]; }
+                if (valid) {
+                    r = res[i];
+                    nd = cn[i];
+                    if (tnode_stops(a, nd.n, depth)) r.feature = -2;        // not searched
+                    else if (nd.len == 1) r.feature = -1;                   // one entry: no candidate
+                }
                 const bool split = valid && r.feature >= 0;
                 uint32_t tot;
                 const uint32_t loc = run_split + block_incl_scan(split ? 1u : 0u, warp_tmp, tot) - (split ? 1u : 0u);
                 TNode L, R;
-                bool bigL = false, bigR = false;
+                bool bigL = false, bigR = false, smallL = false, smallR = false;
                 if (valid) {
                     const uint32_t pos = base + i;
                     const uint32_t left = base + C + 2u * loc;
@@ -2544,13 +2613,15 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     onodes[AIWCRF_IDX(pos, a.node_cap, kBoundOut)] = node;
                     ocnodes[AIWCRF_IDX(pos, a.node_cap, kBoundOut)] = split ? encode_split_coded(r.feature, left, r.rank) : node;
                     if (split) {
-                        L.start = nd.start; L.len = (uint16_t)r.lenL; L.n = r.nL; L.S = r.v; L.idx = 2u * loc; L.pad = 0u;
+                        L.start = nd.start; L.len = (uint16_t)r.lenL; L.n = r.nL; L.S = r.v; L.idx = 2u * loc; L.tried = 0u;
                         R.start = (uint16_t)(nd.start + r.lenL); R.len = (uint16_t)(nd.len - r.lenL); R.n = nd.n - r.nL;
-                        R.S = nd.S - r.v; R.idx = 2u * loc + 1u; R.pad = 0u;
+                        R.S = nd.S - r.v; R.idx = 2u * loc + 1u; R.tried = 0u;
                         nx[AIWCRF_IDX(2u * loc, a.ecap, kBoundOut)] = L;
                         nx[AIWCRF_IDX(2u * loc + 1u, a.ecap, kBoundOut)] = R;
                         bigL = tnode_big(a, L, depth + 1u);
                         bigR = tnode_big(a, R, depth + 1u);
+                        smallL = tnode_small(a, L, depth + 1u);
+                        smallR = tnode_small(a, R, depth + 1u);
                     }
                     const bool evald = r.feature != -2;
                     const bool small = nd.len <= (uint32_t)kSmallNodeRows;
@@ -2561,15 +2632,20 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     v[4] += (evald && small) ? nd.len : 0u;
                     v[5] += (split && small) ? nd.len : 0u;
                 }
-                const uint32_t nbi = (bigL ? 1u : 0u) + (bigR ? 1u : 0u);
+                // big and small nodes to search, in one scan (halves: at most 2 * kTreeThreads each)
+                const uint32_t nbi = (bigL ? 1u : 0u) + (bigR ? 1u : 0u) + (smallL ? 0x10000u : 0u) + (smallR ? 0x10000u : 0u);
                 uint32_t totb;
-                uint32_t bpos = run_big + block_incl_scan(nbi, warp_tmp, totb) - nbi;
+                const uint32_t before = block_incl_scan(nbi, warp_tmp, totb) - nbi;
+                uint32_t bpos = run_big + (before & 0xFFFFu), wpos = run_work + (before >> 16);
                 if (bigL) nbig[AIWCRF_IDX(bpos++, a.big_cap, kBoundOut)] = (uint16_t)(2u * loc);
                 if (bigR) nbig[AIWCRF_IDX(bpos, a.big_cap, kBoundOut)] = (uint16_t)(2u * loc + 1u);
+                if (smallL) work[AIWCRF_IDX(wpos++, a.ecap, kBoundOut)] = L;
+                if (smallR) work[AIWCRF_IDX(wpos, a.ecap, kBoundOut)] = R;
                 run_split += tot;
-                run_big += totb;
+                run_big += totb & 0xFFFFu;
+                run_work += totb >> 16;
             }
-            if (tid == 0) { s_nb[p ^ 1] = run_big; s_next = kTreeWarps; }
+            if (tid == 0) { s_nb[p ^ 1] = run_big; s_nw = run_work; s_next = kTreeWarps; }
             base += C;
             C = 2u * run_split;
             ++depth;
@@ -2620,8 +2696,8 @@ TreeKernel tree_kernel(int warps)
 
 // Warps per tree: as many as leave every tree a place on the chip at once, since a tree is a serial
 // chain of depths that more warps shorten, while trees side by side fill an SM as well with 8 warps
-// each. Measured, tree kernel at 8 / 16 / 32 warps: 128 trees of 2,220 rows 1,235 / 828 / 695 us; 500
-// trees of 2,220 groups 2,750 / 3,010 / 3,640 us.
+// each. Measured, tree kernel at 8 / 16 / 32 warps: 128 trees of 2,220 rows 1,211 / 836 / 711 us; 500
+// trees of 2,220 groups 2,515 / 2,820 / 3,515 us.
 int tree_warps(int64_t T, int sms)
 {
     return T <= sms ? 32 : T <= 2 * (int64_t)sms ? 16 : 8;
@@ -3626,7 +3702,7 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
         if (p.ctas_per_sm > 0) occ = std::min<int>(occ, p.ctas_per_sm);
         const int64_t grid = std::min<int64_t>(T, (int64_t)occ * dev_sms);
         const int64_t node_cap = 2 * (int64_t)tree_ecap;
-        TNode *t_nodes = sc.get<TNode>((size_t)grid * 2 * (size_t)tree_ecap, &rc); if (rc) return rc;
+        TNode *t_nodes = sc.get<TNode>((size_t)grid * 3 * (size_t)tree_ecap, &rc); if (rc) return rc;
         SplitRes *t_res = sc.get<SplitRes>((size_t)grid * (size_t)tree_ecap, &rc); if (rc) return rc;
         Cand *t_cands = sc.get<Cand>((size_t)grid * (size_t)tree_big_cap * 32, &rc); if (rc) return rc;
         uint64_t *slot_nodes = sc.get<uint64_t>((size_t)T * (size_t)node_cap, &rc); if (rc) return rc;
