@@ -3514,10 +3514,11 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
     // a background fit keeps to small CTAs; so does a fit whose histograms for more warps do not fit
     int n_tree_warps = p.ctas_per_sm > 0 ? 8 : tree_warps(T, tree_sms);
     auto tree_bytes = [&](int warps) { return tree_smem_bytes(tree_ecap, tree_bins, tree_big_cap, warps); };
-    while (n_tree_warps > 8 && tree_bytes(n_tree_warps) + 1024 > (size_t)max_smem_optin) n_tree_warps /= 2;
+    auto tree_static = [](int warps) { return std::max<size_t>(1024, 64 * (size_t)warps); };   // its own shared variables, at most
+    while (n_tree_warps > 8 && tree_bytes(n_tree_warps) + tree_static(n_tree_warps) > (size_t)max_smem_optin) n_tree_warps /= 2;
     const size_t tree_smem = tree_bytes(n_tree_warps);
     const bool tree_fits = rank8 && F <= 32 && n_groups <= 65535u && row_cap <= 65535 &&
-                           tree_smem + 1024 <= (size_t)max_smem_optin;
+                           tree_smem + tree_static(n_tree_warps) <= (size_t)max_smem_optin;
     if (gmode == AIWCRF_GROWER_TREE && !tree_fits)
         return fail(AIWCRF_E_LIMIT, "tree-resident growth needs one-byte ranks, F <= 32 and a tree's entries in shared memory");
     const bool use_tree = tree_fits && !use_lists && gmode != AIWCRF_GROWER_LEVEL;
