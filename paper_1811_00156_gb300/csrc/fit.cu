@@ -1979,12 +1979,12 @@ __global__ void __launch_bounds__(kBigThreads, kBigCtasPerSm) level_big_kernel(L
 // split results and the big nodes' per-feature candidates live in a global scratch slot of the
 // CTA. Per depth:
 //   0  the tried features of every node to search, four lanes a node (nodes that stop or have one entry
-//      are in no list: the drawing and skipping warp by warp took 230 of 2,750 us, 500 trees of 2,220
+//      are in no list: drawing and skipping them warp by warp took 230 of 2,750 us, 500 trees of 2,220
 //      groups, and 30 of 740, 128 trees);
 //   A  work items, taken by the warps in turn: (big node, k-th tried feature) -- a warp-private
 //      shared-memory histogram of (sum w, sum w*y) per rank of that feature, a scan and the
 //      best candidate of that feature; then every small node (<= 32 entries) on its list,
-//      searched whole by one warp with the bitonic method of level_small_kernel;
+//      searched whole by one warp;
 //   B  per big node, one warp: the best of its features' candidates, and the stable partition
 //      of its entries;
 //   C  all threads: an exclusive scan of the split flags numbers the children breadth first;
@@ -1996,12 +1996,6 @@ __global__ void __launch_bounds__(kBigThreads, kBigCtasPerSm) level_big_kernel(L
 // tie-breaks and leaf values.
 // ------------------------------------------------------------------------------------------
 // build-time tuning of the tree kernel (the forest does not depend on them)
-#ifndef AIWCRF_TREE_UNROLL
-#define AIWCRF_TREE_UNROLL 0           // 1: small-node sort and scan unrolled per segment width
-#endif
-#ifndef AIWCRF_TREE_PREFETCH
-#define AIWCRF_TREE_PREFETCH 1         // small-node passes whose ranks are loaded together
-#endif
 #ifndef AIWCRF_TREE_DYN
 #define AIWCRF_TREE_DYN 1              // 1: phase-A items handed out by a shared counter
 #endif
@@ -2104,30 +2098,38 @@ __device__ __forceinline__ bool tnode_small(const TreeArgs &a, const TNode &nd, 
     return nd.len > 1 && nd.len <= (uint32_t)kSmallNodeRows && !tnode_stops(a, nd.n, depth);
 }
 
-// One pass of a small node's search with K-entry segments (K a power of two): the keys
-// (rank, entry lane) of every segment sorted by a bitonic network, then the prefix of (w, w*y)
-// in that order. r: this lane's rank in sorted order; nr: the next lane's (sentinel at the end).
-template <int K>
-__device__ __forceinline__ void small_sort_scan(uint32_t rank, int pos, int lane, uint32_t w_live, long long wy_live,
-                                                uint32_t &r, uint32_t &cw, long long &cs, uint32_t &nr)
+// One pass of a small node's search with K-entry segments (K a power of two): every segment's entries in
+// order of (rank, entry), then the prefix of (w, w*y) in that order. r: this lane's rank in that order; nr:
+// the next lane's (sentinel at the end). An entry's place is the number of its segment's entries of a
+// lower rank, or of the same rank before it, from one ballot per bit of the one-byte ranks; src_s, 32 bytes
+// of the warp's bins, turns places into lanes (32 bytes a warp more would leave three CTAs on an SM). The ballots are independent of one another, where
+// a bitonic network is a chain of up to 15 exchanges: with it, and the ranks loaded without the next
+// pass's ahead, the tree kernel took 711 us against 593 (128 trees of 2,220 rows) and 2,515 against 2,280
+// (500 trees of 2,220 groups).
+__device__ __forceinline__ void small_order_scan(int K, uint32_t rank, bool live, int pos, int lane, uint32_t w_live,
+                                                 long long wy_live, uint8_t *src_s, uint32_t &r, uint32_t &cw,
+                                                 long long &cs, uint32_t &nr)
 {
-    uint32_t key = (rank << 5) | (uint32_t)pos;
+    const int first = lane & ~(K - 1);                              // the segment's first lane
+    uint32_t eq = __ballot_sync(kFull, live) & ((kFull >> (32 - K)) << first), lt = 0u;
 #pragma unroll
-    for (int k = 2; k <= K; k <<= 1) {
-#pragma unroll
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            const uint32_t ok = __shfl_xor_sync(kFull, key, jj);
-            const bool asc = (pos & k) == 0;
-            const bool lower = (pos & jj) == 0;
-            key = ((lower == asc) ? (ok < key) : (ok > key)) ? ok : key;
-        }
+    for (int b = 7; b >= 0; --b) {
+        const uint32_t ones = __ballot_sync(kFull, (rank >> b) & 1u);
+        const uint32_t mine = (uint32_t)((int32_t)(rank << (31 - b)) >> 31);      // this lane's bit, spread
+        lt |= eq & ~ones & mine;
+        eq &= ~(ones ^ mine);
     }
-    const int src = (lane & ~(K - 1)) | (int)(key & 31u);
-    r = key >> 5;
+    // a lane without an entry, or whose segment has no feature, keeps its place behind the others
+    src_s[first | (live ? __popc(lt) + __popc(eq & lanemask_lt()) : pos)] = (uint8_t)lane;
+    __syncwarp();
+    const int src = src_s[lane];
+    r = __shfl_sync(kFull, rank, src);
     cw = __shfl_sync(kFull, w_live, src);
     cs = __shfl_sync(kFull, wy_live, src);
+    __syncwarp();                                                   // src_s is written again by the next pass
 #pragma unroll
-    for (int o = 1; o < K; o <<= 1) {
+    for (int o = 1; o < 32; o <<= 1) {
+        if (o >= K) break;                                          // warp-uniform
         const uint32_t tw = __shfl_up_sync(kFull, cw, o);
         const long long ts = __shfl_up_sync(kFull, cs, o);
         if (pos >= o) { cw += tw; cs += ts; }
@@ -2136,40 +2138,10 @@ __device__ __forceinline__ void small_sort_scan(uint32_t rank, int pos, int lane
     if (pos == K - 1) nr = kRankSentinel;
 }
 
-constexpr int kSmallPrefetch = AIWCRF_TREE_PREFETCH;   // passes whose ranks a small node loads at once
-
-// the same pass with the segment width a runtime value (one loop for every width)
-__device__ __forceinline__ void small_sort_scan_rt(int K, uint32_t rank, int pos, int lane, uint32_t w_live,
-                                                   long long wy_live, uint32_t &r, uint32_t &cw, long long &cs,
-                                                   uint32_t &nr)
-{
-    uint32_t key = (rank << 5) | (uint32_t)pos;
-    for (int k = 2; k <= K; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            const uint32_t ok = __shfl_xor_sync(kFull, key, jj);
-            const bool asc = (pos & k) == 0;
-            const bool lower = (pos & jj) == 0;
-            key = ((lower == asc) ? (ok < key) : (ok > key)) ? ok : key;
-        }
-    }
-    const int src = (lane & ~(K - 1)) | (int)(key & 31u);
-    r = key >> 5;
-    cw = __shfl_sync(kFull, w_live, src);
-    cs = __shfl_sync(kFull, wy_live, src);
-    for (int o = 1; o < K; o <<= 1) {
-        const uint32_t tw = __shfl_up_sync(kFull, cw, o);
-        const long long ts = __shfl_up_sync(kFull, cs, o);
-        if (pos >= o) { cw += tw; cs += ts; }
-    }
-    nr = __shfl_down_sync(kFull, r, 1);
-    if (pos == K - 1) nr = kRankSentinel;
-}
-
-// A small node of at least two entries that does not stop, searched whole by one warp: as small_node, on the tree's
-// shared-memory entries and the group records, with the passes' rank loads issued together and
-// the sort and scan unrolled for the node's segment width.
+// A small node of at least two entries that does not stop, searched whole by one warp: as small_node, on
+// the tree's shared-memory entries and the group records, with the next pass's ranks on their way.
 __device__ __forceinline__ void tree_small_node(const TreeArgs &a, const TreeSmem &sm, const uint16_t *ix, uint16_t *ox,
-                                                const TNode &nd, SplitRes *res_j, int lane)
+                                                const TNode &nd, SplitRes *res_j, uint8_t *src_s, int lane)
 {
     const int len = nd.len;
     const int K = len <= 2 ? 2 : (int)(1u << (32 - __clz(len - 1)));
@@ -2189,49 +2161,30 @@ __device__ __forceinline__ void tree_small_node(const TreeArgs &a, const TreeSme
     const int f_lane = lane < n_tried ? nth_feature(mask, lane) : -1;
 
     Cand best = cand_none();
-    for (int q0 = 0; q0 < n_tried; q0 += kSmallPrefetch * P) {
-        uint32_t rk[kSmallPrefetch];
-#pragma unroll
-        for (int u = 0; u < kSmallPrefetch; ++u) {
-            const int qf = q0 + u * P + seg;
-            const int fs = __shfl_sync(kFull, f_lane, qf & 31);
-            rk[u] = (valid && qf < n_tried) ? (uint32_t)__ldg(&rec[fs]) : kRankSentinel;
-        }
-#pragma unroll
-        for (int u = 0; u < kSmallPrefetch; ++u) {
-            if (q0 + u * P >= n_tried) break;                       // warp-uniform
-            const int qf = q0 + u * P + seg;
-            const int fs = __shfl_sync(kFull, f_lane, qf & 31);
-            const int f = qf < n_tried ? fs : -1;
-            const bool live = valid && f >= 0;
-            const uint32_t rank = rk[u];
-            // a pass whose features are all constant over the node has no boundary (lane seg*K
-            // always holds an entry; the shuffle runs in every lane before the vote)
-            const uint32_t rank0 = __shfl_sync(kFull, rank, lane & ~(K - 1));
-            if (__all_sync(kFull, !live || rank == rank0)) continue;
-            uint32_t r, cw, nr;
-            long long cs;
-            const uint32_t wl = live ? ew : 0u;
-            const long long yl = live ? ewy : 0ll;
-#if AIWCRF_TREE_UNROLL
-            switch (K) {                                            // warp-uniform
-            case 2: small_sort_scan<2>(rank, pos, lane, wl, yl, r, cw, cs, nr); break;
-            case 4: small_sort_scan<4>(rank, pos, lane, wl, yl, r, cw, cs, nr); break;
-            case 8: small_sort_scan<8>(rank, pos, lane, wl, yl, r, cw, cs, nr); break;
-            case 16: small_sort_scan<16>(rank, pos, lane, wl, yl, r, cw, cs, nr); break;
-            default: small_sort_scan<32>(rank, pos, lane, wl, yl, r, cw, cs, nr); break;
-            }
-#else
-            small_sort_scan_rt(K, rank, pos, lane, wl, yl, r, cw, cs, nr);
-#endif
-            if (f >= 0 && r != kRankSentinel && nr != kRankSentinel && r != nr) {
-                const i128_t delta = cand_delta(nd.n, nd.S, cw, cs);
-                if (delta != 0) {
-                    Cand cd;
-                    cd.h = cand_h(delta, nd.n, cw);
-                    cd.f = f; cd.r = r; cd.nL = cw; cd.SL = cs;
-                    if (cand_better(cd, best, nd.n, nd.S)) best = cd;
-                }
+    auto load_pass = [&](int q0) {
+        const int fs = __shfl_sync(kFull, f_lane, (q0 + seg) & 31);
+        return valid && q0 + seg < n_tried ? (uint32_t)__ldg(&rec[fs]) : kRankSentinel;
+    };
+    uint32_t rank_next = load_pass(0);
+    for (int q0 = 0; q0 < n_tried; q0 += P) {
+        const uint32_t rank = rank_next;
+        rank_next = load_pass(q0 + P);
+        const int fs = __shfl_sync(kFull, f_lane, (q0 + seg) & 31), f = q0 + seg < n_tried ? fs : -1;
+        const bool live = valid && f >= 0;
+        // a pass whose features are all constant over the node has no boundary (lane seg*K
+        // always holds an entry; the shuffle runs in every lane before the vote)
+        const uint32_t rank0 = __shfl_sync(kFull, rank, lane & ~(K - 1));
+        if (__all_sync(kFull, !live || rank == rank0)) continue;
+        uint32_t r, cw, nr;
+        long long cs;
+        small_order_scan(K, rank, live, pos, lane, live ? ew : 0u, live ? ewy : 0ll, src_s, r, cw, cs, nr);
+        if (f >= 0 && r != kRankSentinel && nr != kRankSentinel && r != nr) {
+            const i128_t delta = cand_delta(nd.n, nd.S, cw, cs);
+            if (delta != 0) {
+                Cand cd;
+                cd.h = cand_h(delta, nd.n, cw);
+                cd.f = f; cd.r = r; cd.nL = cw; cd.SL = cs;
+                if (cand_better(cd, best, nd.n, nd.S)) best = cd;
             }
         }
     }
@@ -2562,7 +2515,8 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                                   card_lane);
                 } else {
                     const TNode nd = work[AIWCRF_IDX(j - nb * (uint32_t)m, a.ecap, kBoundNode)];
-                    tree_small_node(a, sm, ix, ox, nd, &res[AIWCRF_IDX(nd.idx, a.ecap, kBoundNode)], lane);
+                    tree_small_node(a, sm, ix, ox, nd, &res[AIWCRF_IDX(nd.idx, a.ecap, kBoundNode)],
+                                    reinterpret_cast<uint8_t *>(wbins), lane);
                 }
 #if AIWCRF_TREE_DYN
                 uint32_t jn = 0u;
@@ -3506,7 +3460,7 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
 
     // Tree-resident growth when every tree's entries fit in shared memory: one-byte ranks,
     // F <= 32, group ids and entry offsets in 16 bits
-    const int tree_bins = (int)std::max<uint32_t>(max_card, 1u);
+    const int tree_bins = (int)std::max<uint32_t>(max_card, 3u);    // 12 bytes each: 32 for small_order_scan
     const int tree_ecap = (int)std::max<int64_t>(row_cap, 1);
     const int tree_big_cap = tree_ecap / (kSmallNodeRows + 1) + 1;
     int tree_sms = 0;
@@ -3514,7 +3468,10 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
     // a background fit keeps to small CTAs; so does a fit whose histograms for more warps do not fit
     int n_tree_warps = p.ctas_per_sm > 0 ? 8 : tree_warps(T, tree_sms);
     auto tree_bytes = [&](int warps) { return tree_smem_bytes(tree_ecap, tree_bins, tree_big_cap, warps); };
-    auto tree_static = [](int warps) { return std::max<size_t>(1024, 64 * (size_t)warps); };   // its own shared variables, at most
+    // the kernel's own shared variables, at most; 8 warps grow what fits with a bin per value
+    auto tree_static = [&](int warps) {
+        return warps > 8 ? 64 * (size_t)warps : 1024 - 12 * (size_t)warps * (size_t)(tree_bins - std::max<int>((int)max_card, 1));
+    };
     while (n_tree_warps > 8 && tree_bytes(n_tree_warps) + tree_static(n_tree_warps) > (size_t)max_smem_optin) n_tree_warps /= 2;
     const size_t tree_smem = tree_bytes(n_tree_warps);
     const bool tree_fits = rank8 && F <= 32 && n_groups <= 65535u && row_cap <= 65535 &&
