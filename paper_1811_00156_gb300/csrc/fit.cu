@@ -2098,6 +2098,17 @@ __device__ __forceinline__ bool tnode_small(const TreeArgs &a, const TNode &nd, 
     return nd.len > 1 && nd.len <= (uint32_t)kSmallNodeRows && !tnode_stops(a, nd.n, depth);
 }
 
+// The depth's last items are its short ones, so that the warps end it together: a node of at most 8 entries
+// takes up to 3 passes of 10 tried features, one of up to 32 takes 10. Measured, tree kernel of 128 trees
+// of 2,220 rows with the line at 4 / 8 / 16 / 32 entries: 570 / 561 / 564 / 578 us (593 with two scans a
+// depth and one list).
+constexpr uint32_t kTreeShort = 8;
+
+__device__ __forceinline__ bool tnode_short(const TNode &nd)
+{
+    return nd.len <= kTreeShort;
+}
+
 // One pass of a small node's search with K-entry segments (K a power of two): every segment's entries in
 // order of (rank, entry), then the prefix of (w, w*y) in that order. r: this lane's rank in that order; nr:
 // the next lane's (sentinel at the end). An entry's place is the number of its segment's entries of a
@@ -2439,15 +2450,18 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
 {
     constexpr int kTreeThreads = 32 * kTreeWarps;
     extern __shared__ __align__(16) unsigned char tree_sm[];
-    __shared__ uint32_t warp_tmp[32];
+    __shared__ unsigned long long warp_tmp[kTreeWarps];
     __shared__ unsigned long long red[6][kTreeWarps];
-    __shared__ uint32_t s_nb[2], s_nw;                          // big nodes, by depth parity; small nodes to search
+    __shared__ uint32_t s_nb[2], s_nw[2];                       // big nodes, by depth parity; small nodes to search
     __shared__ uint32_t s_next;                                 // the next phase-A item to hand out
     const TreeSmem sm = tree_smem(tree_sm, a, kTreeWarps);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     TNode *const nodes0 = a.nodes + (size_t)blockIdx.x * 3 * (size_t)a.ecap;
     TNode *const nodes1 = nodes0 + a.ecap;
-    TNode *const work = nodes1 + a.ecap;                        // the depth's small nodes to search
+    // the depth's small nodes to search: those of more than kTreeShort entries from the front, the others
+    // from the back
+    TNode *const work = nodes1 + a.ecap;
+    auto work_at = [&](uint32_t i, uint32_t n_long) { return i < n_long ? i : (uint32_t)a.ecap - 1u - (i - n_long); };
     SplitRes *const res = a.res + (size_t)blockIdx.x * (size_t)a.ecap;
     Cand *const cands = a.cands + (size_t)blockIdx.x * (size_t)a.big_cap * 32;
     uint32_t *const wbins = sm.bins + (size_t)warp * (size_t)a.bins * 3;
@@ -2472,10 +2486,11 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             TNode r;
             r.start = 0; r.len = (uint16_t)len0; r.n = root.n; r.S = root.S; r.idx = 0u; r.tried = 0u;
             nodes0[0] = r;
-            work[0] = r;
+            work[work_at(0u, tnode_short(r) ? 0u : 1u)] = r;
             const bool big = tnode_big(a, r, 0u);
             s_nb[0] = big ? 1u : 0u;
-            s_nw = tnode_small(a, r, 0u) ? 1u : 0u;
+            s_nw[0] = tnode_small(a, r, 0u) && !tnode_short(r) ? 1u : 0u;
+            s_nw[1] = tnode_small(a, r, 0u) && tnode_short(r) ? 1u : 0u;
             sm.big[0][0] = 0;
             s_next = kTreeWarps;
         }
@@ -2493,14 +2508,14 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             const uint16_t *big = sm.big[p];
             const uint32_t nb = s_nb[p];
             // the tried features of every node to search, four lanes a node (a big node's items share them)
-            const uint32_t nw = s_nw;
+            const uint32_t n_long = s_nw[0], nw = n_long + s_nw[1];
             for (uint32_t i0 = 8u * (uint32_t)warp; i0 < nb + nw; i0 += 8u * kTreeWarps) {
                 const uint32_t i = i0 + (uint32_t)(lane >> 2);
-                const uint32_t idx = i < nb ? (uint32_t)big[i] : i < nb + nw ? work[i - nb].idx : 0u;
+                const uint32_t idx = i < nb ? (uint32_t)big[i] : i < nb + nw ? work[work_at(i - nb, n_long)].idx : 0u;
                 const uint32_t tried = quad_mtry(a.F, a.mtry, depth, a.seed_lo, a.seed_hi, tg, idx);
                 if ((lane & 3) == 0) {
                     if (i < nb) sm.big_mask[i] = tried;
-                    else if (i < nb + nw) work[i - nb].tried = tried;
+                    else if (i < nb + nw) work[work_at(i - nb, n_long)].tried = tried;
                 }
             }
             __syncthreads();
@@ -2514,7 +2529,7 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     tree_big_item(a, sm, ix, nd, sm.big_mask[bi], (int)k, wbins, &cands[(size_t)bi * 32 + k], lane,
                                   card_lane);
                 } else {
-                    const TNode nd = work[AIWCRF_IDX(j - nb * (uint32_t)m, a.ecap, kBoundNode)];
+                    const TNode nd = work[AIWCRF_IDX(work_at(j - nb * (uint32_t)m, n_long), a.ecap, kBoundNode)];
                     tree_small_node(a, sm, ix, ox, nd, &res[AIWCRF_IDX(nd.idx, a.ecap, kBoundNode)],
                                     reinterpret_cast<uint8_t *>(wbins), lane);
                 }
@@ -2530,7 +2545,8 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             // B: big nodes' decisions and partitions (a node per warp, or several warps per
             // node when the depth has fewer big nodes than warps)
             if (nb > 0u && nb < (uint32_t)kTreeWarps) {
-                tree_big_split_w<kTreeWarps>(a, sm, ix, ox, cn, big, nb, m, cands, res, warp_tmp, warp, lane);
+                tree_big_split_w<kTreeWarps>(a, sm, ix, ox, cn, big, nb, m, cands, res,
+                                             reinterpret_cast<uint32_t *>(warp_tmp), warp, lane);
             } else {
                 for (uint32_t bi = (uint32_t)warp; bi < nb; bi += kTreeWarps) {
                     const uint32_t i = AIWCRF_IDX(big[bi], a.ecap, kBoundNode);
@@ -2539,13 +2555,14 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
             }
             __syncthreads();
             // C: number the children, encode every node, list the next depth
-            uint32_t run_split = 0u, run_big = 0u, run_work = 0u;
+            // (16-bit fields of one scan: splits, children that are big, small and long, small and short)
+            unsigned long long run = 0ull;
             uint16_t *nbig = sm.big[p ^ 1];
             for (uint32_t i0 = 0; i0 < C; i0 += kTreeThreads) {
                 const uint32_t i = i0 + (uint32_t)tid;
                 const bool valid = i < C;
                 SplitRes r;
-                TNode nd;
+                TNode nd, L, R;
                 r.feature = -2;
                 if (valid) {
                     r = res[i];
@@ -2554,10 +2571,22 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     else if (nd.len == 1) r.feature = -1;                   // one entry: no candidate
                 }
                 const bool split = valid && r.feature >= 0;
-                uint32_t tot;
-                const uint32_t loc = run_split + block_incl_scan(split ? 1u : 0u, warp_tmp, tot) - (split ? 1u : 0u);
-                TNode L, R;
-                bool bigL = false, bigR = false, smallL = false, smallR = false;
+                uint32_t kindL = 0u, kindR = 0u;                            // a child's field of the scan (0: none)
+                if (split) {
+                    L.start = nd.start; L.len = (uint16_t)r.lenL; L.n = r.nL; L.S = r.v; L.tried = 0u;
+                    R.start = (uint16_t)(nd.start + r.lenL); R.len = (uint16_t)(nd.len - r.lenL); R.n = nd.n - r.nL;
+                    R.S = nd.S - r.v; R.tried = 0u;
+                    auto kind = [&](const TNode &c) {
+                        return tnode_big(a, c, depth + 1u) ? 1u : !tnode_small(a, c, depth + 1u) ? 0u : tnode_short(c) ? 3u : 2u;
+                    };
+                    kindL = kind(L);
+                    kindR = kind(R);
+                }
+                const unsigned long long one = 1ull, oneL = kindL ? one << (16u * kindL) : 0ull, oneR = kindR ? one << (16u * kindR) : 0ull;
+                const unsigned long long mine = (split ? one : 0ull) + oneL + oneR;
+                unsigned long long tot;
+                const unsigned long long at = run + block_incl_scan64(mine, warp_tmp, tot) - mine;
+                const uint32_t loc = (uint32_t)at & 0xFFFFu;
                 if (valid) {
                     const uint32_t pos = base + i;
                     const uint32_t left = base + C + 2u * loc;
@@ -2567,15 +2596,18 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     onodes[AIWCRF_IDX(pos, a.node_cap, kBoundOut)] = node;
                     ocnodes[AIWCRF_IDX(pos, a.node_cap, kBoundOut)] = split ? encode_split_coded(r.feature, left, r.rank) : node;
                     if (split) {
-                        L.start = nd.start; L.len = (uint16_t)r.lenL; L.n = r.nL; L.S = r.v; L.idx = 2u * loc; L.tried = 0u;
-                        R.start = (uint16_t)(nd.start + r.lenL); R.len = (uint16_t)(nd.len - r.lenL); R.n = nd.n - r.nL;
-                        R.S = nd.S - r.v; R.idx = 2u * loc + 1u; R.tried = 0u;
+                        L.idx = 2u * loc;
+                        R.idx = 2u * loc + 1u;
                         nx[AIWCRF_IDX(2u * loc, a.ecap, kBoundOut)] = L;
                         nx[AIWCRF_IDX(2u * loc + 1u, a.ecap, kBoundOut)] = R;
-                        bigL = tnode_big(a, L, depth + 1u);
-                        bigR = tnode_big(a, R, depth + 1u);
-                        smallL = tnode_small(a, L, depth + 1u);
-                        smallR = tnode_small(a, R, depth + 1u);
+                        auto enlist = [&](uint32_t kind, const TNode &c, unsigned long long from) {
+                            if (!kind) return;
+                            const uint32_t k = (uint32_t)(from >> (16u * kind)) & 0xFFFFu;
+                            if (kind == 1u) nbig[AIWCRF_IDX(k, a.big_cap, kBoundOut)] = (uint16_t)c.idx;
+                            else work[AIWCRF_IDX(kind == 2u ? k : (uint32_t)a.ecap - 1u - k, a.ecap, kBoundOut)] = c;
+                        };
+                        enlist(kindL, L, at);
+                        enlist(kindR, R, at + oneL);
                     }
                     const bool evald = r.feature != -2;
                     const bool small = nd.len <= (uint32_t)kSmallNodeRows;
@@ -2586,20 +2618,15 @@ __global__ void __launch_bounds__(32 * kTreeWarps, kTreeSmWarps / kTreeWarps) tr
                     v[4] += (evald && small) ? nd.len : 0u;
                     v[5] += (split && small) ? nd.len : 0u;
                 }
-                // big and small nodes to search, in one scan (halves: at most 2 * kTreeThreads each)
-                const uint32_t nbi = (bigL ? 1u : 0u) + (bigR ? 1u : 0u) + (smallL ? 0x10000u : 0u) + (smallR ? 0x10000u : 0u);
-                uint32_t totb;
-                const uint32_t before = block_incl_scan(nbi, warp_tmp, totb) - nbi;
-                uint32_t bpos = run_big + (before & 0xFFFFu), wpos = run_work + (before >> 16);
-                if (bigL) nbig[AIWCRF_IDX(bpos++, a.big_cap, kBoundOut)] = (uint16_t)(2u * loc);
-                if (bigR) nbig[AIWCRF_IDX(bpos, a.big_cap, kBoundOut)] = (uint16_t)(2u * loc + 1u);
-                if (smallL) work[AIWCRF_IDX(wpos++, a.ecap, kBoundOut)] = L;
-                if (smallR) work[AIWCRF_IDX(wpos, a.ecap, kBoundOut)] = R;
-                run_split += tot;
-                run_big += totb & 0xFFFFu;
-                run_work += totb >> 16;
+                run += tot;
             }
-            if (tid == 0) { s_nb[p ^ 1] = run_big; s_nw = run_work; s_next = kTreeWarps; }
+            const uint32_t run_split = (uint32_t)run & 0xFFFFu;
+            if (tid == 0) {
+                s_nb[p ^ 1] = (uint32_t)(run >> 16) & 0xFFFFu;
+                s_nw[0] = (uint32_t)(run >> 32) & 0xFFFFu;
+                s_nw[1] = (uint32_t)(run >> 48);
+                s_next = kTreeWarps;
+            }
             base += C;
             C = 2u * run_split;
             ++depth;
@@ -2650,8 +2677,8 @@ TreeKernel tree_kernel(int warps)
 
 // Warps per tree: as many as leave every tree a place on the chip at once, since a tree is a serial
 // chain of depths that more warps shorten, while trees side by side fill an SM as well with 8 warps
-// each. Measured, tree kernel at 8 / 16 / 32 warps: 128 trees of 2,220 rows 1,211 / 836 / 711 us; 500
-// trees of 2,220 groups 2,515 / 2,820 / 3,515 us.
+// each. Measured, tree kernel at 8 / 16 / 32 warps: 128 trees of 2,220 rows 1,006 / 670 / 558 us; 500
+// trees of 2,220 groups 2,250 / 2,489 / 2,963 us.
 int tree_warps(int64_t T, int sms)
 {
     return T <= sms ? 32 : T <= 2 * (int64_t)sms ? 16 : 8;

@@ -143,6 +143,35 @@ __device__ __forceinline__ uint32_t block_incl_scan(uint32_t v, uint32_t *warp_t
     return x + off;
 }
 
+// the same for 64-bit values (fields side by side); warp_tmp: one per warp
+__device__ __forceinline__ unsigned long long block_incl_scan64(unsigned long long v, unsigned long long *warp_tmp,
+                                                                unsigned long long &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    unsigned long long x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += t;
+    }
+    if (lane == 31) warp_tmp[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        unsigned long long w = lane < nw ? warp_tmp[lane] : 0ull;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(kFull, w, o);
+            if (lane >= o) w += t;
+        }
+        if (lane < nw) warp_tmp[lane] = w;
+    }
+    __syncthreads();
+    const unsigned long long off = warp > 0 ? warp_tmp[warp - 1] : 0ull;
+    total = warp_tmp[nw - 1];
+    __syncthreads();
+    return x + off;
+}
+
 // ------------------------------------------------------------------------------------------
 // Split candidates. Within a node (n = sum w, S = sum w*y) the CART gain of "left = ranks <= r"
 // is G = S_L^2/n_L + S_R^2/n_R = S^2/n + delta^2 / (n n_L n_R), delta = n S_L - n_L S.
