@@ -31,6 +31,7 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -1177,7 +1178,7 @@ inline int big_bin_cap(int mtry, int F, uint32_t max_card)
 //    winning feature's list, whose first lenL words are the left side; a bit and a prefix count give an
 //    entry's side and place, for the entries and in every list.
 // 500 trees of 111,000 rows with 32 features of as many values, 10 tried (666 million entries searched):
-// draw 1.7 ms, search 44, split 66, beside 50 of level_small_kernel. One CTA per node, four warps over its
+// draw 1.7 ms, search 44, split 60, beside 50 of level_small_kernel. One CTA per node, four warps over its
 // features with a rank gathered beside each entry, and a second kernel over all lists took 128 and 125 ms;
 // the lists are 134 GB of reads and writes, 20 ms of memory time.
 constexpr int kListWarps = 8;            // of a CTA of the warp-per-item kernels
@@ -1428,8 +1429,9 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_huge
 // carries each into the side's next word (and out of the top into the next step). needL / needR: whether
 // the child will search its lists (otherwise its words are not written: a child of at most 32 entries is
 // searched from the entries, a stopping one not at all). The next words, of this feature or the next, are
-// on their way while these are placed.
-constexpr int kPartIlp = 4;
+// on their way while these are placed. 256 words a step, whole steps without their bounds tests: the splits
+// of 500 trees of 111,000 rows take 62 ms, 68 with 128 words and every test.
+constexpr int kPartIlp = 8;
 template <typename Place>
 __device__ __forceinline__ void list_partition(const LevelArgs &a, const NodeRec &nd, int f0, int df, uint32_t lenL,
                                                bool needL, bool needR, const Place &place)
@@ -1450,30 +1452,37 @@ __device__ __forceinline__ void list_partition(const LevelArgs &a, const NodeRec
     uint32_t *__restrict__ Lo = a.lists_out + (size_t)f0 * (size_t)a.list_stride + tb;
     const size_t stride = (size_t)df * (size_t)a.list_stride;
     load(Li, 0u, p);
+    uint32_t rl, cl, cr;                           // words left so far; a break pending for either side (or no word yet)
+    auto put = [&](auto whole, uint32_t b0, const uint32_t (&x)[kPartIlp], const uint32_t (&d)[kPartIlp]) {
+        constexpr bool kWhole = decltype(whole)::value;            // every lane of the step holds a word
+#pragma unroll
+        for (int u = 0; u < kPartIlp; ++u) {
+            const uint32_t s0 = b0 + 32u * u, i = s0 + (uint32_t)lane;
+            if (!kWhole && s0 >= nd.len) break;                     // warp-uniform
+            const bool valid = kWhole || i < nd.len, left = valid && (d[u] & kListBreak);
+            const uint32_t bl = __ballot_sync(kFull, left), br = kWhole ? ~bl : __ballot_sync(kFull, valid) & ~bl;
+            const uint32_t bk = __ballot_sync(kFull, valid && (x[u] & kListBreak));
+            const uint64_t sl = (uint64_t)(~bl) + (bk & ~bl) + cl, sr = (uint64_t)(~br) + (bk & ~br) + cr;
+            cl = (uint32_t)(sl >> 32);
+            cr = (uint32_t)(sr >> 32);
+            const uint32_t brk = ((left ? (uint32_t)sl : (uint32_t)sr) | bk) >> lane << 31;
+            const uint32_t nl = rl + (uint32_t)__popc(bl & lt);
+            if (valid && (left ? needL : needR))
+                Lo[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)] = (d[u] & kListPos) | brk;
+            rl += (uint32_t)__popc(bl);
+        }
+    };
     for (int f = f0; f < a.F; f += df, Lo += stride) {
-        uint32_t rl = 0u, cl = 1u, cr = 1u;        // words left so far; a break pending for either side (or no word yet)
+        rl = 0u;
+        cl = cr = 1u;
         for (uint32_t b0 = 0; b0 < nd.len; b0 += 32u * kPartIlp) {
             if (b0 + 32u * kPartIlp < nd.len) load(Li, b0 + 32u * kPartIlp, pn);
             else if (f + df < a.F) { Li += stride; load(Li, 0u, pn); }
             uint32_t d[kPartIlp];
 #pragma unroll
             for (int u = 0; u < kPartIlp; ++u) d[u] = place(AIWCRF_IDX(p[u] & kListPos, nd.len, kBoundOut));
-#pragma unroll
-            for (int u = 0; u < kPartIlp; ++u) {
-                const uint32_t s0 = b0 + 32u * u, i = s0 + (uint32_t)lane;
-                if (s0 >= nd.len) break;                            // warp-uniform
-                const bool valid = i < nd.len, left = valid && (d[u] & kListBreak);
-                const uint32_t bl = __ballot_sync(kFull, left), br = __ballot_sync(kFull, valid) & ~bl;
-                const uint32_t bk = __ballot_sync(kFull, valid && (p[u] & kListBreak));
-                const uint64_t sl = (uint64_t)(~bl) + (bk & ~bl) + cl, sr = (uint64_t)(~br) + (bk & ~br) + cr;
-                cl = (uint32_t)(sl >> 32);
-                cr = (uint32_t)(sr >> 32);
-                const uint32_t brk = ((left ? (uint32_t)sl : (uint32_t)sr) | bk) >> lane << 31;
-                const uint32_t nl = rl + (uint32_t)__popc(bl & lt);
-                if (valid && (left ? needL : needR))
-                    Lo[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)] = (d[u] & kListPos) | brk;
-                rl += (uint32_t)__popc(bl);
-            }
+            if (b0 + 32u * kPartIlp <= nd.len) put(std::true_type{}, b0, p, d);
+            else put(std::false_type{}, b0, p, d);
 #pragma unroll
             for (int u = 0; u < kPartIlp; ++u) p[u] = pn[u];
         }
