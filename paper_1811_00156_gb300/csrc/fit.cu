@@ -16,6 +16,8 @@
 //     level_big_kernel   one CTA per node with > 32 entries: mtry draw, shared-memory histogram
 //                        (sum w, sum w*y) per rank of every tried feature, block scan, exact
 //                        argmax of the gain, stable partition of the entries
+//                        (list_draw / search / split kernels instead where a column has more than
+//                        kListMinCard values: the entries kept sorted by every feature)
 //     level_small_kernel one warp per node with <= 32 entries: the same search with a register
 //                        bitonic sort per feature instead of a histogram (runs concurrently with
 //                        level_big_kernel; both count each tile's splits)
@@ -23,7 +25,10 @@
 //                        children breadth first, writes the next depth's node table and its
 //                        warp/CTA work lists; its last CTA advances the per-tree node counts,
 //                        next-depth offsets and level counts
-//   pack_kernel        scatters every finished node to its forest / tree / BFS position
+//   tree_grow_kernel   instead of the depths' kernels where a tree's entries fit in shared memory: one
+//                      CTA grows a tree through all its depths
+//   pack_kernel, forest_place_kernel, forest_values_kernel   the finished nodes to their forest / tree /
+//                      BFS positions, the padding, the compact form and the value tables
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -958,20 +963,26 @@ __device__ __forceinline__ void small_node(const LevelArgs &a, const RT *__restr
         if (__all_sync(kFull, !live || rank == rank0)) continue;
         uint32_t key = (rank << 5) | (uint32_t)pos;                  // unique within a segment
         // bitonic sort of the keys within each segment, ascending; the low five bits name the
-        // entry's lane, whose w and w*y are fetched once the order is known
-        for (int k = 2; k <= K; k <<= 1) {
+        // entry's lane, whose w and w*y are fetched once the order is known (unrolled, with a way out at
+        // K: the loops over run-time widths took 57 against 51 ms, 500 trees of 111,000 distinct rows)
+#pragma unroll
+        for (int k = 2; k <= 32; k <<= 1) {
+            if (k > K) break;
+#pragma unroll
             for (int jj = k >> 1; jj > 0; jj >>= 1) {
                 const uint32_t ok = __shfl_xor_sync(kFull, key, jj);
-                const bool asc = (pos & k) == 0;
-                const bool lower = (pos & jj) == 0;
-                key = ((lower == asc) ? (ok < key) : (ok > key)) ? ok : key;
+                const bool up = ((pos & k) == 0) == ((pos & jj) == 0);
+                const uint32_t mn = min(ok, key), mx = max(ok, key);
+                key = up ? mn : mx;
             }
         }
         const int src = (lane & ~(K - 1)) | (int)(key & 31u);
         const uint32_t r = key >> 5;
         uint32_t cw = __shfl_sync(kFull, live ? e.w : 0u, src);
         long long cs = __shfl_sync(kFull, live ? (long long)e.wy : 0ll, src);
-        for (int o = 1; o < K; o <<= 1) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            if (o >= K) break;
             const uint32_t tw = __shfl_up_sync(kFull, cw, o);
             const long long ts = __shfl_up_sync(kFull, cs, o);
             if (pos >= o) { cw += tw; cs += ts; }
@@ -1178,7 +1189,7 @@ inline int big_bin_cap(int mtry, int F, uint32_t max_card)
 //    winning feature's list, whose first lenL words are the left side; a bit and a prefix count give an
 //    entry's side and place, for the entries and in every list.
 // 500 trees of 111,000 rows with 32 features of as many values, 10 tried (666 million entries searched):
-// draw 1.7 ms, search 44, split 60, beside 50 of level_small_kernel. One CTA per node, four warps over its
+// draw 1.7 ms, search 45, split 60, beside 45 of level_small_kernel. One CTA per node, four warps over its
 // features with a rank gathered beside each entry, and a second kernel over all lists took 128 and 125 ms;
 // the lists are 134 GB of reads and writes, 20 ms of memory time.
 constexpr int kListWarps = 8;            // of a CTA of the warp-per-item kernels
