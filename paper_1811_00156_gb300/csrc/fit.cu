@@ -1180,14 +1180,17 @@ inline int big_bin_cap(int mtry, int F, uint32_t max_card)
 // entry) and issue slots, so a node is a warp's work, without block barriers, unless it is large:
 //  - list_draw_kernel, a warp per node: its tried features; nodes of more than kWarpNode entries are
 //    listed for the CTA forms of the other two.
-//  - list_search_kernel, a warp per (node, tried feature), or a CTA above kCtaSearch entries: consecutive
+//  - list_search_kernel, a warp per (node, tried feature), or a CTA above list_cta_search entries: consecutive
 //    items share a node, so its entries (1.1 MB at a root of 70,000) are in L2 while its features are
 //    searched. With a warp per item at the root, 500 trees' entries were in use at once, 7.7 ms of that
 //    depth; a CTA per item takes 2.2.
 //  - list_split_kernel, a warp per node, or CTAs: the best of its features' candidates, the entries' stable
 //    partition and that of every feature's list. Which entries go left is a bit set, filled from the
 //    winning feature's list, whose first lenL words are the left side; a bit and a prefix count give an
-//    entry's side and place, for the entries and in every list.
+//    entry's side and place, for the entries and in every list. A depth with fewer nodes than warps gives
+//    each node several.
+// Each of the two is one launch, CTA form first: as launches of their own, and with a warp a node at every
+// depth, 60 trees of 4,440 rows took 4.2 ms, 20 of 44,400 8.4; this 2.9 and 7.1.
 // 500 trees of 111,000 rows with 32 features of as many values, 10 tried (666 million entries searched):
 // draw 1.7 ms, search 45, split 60, beside 45 of level_small_kernel. One CTA per node, four warps over its
 // features with a rank gathered beside each entry, and a second kernel over all lists took 128 and 125 ms;
@@ -1216,6 +1219,7 @@ struct ListArgs {
     int m;                        // tried features of a node
     int32_t *huge;                // nodes for the CTA form
     uint32_t *n_huge;             // their number, by depth parity
+    uint32_t warps;               // of a full grid of the search and split kernels
 };
 
 __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_draw_kernel(LevelArgs a, ListArgs l)
@@ -1392,35 +1396,25 @@ __device__ __forceinline__ Cand list_search(const LevelArgs &a, const ListNode &
     return warp_best(best, nd.n, nd.S);
 }
 
-__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_kernel(LevelArgs a, ListArgs l)
+// Entries of a node above which a CTA searches a feature, 1,024 words a step: fewer while the depth has not
+// an item for every warp.
+__device__ __forceinline__ uint32_t list_cta_search(const ListArgs &l, uint32_t list_n)
 {
-    const uint32_t list_n = *a.list_n, m = (uint32_t)l.m, step = gridDim.x * kListWarps;
-    const uint32_t first = blockIdx.x * kListWarps + (threadIdx.x >> 5), dk = step / m, dq = step - dk * m;
-    uint32_t k = first / m, q = first - k * m;
-    while (k < list_n) {
-        const ListNode nd = l.node[k];
-        if (nd.len != 0u && nd.len <= kCtaSearch) {
-            const size_t at = (size_t)k * m + q;
-            const Cand c = list_search<1>(a, nd, l.feat[at], 0, nullptr);
-            if ((threadIdx.x & 31) == 0) l.cand[at] = c;
-        }
-        k += dk;
-        q += dq;
-        if (q >= m) { q -= m; ++k; }
-    }
+    return (uint64_t)list_n * (uint32_t)l.m <= l.warps ? kWarpNode : kCtaSearch;
 }
 
-// The same by a CTA per (node, tried feature), for nodes of more than kCtaSearch entries: 1,024 words a step.
-__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_huge_kernel(LevelArgs a, ListArgs l)
+// first the CTAs' items, then the warps'
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_kernel(LevelArgs a, ListArgs l)
 {
     __shared__ ListTotals tot;
     __shared__ Cand cands[kListWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t n = l.n_huge[level_depth(a) & 1], m = (uint32_t)l.m;
+    const uint32_t list_n = *a.list_n, m = (uint32_t)l.m, above = list_cta_search(l, list_n);
+    const uint32_t n = l.n_huge[level_depth(a) & 1];
     for (uint32_t it = blockIdx.x; it < n * m; it += gridDim.x) {
         const uint32_t k = (uint32_t)l.huge[it / m];
         const ListNode nd = l.node[k];
-        if (nd.len <= kCtaSearch) continue;                        // block-uniform
+        if (nd.len <= above) continue;                             // block-uniform
         const size_t at = (size_t)k * m + it % m;
         const Cand c = list_search<kListWarps>(a, nd, l.feat[at], warp, &tot);
         if (lane == 0) cands[warp] = c;
@@ -1430,6 +1424,19 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_search_huge
             if (lane == 0) l.cand[at] = b;
         }
         __syncthreads();
+    }
+    const uint32_t step = gridDim.x * kListWarps, first = blockIdx.x * kListWarps + (uint32_t)warp, dk = step / m, dq = step - dk * m;
+    uint32_t k = first / m, q = first - k * m;
+    while (k < list_n) {
+        const ListNode nd = l.node[k];
+        if (nd.len != 0u && nd.len <= above) {
+            const size_t at = (size_t)k * m + q;
+            const Cand c = list_search<1>(a, nd, l.feat[at], 0, nullptr);
+            if (lane == 0) l.cand[at] = c;
+        }
+        k += dk;
+        q += dq;
+        if (q >= m) { q -= m; ++k; }
     }
 }
 
@@ -1533,20 +1540,27 @@ __device__ __forceinline__ void write_list_split(const LevelArgs &a, int j, cons
     atomicAdd(&a.tile_splits[(uint32_t)j / (uint32_t)kScanTile], 1u);
 }
 
+struct ListWarpNodes {            // shared memory of the warp form
+    uint32_t bits[kListWarps][32];
+    uint16_t dest[kListWarps][kWarpNode];
+};
+
+// The warp form. While the depth has fewer nodes than warps, several warps take a node, each a share of its
+// features (the first also the entries).
 template <typename RT>
-__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kernel(LevelArgs a, ListArgs l)
+__device__ __forceinline__ void list_split_warps(const LevelArgs &a, const ListArgs &l, ListWarpNodes &sh)
 {
-    __shared__ uint32_t bits_s[kListWarps][32];
-    __shared__ uint16_t dest_s[kListWarps][kWarpNode];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t list_n = *a.list_n, step = gridDim.x * kListWarps, lt = lanemask_lt();
-    for (uint32_t k = blockIdx.x * kListWarps + warp; k < list_n; k += step) {
+    const uint32_t parts = max(1u, min((uint32_t)a.F, l.warps / max(list_n, 1u)));
+    for (uint32_t it = blockIdx.x * kListWarps + warp; it < list_n * parts; it += step) {
+        const uint32_t k = it / parts, part = it - k * parts;
         const int j = AIWCRF_IDX(a.list[k], a.node_cap, kBoundNode);
         const NodeRec nd = a.nodes[j];
         if (nd.len > kWarpNode || node_stops(a, nd)) continue;
         const Cand c = list_winner(a, l, k, nd);
         if (c.h < 0.0f) {
-            if (lane == 0) write_leaf(a.res, j, -1, 0);
+            if (part == 0u && lane == 0) write_leaf(a.res, j, -1, 0);
             continue;
         }
         const size_t tb = (size_t)nd.tree * (size_t)a.row_cap + nd.start;
@@ -1554,14 +1568,17 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kerne
         Entry *__restrict__ rout = a.rows_out + tb;
         const uint32_t *__restrict__ L = a.lists_in + (size_t)c.f * (size_t)a.list_stride + tb;
         const uint32_t lenL = c.r + 1u;
-        bits_s[warp][lane] = 0u;
+        const bool needL = needs_lists(a, lenL, c.nL), needR = needs_lists(a, nd.len - lenL, nd.n - c.nL);
+        if (part != 0u && !needL && !needR) continue;
+        uint32_t (&bits_s)[32] = sh.bits[warp];
+        bits_s[lane] = 0u;
         __syncwarp();
         for (uint32_t i = (uint32_t)lane; i < lenL; i += 32u) {
             const uint32_t p = AIWCRF_IDX(__ldg(&L[i]) & kListPos, nd.len, kBoundOut);
-            atomicOr(&bits_s[warp][p >> 5], 1u << (p & 31u));
+            atomicOr(&bits_s[p >> 5], 1u << (p & 31u));
         }
         __syncwarp();
-        const uint32_t bits = bits_s[warp][lane];
+        const uint32_t bits = bits_s[lane];
         uint32_t before = __popc(bits);                             // entries of the earlier words that go left
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1569,13 +1586,13 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kerne
             if (lane >= o) before += t;
         }
         before -= __popc(bits);
-        uint16_t *dest = dest_s[warp];                              // place within the child; top bit: left
+        uint16_t *dest = sh.dest[warp];                              // place within the child; top bit: left
         for (uint32_t w0 = 0; 32u * w0 < nd.len; w0 += 4u) {        // four words of entries in flight
             Entry e[4];
 #pragma unroll
             for (uint32_t u = 0; u < 4u; ++u) {
                 const uint32_t i = 32u * (w0 + u) + (uint32_t)lane;
-                if (i < nd.len) e[u] = load_entry(rin + i);
+                if (part == 0u && i < nd.len) e[u] = load_entry(rin + i);
             }
 #pragma unroll
             for (uint32_t u = 0; u < 4u; ++u) {
@@ -1584,20 +1601,19 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kerne
                 const uint32_t nl = __shfl_sync(kFull, before, (int)(w0 + u) & 31) + __popc(bw & lt);
                 if (i < nd.len) {
                     const bool left = (bw >> lane) & 1u;
-                    store_entry(&rout[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)], e[u]);
+                    if (part == 0u) store_entry(&rout[AIWCRF_IDX(left ? nl : lenL + i - nl, nd.len, kBoundOut)], e[u]);
                     dest[i] = (uint16_t)(left ? nl | 0x8000u : i - nl);
                 }
             }
         }
-        const bool needL = needs_lists(a, lenL, c.nL), needR = needs_lists(a, nd.len - lenL, nd.n - c.nL);
         if (needL || needR) {
             __syncwarp();
-            list_partition(a, nd, 0, 1, lenL, needL, needR, [&](uint32_t p) {
+            list_partition(a, nd, (int)part, (int)parts, lenL, needL, needR, [&](uint32_t p) {
                 const uint32_t d = dest[p];
                 return (d & 0x8000u) << 16 | (d & 0x7FFFu);
             });
         }
-        if (lane == 0) write_list_split<RT>(a, j, c, L, rin);
+        if (part == 0u && lane == 0) write_list_split<RT>(a, j, c, L, rin);
         __syncwarp();
     }
 }
@@ -1607,13 +1623,18 @@ __global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kerne
 // kCtaNodeWords entries has no room there: its entries' new positions go to a.newpos instead.
 // kHugeParts CTAs take one node, each a share of its features (the first also the entries): 500 roots of
 // 70,000 entries are then 2,000 items for 608 resident CTAs.
-constexpr int kHugeThreads = 256, kHugeParts = 4, kHugeCtasPerSm = 4;
+constexpr int kHugeThreads = kListThreads, kHugeParts = 4;
+struct ListCtaNode {              // shared memory of the CTA form
+    uint2 bits[kCtaNodeWords];    // a word, entries of the earlier words that go left
+    uint32_t warp_tmp[32];
+    Cand winner;
+};
+
 template <typename RT>
-__global__ void __launch_bounds__(kHugeThreads, kHugeCtasPerSm) list_split_huge_kernel(LevelArgs a, ListArgs l)
+__device__ __forceinline__ void list_split_ctas(const LevelArgs &a, const ListArgs &l, ListCtaNode &sh)
 {
-    __shared__ uint2 bits[kCtaNodeWords];                           // a word, entries of the earlier words that go left
-    __shared__ uint32_t warp_tmp[32];
-    __shared__ Cand winner;
+    uint2 *bits = sh.bits;
+    uint32_t *warp_tmp = sh.warp_tmp;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t n = l.n_huge[level_depth(a) & 1];
     for (uint32_t h = blockIdx.x; h < n * kHugeParts; h += gridDim.x) {
@@ -1625,10 +1646,10 @@ __global__ void __launch_bounds__(kHugeThreads, kHugeCtasPerSm) list_split_huge_
         __syncthreads();                                            // the node before is done with shared memory
         if (warp == 0) {
             const Cand c = list_winner(a, l, k, nd);
-            if (lane == 0) winner = c;
+            if (lane == 0) sh.winner = c;
         }
         __syncthreads();
-        const Cand c = winner;
+        const Cand c = sh.winner;
         if (c.h < 0.0f) {
             if (first && tid == 0) write_leaf(a.res, j, -1, 0);
             continue;                                               // block-uniform
@@ -1705,6 +1726,20 @@ __global__ void __launch_bounds__(kHugeThreads, kHugeCtasPerSm) list_split_huge_
         }
         if (first && tid == 0) write_list_split<RT>(a, j, c, L, rin);
     }
+}
+
+// first the large nodes by CTAs, then the others by warps
+template <typename RT>
+__global__ void __launch_bounds__(kListThreads, kListCtasPerSm) list_split_kernel(LevelArgs a, ListArgs l)
+{
+    __shared__ union Shared {
+        ListCtaNode cta;
+        ListWarpNodes warps;
+        __device__ Shared() {}
+    } sh;
+    list_split_ctas<RT>(a, l, sh.cta);
+    __syncthreads();
+    list_split_warps<RT>(a, l, sh.warps);
 }
 
 // One CTA per node with more than 32 entries. Shared bins, bin_cap of them, hold per rank
@@ -3834,22 +3869,16 @@ int fit_batch(const aiwcrf_fit_params &p, const float *dX, const int64_t *dy, in
                 if (use_lists) {
                     // warps per node and per (node, feature); a depth has at most Cb nodes in its list
                     const int64_t cps = p.ctas_per_sm > 0 ? p.ctas_per_sm : kListCtasPerSm;
-                    auto warps = [&](int64_t items) {
-                        return (unsigned)std::max<int64_t>(1, std::min<int64_t>((items + kListWarps - 1) / kListWarps, cps * dev_sms));
-                    };
-                    list_draw_kernel<<<warps(Cb), kListThreads, 0, s>>>(la, ll);
+                    ll.warps = (uint32_t)(cps * dev_sms * kListWarps);
+                    const unsigned all = (unsigned)(cps * dev_sms);
+                    list_draw_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((Cb + kListWarps - 1) / kListWarps, all)),
+                                       kListThreads, 0, s>>>(la, ll);
                     AIWCRF_LAUNCH_CHECK("list_draw_kernel");
-                    list_search_kernel<<<warps(Cb * ll.m), kListThreads, 0, s>>>(la, ll);
+                    list_search_kernel<<<all, kListThreads, 0, s>>>(la, ll);
                     AIWCRF_LAUNCH_CHECK("list_search_kernel");
-                    list_search_huge_kernel<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb * ll.m, cps * dev_sms)),
-                                              kListThreads, 0, s>>>(la, ll);
-                    AIWCRF_LAUNCH_CHECK("list_search_huge_kernel");
                     prof_end(s, kProfLevelBig);
                     prof_begin(s, kProfListPart);
-                    const unsigned hgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(Cb * kHugeParts, std::min<int64_t>(cps, kHugeCtasPerSm) * dev_sms));
-                    AIWCRF_BY_RANK(rank_bytes, list_split_huge_kernel<RT><<<hgrid, kHugeThreads, 0, s>>>(la, ll))
-                    AIWCRF_LAUNCH_CHECK("list_split_huge_kernel");
-                    AIWCRF_BY_RANK(rank_bytes, list_split_kernel<RT><<<warps(Cb), kListThreads, 0, s>>>(la, ll))
+                    AIWCRF_BY_RANK(rank_bytes, list_split_kernel<RT><<<all, kListThreads, 0, s>>>(la, ll))
                     AIWCRF_LAUNCH_CHECK("list_split_kernel");
                     prof_end(s, kProfListPart);
                 } else {
