@@ -155,13 +155,31 @@ __device__ __forceinline__ void code_columns(int nf, const float *__restrict__ f
             tab[u] = fvals + (size_t)(f < nf ? f : 0) * (size_t)fstride;
             pos[u] = 0u;
         }
-        // lower bound by halving powers of two: pos + bit values are below x if the last of
-        // them is (tables are sorted; a position past the table, or a NaN, never is)
-        for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
+        if constexpr (sizeof(CT) == 1) {
+            // lower bound by halving powers of two: pos + bit values are below x if the last of
+            // them is (tables are sorted; a position past the table, or a NaN, never is)
+            for (uint32_t bit = 1u << (steps - 1); bit; bit >>= 1) {
 #pragma unroll
-            for (int u = 0; u < kCodeGroup; ++u) {
-                const uint32_t at = pos[u] + bit;
-                if (at <= n[u] && __ldg(&tab[u][at - 1]) < x[u]) pos[u] = at;
+                for (int u = 0; u < kCodeGroup; ++u) {
+                    const uint32_t at = pos[u] + bit;
+                    if (at <= n[u] && __ldg(&tab[u][at - 1]) < x[u]) pos[u] = at;
+                }
+            }
+        } else {
+            // larger tables (over 255 values): halves of what is left, whose probes spread over L1's sets;
+            // those at powers of two meet in a few. 700,000 queries x 32 columns of 6,660 values 434 ->
+            // 325 us, 400,000 of 111,000 values 810 -> 355; small tables are faster the other way.
+            uint32_t len[kCodeGroup];
+#pragma unroll
+            for (int u = 0; u < kCodeGroup; ++u) len[u] = n[u];
+            for (int it = 0; it < steps; ++it) {
+#pragma unroll
+                for (int u = 0; u < kCodeGroup; ++u) {
+                    const uint32_t half = len[u] >> 1;
+                    const bool below = len[u] != 0u && __ldg(&tab[u][pos[u] + half]) < x[u];
+                    pos[u] += below ? half + 1u : 0u;
+                    len[u] = below ? len[u] - half - 1u : half;
+                }
             }
         }
 #pragma unroll
