@@ -333,7 +333,8 @@ __device__ __forceinline__ void walk_tree(NodePtr tn, const CT *const (&xr)[QPT]
 // queries; with more than one part, each CTA adds its queries' partial sums (and sums of squares)
 // into sum / sq, and the last CTA of a tile to arrive (ticket) writes the results: exact integers,
 // so the order does not matter. sum, sq and ticket are zero on entry (the coding kernel clears
-// them). A square sum is kept as its low 32 bits' sum and the rest's, which 64 bits hold.
+// them). A square sum keeps all its 128 bits, as an unsplit walk's does: the low words are added first,
+// and whoever's addition wraps carries into the high word.
 // Adding costs the last CTA one read per query; summing the parts' separate sums there instead
 // took 35 us of a 2,220-query call with 128 parts.
 struct TreeParts {
@@ -379,8 +380,8 @@ __device__ __forceinline__ void finish_tile(const TreeParts &tp, int64_t (&acc)[
             const size_t k = (size_t)q0 + (size_t)(tid + i * kPredThreads);
             atomicAdd(&tp.sum[k], (unsigned long long)acc[i]);
             if (VAR) {
-                atomicAdd(&tp.sq[2 * k], (unsigned long long)(uint32_t)sq[i]);
-                atomicAdd(&tp.sq[2 * k + 1], (unsigned long long)(sq[i] >> 32));
+                const unsigned long long lo = (unsigned long long)sq[i], was = atomicAdd(&tp.sq[2 * k], lo);
+                atomicAdd(&tp.sq[2 * k + 1], (unsigned long long)(sq[i] >> 64) + (was + lo < lo ? 1ull : 0ull));
             }
         }
         __threadfence();
@@ -393,7 +394,7 @@ __device__ __forceinline__ void finish_tile(const TreeParts &tp, int64_t (&acc)[
         for (int i = 0; i < QPT; ++i) {
             const size_t k = (size_t)q0 + (size_t)(tid + i * kPredThreads);
             acc[i] = (int64_t)__ldcg(&tp.sum[k]);
-            if (VAR) sq[i] = (u128_t)__ldcg(&tp.sq[2 * k]) + ((u128_t)__ldcg(&tp.sq[2 * k + 1]) << 32);
+            if (VAR) sq[i] = (u128_t)__ldcg(&tp.sq[2 * k]) | ((u128_t)__ldcg(&tp.sq[2 * k + 1]) << 64);
         }
     }
 #pragma unroll
