@@ -1033,11 +1033,11 @@ __global__ void argmin_kernel(const int64_t *pred, DeviceIds dev, int32_t K, int
     const int32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K) return;
     int64_t bp = 0;
-    int32_t bd = -1;
+    int32_t bd = 0;
     for (int32_t jd = 0; jd < D; ++jd) {
         const int64_t p = pred[(size_t)k * (size_t)D + jd];
         if (out_pred) out_pred[(size_t)k * (size_t)D + jd] = p;
-        if (bd < 0 || p < bp || (p == bp && dev[jd] < bd)) { bp = p; bd = dev[jd]; }
+        if (jd == 0 || p < bp || (p == bp && dev[jd] < bd)) { bp = p; bd = dev[jd]; }   // any id, negative ones too
     }
     best[k] = bd;
 }
