@@ -211,6 +211,18 @@ PtrKind classify(const void *p, int device)
     }
 }
 
+// Pageable host memory: CUDA stages a copy from it while the call is made, so that reading it then is the
+// same. Page-locked memory is read when the stream gets there: its earlier work may still be filling it.
+bool pageable_host(const void *p)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return at.type == cudaMemoryTypeUnregistered;
+}
+
 // An input array: device pointers pass through; host arrays are copied to a stream-ordered
 // device buffer.
 struct InArg {
@@ -664,9 +676,10 @@ int aiwcrf_select_device(const aiwcrf_forest *forest, const float *kfeat, int32_
     InArg ak, ad;
     OutArg ob, op;
     if ((rc = stage_in(ak, kfeat, sizeof(float) * (size_t)(forest->F - 2) * (size_t)n_kernels, dev, s, "kfeat"))) return rc;
-    // a host array of a few ids travels with the launches
+    // a few ids in pageable memory are read now and travel with the launches; others are copied in stream
+    // order, as every input
     DeviceIds ids;
-    if (n_devices <= kSelectMaxDevices && classify(device_ids, dev) == kPtrHost) {
+    if (n_devices <= kSelectMaxDevices && pageable_host(device_ids)) {
         std::memcpy(ids.id, device_ids, sizeof(int32_t) * (size_t)n_devices);
     } else {
         if ((rc = stage_in(ad, device_ids, sizeof(int32_t) * (size_t)n_devices, dev, s, "device_ids"))) return rc;

@@ -1,4 +1,5 @@
-"""Device ids of a selection: negative ones on every route."""
+"""Device ids of a selection: negative ones on every route, and page-locked ids that earlier work of
+the call's stream writes."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,30 @@ def test_negative_device_ids(K, ids):
     rp = ref.select_device(kf, 1, ids)[1]
     assert np.array_equal(pred.cpu().numpy(), rp)
     assert np.array_equal(best.cpu().numpy(), fastest(rp, ids))
+
+
+@pytest.mark.parametrize("K", [3, 20000])
+def test_page_locked_ids_are_read_in_stream_order(K):
+    """Host inputs are copied on the call's stream: ids that the stream's earlier work writes into
+    page-locked memory are the ones that count."""
+    gpu, ref = forests()
+    kf = np.random.default_rng(K).normal(0.0, 3.0, (3, K)).astype(np.float32)
+    dk = torch.from_numpy(kf).cuda()
+    old, new = [0, 1, 2, 3], [9, -2, 6, 4]
+    ids = torch.tensor(old, dtype=torch.int32).pin_memory()
+    dnew = torch.tensor(new, dtype=torch.int32, device="cuda")
+    best = torch.full((K,), -9, dtype=torch.int32, device="cuda")
+    pred = torch.empty(K, 4, dtype=torch.int64, device="cuda")
+    big = torch.randn(4096, 4096, device="cuda")
+    A.aiwcrf_select_device(gpu, dk, 1, old, best, pred)             # everything is loaded
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        for _ in range(20):                                         # some milliseconds before the ids are written
+            big = big @ big * 1e-4
+        ids.copy_(dnew, non_blocking=True)
+        A.aiwcrf_select_device(gpu, dk, 1, ids.numpy(), best, pred)
+    torch.cuda.synchronize()
+    rp = ref.select_device(kf, 1, new)[1]
+    assert np.array_equal(pred.cpu().numpy(), rp)
+    assert np.array_equal(best.cpu().numpy(), fastest(rp, new))
