@@ -279,11 +279,7 @@ __device__ __forceinline__ void stage_weights(unsigned char *dst, const bf16 *__
 // the tile's 128 x 64 accumulator columns [16 group, 16 group + 16) of this thread's row
 __device__ __forceinline__ void train_acc(uint32_t tbase, int q4, int group, float (&x)[16])
 {
-    uint32_t v[16];
-    tc::tmem_start16(tbase + ((uint32_t)(32 * q4) << 16) + 16u * group, v);
-    tc::tmem_wait16(v);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
+    tc::tmem_ld16(tbase + ((uint32_t)(32 * q4) << 16) + 16u * group, x);
 }
 
 // CTA (slice, tile): encode the tile's rows, layer 1's columns [64 slice, ...): activations and GELU'.
@@ -954,18 +950,13 @@ __global__ void __launch_bounds__(kInferThreads, 1) surrogate_infer_kernel(
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, parity ^= 1u) {
             const int64_t q0 = tile * 128;
             wait(&bar_x, parity);
-            uint32_t v[16];
-            tc::tmem_start16(mine + 16u * group, v);
 #pragma unroll 1
             for (int c = 0; c < 4; ++c) {   // epilogue 1: bias, GELU, BF16 back into TMEM
                 const uint32_t col0 = 64u * c + 16u * group;
                 const float4 *bias = reinterpret_cast<const float4 *>(b1s + col0);
                 uint32_t w[8];
                 float x[16];
-                tc::tmem_wait16(v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
-                if (c < 3) tc::tmem_start16(mine + col0 + 64u, v);
+                tc::tmem_ld16(mine + col0, x);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float4 b = bias[i];
@@ -979,7 +970,6 @@ __global__ void __launch_bounds__(kInferThreads, 1) surrogate_infer_kernel(
                 arrive(&full_h[c]);
             }
             wait(&bar_h, parity);
-            tc::tmem_start16(mine + 256u + (uint32_t)(kInferCols * group), v);
             uint64_t dot = pack2(0.0f, 0.0f);
 #pragma unroll 1
             for (int c = 0; c < kInferCols / 16; ++c) {     // epilogue 2: bias, GELU, dot with w3
@@ -987,10 +977,7 @@ __global__ void __launch_bounds__(kInferThreads, 1) surrogate_infer_kernel(
                 const float4 *bias = reinterpret_cast<const float4 *>(b2s + col0);
                 const float4 *wt = reinterpret_cast<const float4 *>(w3s + col0);
                 float x[16];
-                tc::tmem_wait16(v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) x[i] = __uint_as_float(v[i]);
-                if (c + 1 < kInferCols / 16) tc::tmem_start16(mine + 256u + (uint32_t)(col0 + 16), v);
+                tc::tmem_ld16(mine + 256u + (uint32_t)col0, x);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const float4 b = bias[i], w = wt[i];
