@@ -126,7 +126,8 @@ __device__ __forceinline__ uint64_t gelu2_layer1(uint64_t x)
 // smooth on [0, 6] that a degree-8 polynomial q (a weighted minimax fit, here in s = -t) gives
 // |2^q - Phi(-t)| <= 7.6e-9; evaluated in FP32 it stays below 4e-8, and the exponential adds at most
 // 2^-22 of a value below 1/2 (formula 7.1.26 leaves 7e-8 on the same scale before rounding). Beyond 6,
-// Phi(-t) < 1e-9 is taken as Phi(-6). One exponential and nine multiply-adds a value. NaN stays NaN.
+// Phi(-t) < 1e-9 is taken as Phi(-6), for minus infinity too (GELU's limit there; x times 1 + erf would be
+// NaN). One exponential and nine multiply-adds a value. NaN stays NaN.
 __device__ __forceinline__ uint64_t gelu2(uint64_t x)
 {
     constexpr float kQ[9] = {-1.0f, 1.1511057615280151f, -0.45920491218566895f, 0.052505023777484894f,
@@ -289,8 +290,8 @@ __global__ void __launch_bounds__(kTrainThreads) train_layer1_kernel(TrainArgs a
     __shared__ __align__(1024) unsigned char sW[kSliceCols * kIn * 2];
     __shared__ __align__(8) uint64_t bar_c, bar_m;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
-    const int64_t tile = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
+    const int64_t tile = blockIdx.x / kSlices;
     train_begin(&bar_c, &bar_m, &tmem_base, 64);
     {   // thread (row, part) encodes inputs [8 part, 8 part + 8) and [32 + 8 part, ...) of one row; the
         // row's values are loaded together before any is used
@@ -370,8 +371,8 @@ __global__ void __launch_bounds__(kTrainThreads) train_layer2_kernel(TrainArgs a
     unsigned char *sH = sm, *sW = sm + kTileH;
     __shared__ __align__(8) uint64_t bar_c, bar_m;
     __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
-    const int64_t tile = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
+    const int64_t tile = blockIdx.x / kSlices;
     train_begin(&bar_c, &bar_m, &tmem_base, 64);
     if (tid == 0) {
         tc::mbar_expect(&bar_c, kTileH);
@@ -439,8 +440,8 @@ __global__ void __launch_bounds__(kTrainThreads) train_back_kernel(TrainArgs a)
     __shared__ __align__(8) uint64_t bar_c, bar_m;
     __shared__ uint32_t tmem_base;
     __shared__ float dout_s[128], w3s[kHid];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x;
-    const int64_t tile = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
+    const int64_t tile = blockIdx.x / kSlices;
     train_begin(&bar_c, &bar_m, &tmem_base, 64);
     // thread (row, part) computes dz2 of one row's columns [64 part, ...): half of GELU' loaded ahead
     const int zrow = tid & 127, part = tid >> 7;
@@ -1153,10 +1154,12 @@ int forward_backward(const aiwcrf_surrogate *sg, Batch &bt, const float *X, int6
     a.P = sg->d_param; a.W1b = sg->d_W1b; a.W2b = sg->d_W2b;
     const cudaError_t e = train_kernel_attributes(sg->device);
     if (e != cudaSuccess) return cuda_fail(e, "surrogate training attributes");
-    const dim3 grid(kSlices, (unsigned)(a.B / 128));
+    // slices and tiles in one dimension: the second one ends at 65,535
+    const unsigned grid = (unsigned)kSlices * (unsigned)(a.B / 128);
     train_layer1_kernel<<<grid, kTrainThreads, 0, s>>>(a);
     train_layer2_kernel<<<grid, kTrainThreads, kLayer2Smem, s>>>(a);
     train_back_kernel<<<grid, kTrainThreads, kBackSmem, s>>>(a);
+    SG_LAUNCH_CHECK("surrogate training step");      // before anything is written to the caller's arrays
     train_wgrad_kernel<<<dim3(2, (unsigned)a.splits), kTrainThreads, kWgradSmem, s>>>(a, step);
     train_reduce_kernel<<<(kParams + kReduceThreads) / kReduceThreads, kReduceThreads, 0, s>>>(a, bt.grad, bt.loss, adam);
     count_launches(5);
