@@ -74,8 +74,6 @@ __device__ __forceinline__ void fence_mbar_init()
 }
 
 constexpr int kPredThreads = 256;
-// device selections with at most this many walks use the tree-parallel kernel (select_launch)
-constexpr int64_t kTreeParallelMaxWalks = 1 << 21;
 constexpr uint32_t kWaitLimit = 1u << 24;     // try_wait polls before giving up
 
 // stage tree t into slot (or just complete the phase if it does not fit)
@@ -1434,13 +1432,32 @@ int round_mean_launch(const int64_t *d_sum, int64_t Q, int64_t total_trees, int6
 }
 
 // Which kernels answer a device selection of K kernels x D devices:
-//  - D <= 64 and at most kTreeParallelMaxWalks walks (queries x trees): the tree-parallel kernel;
+//  - D <= 64 and few CTAs of the tree-parallel kernel (tree_parallel_selection): that kernel;
 //  - D <= 64 beyond that: the walk of predict, whose trees pass through shared memory once for 512
 //    queries, on rows coded once per kernel;
 //  - more devices: the queries written out, and predict.
-// Measured per call (us), tree-parallel / shared-memory walk, x 15 devices: 256 kernels x 500 trees 80 /
-// 90, 512 143 / 94, 1,024 250 / 130, 4,096 856 / 290; 1,024 x 50 64 / 75, 2,048 76 / 77, 4,096 149 / 95;
-// 8,192 x 16 118 / 160.
+// A CTA of the tree-parallel kernel is a kernel and 32 trees, however few the forest has, and codes the
+// kernel's features, then takes 16 devices a pass: it costs about as much as (passes + 1) / 2 CTAs of one
+// pass, 8 ns of the chip's time with one tree and 12 with 32. The batch walk costs 57 to 85 us whatever the
+// trees while it has few queries, and 130 and more once it sorts them. Measured per call (us), tree-parallel /
+// batch walk, compact forests, D = 15: 2,048 CTAs 58 / 61 (1 tree), 65 / 78 (64), 64 / 73 (500); 4,096 73 /
+// 62, 86 / 83, 83 / 83; 6,000 87 / 131 (sorted), 106 / 96, 101 / 94; 12,000 135 / 136 (1 tree), 182 / 208 (32);
+// 16,384 169 / 142, 234 / 221. With few devices the batch is smaller and the lines cross earlier: D = 1 56 / 57
+// at 2,048 CTAs, 70 / 57 at 4,096 (1 tree), 62 / 58 and 80 / 59 (64), 59 / 66 and 77 / 68 (500). D = 64, 1 tree:
+// 4,096 kernels 133 / 145, 6,000 171 / 163. Two-byte codes, unsorted, D = 15: 4,096 CTAs 81 / 70 (1 tree), 95 /
+// 109 (64), 92 / 105 (500). (A line in walks alone sent 1,000,000 kernels x 1 device x 1 tree to the
+// tree-parallel kernel: 7,834 us against 428.)
+constexpr int64_t kTreeParallelCtas = 4096, kTreeParallelCtasFewDevices = 2048, kTreeParallelCtasSorted = 12288;
+
+bool tree_parallel_selection(const aiwcrf_forest *f, int64_t K, int64_t D, int32_t size_class)
+{
+    if (D > kSelectMaxDevices || size_class < 0) return false;
+    const bool sorts = f->compact && K * D >= kSortMinQueries;
+    const int64_t line = sorts ? kTreeParallelCtasSorted : D <= 8 ? kTreeParallelCtasFewDevices : kTreeParallelCtas;
+    const int64_t ctas = K * ((f->T + 31) / 32), passes = (D + 15) / 16;
+    return ctas * (passes + 1) <= 2 * line;
+}
+
 int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32_t size_class, const DeviceIds &ids,
                   int32_t D, int32_t *d_best, int64_t *d_pred, cudaStream_t s)
 {
@@ -1448,7 +1465,7 @@ int select_launch(const aiwcrf_forest *f, const float *d_kfeat, int32_t K, int32
     keep_pool_memory(f->device);
     // one block of scratch: sums and counters of the tree-parallel kernel, or an error flag; the
     // predictions if the caller wants none; the queries where they are written out
-    const bool tree_parallel = D <= kSelectMaxDevices && Qn * f->T <= kTreeParallelMaxWalks && size_class >= 0;
+    const bool tree_parallel = tree_parallel_selection(f, K, D, size_class);
     const bool expand = D > kSelectMaxDevices;
     const size_t b_cnt = tree_parallel ? up256(8 * (size_t)Qn + 4 * (size_t)K) : 256;
     const size_t b_pred = d_pred ? 0 : up256(8 * (size_t)Qn), b_q = expand ? up256(4 * (size_t)f->F * (size_t)Qn) : 0;
