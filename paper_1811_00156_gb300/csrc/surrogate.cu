@@ -151,30 +151,12 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
+// Of a row's features a network's inputs: standardised AIWC columns, one-hot device, one-hot size, zeros.
 struct Encoder {
     const float *mu, *sd;
     const uint8_t *logf;
     int n_aiwc, n_dev, n_size;
 };
-
-// input vector of one row: standardised AIWC columns, one-hot device, one-hot size, zeros
-__device__ __forceinline__ float encode_value(const Encoder &e, const float *X, int64_t ld, int64_t row, int k)
-{
-    if (k < e.n_aiwc) {
-        float x = X[(size_t)k * (size_t)ld + row];
-        if (e.logf[k]) x = log2f(fmaxf(x, 1.0f));
-        return (x - e.mu[k]) / e.sd[k];
-    }
-    if (k < e.n_aiwc + e.n_dev) {
-        const float d = X[(size_t)e.n_aiwc * (size_t)ld + row];
-        return (d == (float)(k - e.n_aiwc)) ? 1.0f : 0.0f;
-    }
-    if (k < e.n_aiwc + e.n_dev + e.n_size) {
-        const float s = X[(size_t)(e.n_aiwc + 1) * (size_t)ld + row];
-        return (s == (float)(k - e.n_aiwc - e.n_dev)) ? 1.0f : 0.0f;
-    }
-    return 0.0f;
-}
 
 // ------------------------------------------------------------------------------------------
 // training kernels
@@ -231,17 +213,17 @@ __device__ __forceinline__ void gelu_both(float x, float &h, float &g)
     g = 0.5f * (1.0f + e) + x * 0.39894228040143268f * expf(-0.5f * x * x);
 }
 
-// What the training kernels share: an mbarrier for copies and one for MMAs, an accumulator of ncols
-// TMEM columns, and an orderly end when a bounded wait runs out.
-__device__ __forceinline__ void train_begin(uint64_t *bar_c, uint64_t *bar_m, uint32_t *tmem_base, uint32_t ncols)
+// What the training kernels share: an mbarrier for MMAs and one for copies (or none), an accumulator of
+// ncols TMEM columns, and an orderly end when a bounded wait runs out.
+__device__ __forceinline__ void train_begin(uint64_t *bar_m, uint64_t *bar_c, uint32_t *tmem_base, uint32_t ncols)
 {
     if (threadIdx.x < 32) {
         tc::tmem_alloc(tmem_base, ncols);
         tc::tmem_relinquish();
     }
     if (threadIdx.x == 0) {
-        tc::mbar_init(bar_c, 1);
         tc::mbar_init(bar_m, 1);
+        if (bar_c) tc::mbar_init(bar_c, 1);
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -288,11 +270,11 @@ __global__ void __launch_bounds__(kTrainThreads) train_layer1_kernel(TrainArgs a
 {
     __shared__ __align__(1024) unsigned char sX[kTileX];
     __shared__ __align__(1024) unsigned char sW[kSliceCols * kIn * 2];
-    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ __align__(8) uint64_t bar_m;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
     const int64_t tile = blockIdx.x / kSlices;
-    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    train_begin(&bar_m, nullptr, &tmem_base, 64);
     {   // thread (row, part) encodes inputs [8 part, 8 part + 8) and [32 + 8 part, ...) of one row; the
         // row's values are loaded together before any is used
         const int row = tid & 127, part = tid >> 7;
@@ -373,7 +355,7 @@ __global__ void __launch_bounds__(kTrainThreads) train_layer2_kernel(TrainArgs a
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
     const int64_t tile = blockIdx.x / kSlices;
-    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    train_begin(&bar_m, &bar_c, &tmem_base, 64);
     if (tid == 0) {
         tc::mbar_expect(&bar_c, kTileH);
         tc::bulk_load(sH, a.ht + (size_t)tile * kTileH, kTileH, &bar_c);
@@ -437,12 +419,12 @@ __global__ void __launch_bounds__(kTrainThreads) train_back_kernel(TrainArgs a)
 {
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *sZ = sm, *sW = sm + kTileH;       // dz2 (later dz1's columns in FP32), W2's columns
-    __shared__ __align__(8) uint64_t bar_c, bar_m;
+    __shared__ __align__(8) uint64_t bar_m;
     __shared__ uint32_t tmem_base;
     __shared__ float dout_s[128], w3s[kHid];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, slice = blockIdx.x % kSlices;
     const int64_t tile = blockIdx.x / kSlices;
-    train_begin(&bar_c, &bar_m, &tmem_base, 64);
+    train_begin(&bar_m, nullptr, &tmem_base, 64);
     // thread (row, part) computes dz2 of one row's columns [64 part, ...): half of GELU' loaded ahead
     const int zrow = tid & 127, part = tid >> 7;
     const float *g2z = a.g2 + ((size_t)tile * kHid + kSliceCols * part) * 128 + zrow;
@@ -560,7 +542,7 @@ __global__ void __launch_bounds__(kTrainThreads) train_wgrad_kernel(TrainArgs a,
     __shared__ __align__(8) uint64_t bar_c, bar_m;
     __shared__ uint32_t tmem_base;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = blockIdx.x, split = blockIdx.y;
-    train_begin(&bar_c, &bar_m, &tmem_base, 512);
+    train_begin(&bar_m, &bar_c, &tmem_base, 512);
     const uint32_t tbase = tmem_base;
     if (advance && tid == 0 && half == 0 && split == 0) *advance += 1;     // nobody reads it in this kernel
     const int tiles = a.B / 128, per = (tiles + a.splits - 1) / a.splits;
