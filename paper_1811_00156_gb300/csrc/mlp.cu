@@ -1,5 +1,5 @@
-// mlp.cu -- tensor-core (tcgen05) BF16 GEMM with FP32 accumulation in TMEM, the building block
-// of the learned surrogate's training and inference kernels.
+// mlp.cu -- tensor-core (tcgen05) BF16 GEMM with FP32 accumulation in TMEM, behind aiwcrf_tc_gemm_bf16. (The
+// learned surrogate's training and inference kernels issue their own MMAs, with tc.cuh.)
 //
 // tc_gemm_kernel: C = A * B^T with A (M x K) and B (N x K) in BF16; one CTA owns 128 rows of C
 // and a range of K. Every 64-wide K chunk of A and B is staged into shared memory in core matrices

@@ -4,8 +4,9 @@
 // the feature < x}; the forest keeps a copy of its nodes whose thresholds are the ranks of the
 // training values they are, and x <= threshold  <=>  c(x) <= rank, so the walk is exact.
 // predict_kernel: one CTA owns 256 * QPT queries whose codes (one byte per feature when every
-// column has at most 255 values) it stages once in shared memory. It then walks every tree for
-// all its queries, QPT independent walks per thread. Trees stream through two shared-memory
+// column has at most 255 values) it stages once in shared memory. It then walks a part of the trees for
+// all its queries, QPT independent walks per thread: every tree, or, where that leaves the chip idle or
+// its last wave nearly empty, one of several shares (tree_parts). Trees stream through two shared-memory
 // slots with 1-D bulk asynchronous copies (cp.async.bulk, completion counted on an mbarrier):
 // while the CTA walks tree t from one slot, tree t + 1 is landing in the other. A tree larger
 // than a slot is walked straight from global memory. Per-query sums are exact int64 (plus an
@@ -717,7 +718,9 @@ __global__ void oob_kernel(const uint64_t *__restrict__ cnodes, const int64_t *_
 // Repeated runs of one cell follow each other in a table as it is measured, and their codes are
 // alike: a tile whose neighbouring rows hold at most kOobDistinct different ones walks only those
 // (from L2: a few walks per thread), a batch of trees at a time, and then adds up every row's leaves:
-// 111,000 rows of 50 runs a cell x 500 trees 420 -> 122 us.
+// 111,000 rows of 50 runs a cell x 500 trees 420 -> 122 us. At the line itself, rows alike in fours (128
+// different ones a tile) of trees of about 11,000 nodes, the whole call 8,190 -> 3,361 us; by eights 6,761 ->
+// 1,738. Rows that are not beside their like are all walked.
 // What bounds it is instruction issue, as the walk of predict; the walk from global memory it
 // replaces waited for a load per node: 111,000 rows x 500 trees 1,072 -> 420 us.
 __device__ __forceinline__ void copy_tree4_async(const uint32_t *src, int64_t nodes, uint32_t *slot)
