@@ -4,7 +4,9 @@
 One step = fit a 500-tree forest (presort/rank, Philox bootstrap, breadth-first growth, pack)
 on 111,000 rows x 32 features, predict 1,000,000 queries, and select the fastest of 15
 devices for 64 kernels. Inputs are resident in device memory when the timed region starts;
-L2 is flushed between steps. Prints one JSON line (rank 0).
+L2 is flushed between steps. Rank 0 prints one JSON line, the result and what it was measured on; the
+reports beside it (per-kernel figures, cross-validation, tuning, surrogate, serving) are far longer and go
+to the standard error as a line of their own, the same keys and more.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -163,6 +165,23 @@ def run_reference(args):
 
 
 # ------------------------------------------------------------------------------ ours
+# what the result line carries of the report: whole entries, and of the rooflines their plain figures
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "cpu_baseline", "fit_ms", "predict",
+            "select", "parity")
+ROOFLINE = ("kernel", "bound", "achieved", "peak", "unit", "frac", "smem_frac", "ms_per_launch")
+
+
+def headline(out: dict) -> dict:
+    """The result line of a report: a reader that keeps only the last few thousand characters of the
+    output still has it whole."""
+    line = {k: out[k] for k in HEADLINE if k in out}
+    for r in ("roofline", "roofline_fit"):
+        if r in out:
+            line[r] = {k: out[r][k] for k in ROOFLINE if k in out[r]}
+    return line
+
+
 # the sources of each kernel class: its ncu counters are reported only while these are unchanged
 CLASS_SOURCES = {"tree": ("fit.cu", "internal.cuh"), "level_big": ("fit.cu", "internal.cuh"),
                  "level_small": ("fit.cu", "internal.cuh"), "walk": ("predict.cu", "internal.cuh"),
@@ -461,7 +480,8 @@ def run_ours(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline(wl)
     if rank == 0:
-        print(json.dumps(out))
+        print(json.dumps({"report": out}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(out)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
