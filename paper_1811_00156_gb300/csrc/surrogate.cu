@@ -665,9 +665,10 @@ __global__ void to_bf16_kernel(const float *__restrict__ src, bf16 *__restrict__
 // one, which every warp's arrivals of this tile precede, and the next layer 1 is issued after it.
 // Shared memory holds W1 (32 KB), W2 (128), the input tile (16) and its raw features (32).
 // Measured at 1,000,000 queries (32 features): 980 us with every part of a
-// tile after the other and eight instructions more a GELU, 413 us now = 400 TFLOP/s of the MMAs; a
-// tile's clocks are 5,200 of epilogue 1, 4,300 of epilogue 2 (6,400 together at the FP32 pipe's rate)
-// and about 2,500 of waiting for the slowest warp and the last chunk.
+// tile after the other and eight instructions more a GELU, 420 us now = 390 TFLOP/s of the MMAs. With
+// TMEM loads started a chunk ahead and approximate quotients it was 409, a tile's clocks then 5,200 of
+// epilogue 1, 4,300 of epilogue 2 (6,400 together at the FP32 pipe's rate) and about 2,500 of waiting for
+// the slowest warp and the last chunk.
 constexpr int kInferWarps = 16;                                // epilogue warps
 constexpr int kEncodeWarps = 4;                                // the first of them issues the MMAs
 constexpr int kInferThreads = 32 * (kInferWarps + kEncodeWarps);
